@@ -170,6 +170,8 @@ k3_trispec_tc(const __grid_constant__ CUtensorMap tm_img, const float* __restric
   __shared__ __align__(8) uint64_t psempty[kPsSlots];   // group slot read by the epilogue
   __shared__ __align__(8) uint64_t afull[kBufs];        // TMEM buffer holds a finished group
   __shared__ __align__(8) uint64_t aempty[kBufs];       // TMEM buffer read by the epilogue
+  __shared__ __align__(8) uint64_t turn[kMmaWarps];     // the warp's group has seen its stages land
+  __shared__ __align__(8) uint64_t drain[kMmaWarps];    // every product the warp issued is complete
   __shared__ GroupRec prec[kPsSlots];
   // FP16: the row scales 1/s of the tile's k rows, then of its l columns
   __shared__ __align__(16) float psr[kPsSlots][F::kScaled ? kTM + kTN : 4];
@@ -190,6 +192,10 @@ k3_trispec_tc(const __grid_constant__ CUtensorMap tm_img, const float* __restric
     for (int b = 0; b < kBufs; ++b) {
       mbar_init(&afull[b], 1);
       mbar_init(&aempty[b], kEpiWarps);
+    }
+    for (int w = 0; w < kMmaWarps; ++w) {
+      mbar_init(&turn[w], 1);
+      mbar_init(&drain[w], 1);
     }
     s_fail = 0;
     fence_mbar_init();
@@ -293,8 +299,7 @@ k3_trispec_tc(const __grid_constant__ CUtensorMap tm_img, const float* __restric
       const uint64_t a_desc0 = smem_desc(smem_addr(base), 128, kRowGroupBytes);
       const uint64_t b_desc0 = smem_desc(smem_addr(base) + kABytes, 128, kRowGroupBytes);
       const uint32_t nst = (uint32_t)((nkc + KC - 1) / KC);  // stages per group
-      int last_s = -1;
-      uint32_t last_ph = 0;
+      bool issued = false;
       for (uint32_t gc = w;; gc += kMmaWarps) {
         // the group's record (tile columns, or stop)
         const int p = gc & (kPsSlots - 1);
@@ -311,6 +316,12 @@ k3_trispec_tc(const __grid_constant__ CUtensorMap tm_img, const float* __restric
         // staged operands need no fence (TMA writes and MMA reads are both
         // async-proxy accesses ordered by the stage barrier)
         tc_fence_after();
+        // The group before this one belongs to the other warp.  A wait for the parity of
+        // a stage's current use passes at once while the use before it is still
+        // outstanding, so this warp looks at its stages only after the other warp has
+        // seen all of its own (and, by induction, every earlier one) land.
+        if (gc > 0 && !mbar_wait_bounded(&turn[w ^ 1u], ((gc - 1) / kMmaWarps) & 1u, status))
+          break;
         bool stop = false;
         for (uint32_t i = 0; i < nst; ++i) {
           const uint32_t q = gc * nst + i;  // the group's stages are loaded in order
@@ -320,6 +331,10 @@ k3_trispec_tc(const __grid_constant__ CUtensorMap tm_img, const float* __restric
             stop = true;
             break;
           }
+          if (i == nst - 1)
+            asm volatile("mbarrier.arrive.release.cta.shared::cta.b64 _, [%0];" ::"r"(
+                             smem_addr(&turn[w]))
+                         : "memory");
           const int kc0 = (int)i * KC;
           // descriptors of the stage; every MMA adds a compile-time offset
           const uint64_t sa = a_desc0 + (uint64_t)((s * kStageBytes) >> 4);
@@ -344,15 +359,18 @@ k3_trispec_tc(const __grid_constant__ CUtensorMap tm_img, const float* __restric
             }
           }
           mma_commit(&sdone[s]);
-          last_s = s;
-          last_ph = ph;
+          issued = true;
         }
         if (stop) break;
         mma_commit(&afull[b]);  // arrives when the group's products are complete
       }
       if (*(volatile int*)status != 0) atomicExch(&s_fail, 1);
-      // the products issued must be complete before the TMEM is freed
-      if (last_s >= 0) mbar_wait_bounded(&sdone[last_s], last_ph, status);
+      // the products issued must be complete before the TMEM is freed (a barrier of
+      // the warp's own: a stage's may have moved on to the other warp's next use)
+      if (issued) {
+        mma_commit(&drain[w]);
+        mbar_wait_bounded(&drain[w], 0u, status);
+      }
     }
     __syncwarp();
   } else {
