@@ -361,8 +361,6 @@ k3_trispec_cross_tc(const __grid_constant__ CUtensorMap tm_ab,
           tw = lv ? ssc[F::kRawSD / 4 + tli] : 1.f;
         }
       }
-      __syncwarp();
-      if (lane == 0) mbar_arrive_x(&rempty[rs]);  // the warp's coefficients are in registers
       ++rq;
       const int s = (int)(q % kSt);
       ok = __all_sync(0xffffffffu,
@@ -452,7 +450,13 @@ k3_trispec_cross_tc(const __grid_constant__ CUtensorMap tm_ab,
       // the generic-proxy writes become visible to the tensor cores' reads
       fence_async_smem();
       __syncwarp();
-      if (lane == 0) mbar_arrive_x(&full[s]);
+      if (lane == 0) {
+        // the staged coefficients are free only now, with every lane's operands
+        // written from them: released right after the loads were issued, rows of a
+        // warp whose lanes diverge were now and then built from the next copy
+        mbar_arrive_x(&rempty[rs]);
+        mbar_arrive_x(&full[s]);
+      }
       ++q;
       if (rec.flags & kRecLast) {
         // the group's one-bin sums (the two chunks of a row are lanes 8 apart; the

@@ -3,6 +3,8 @@
 One channel: with more stages per group than the ring holds (TF32x3 from m = 11,
 FP16x3 from m = 16), and with one stage per group over thousands of short groups,
 a product must wait for its own load and not for the ring's previous use.
+Several channels: a staged coefficient must not be overwritten before every lane
+has used it, so passes over one record agree to the rounding of the float64 sums.
 """
 import numpy as np
 import pytest
@@ -51,3 +53,22 @@ def test_one_stage_per_group_over_many_short_groups(precision):
     peak = np.max(np.abs(outs[0]))
     for o in outs[1:]:  # both within 1e-5 of the definition
         assert np.max(np.abs(o - outs[0])) <= 2e-5 * peak
+
+
+@pytest.mark.parametrize("precision", ["fp16x3", "tf32x3"])
+def test_cross_channel_passes_agree(precision):
+    T, m, G = 512, 20, 1200
+    z = torch.from_numpy(synth.multichannel_shared(2, T * m * G, seed=4)).cuda()
+    plan = P().Plan(channels=2, T=T, dt=0.5, m=m, orders=(4,), precision=precision)
+    outs = []
+    for _ in range(4):
+        plan.reset()
+        plan.accumulate(z)
+        outs.append(plan.finalize())
+    plan.close()
+    for key in ("S4", "S4_err"):
+        peak = np.max(np.abs(outs[0][key]))
+        for o in outs[1:]:
+            # the order of the float64 additions is all that differs between passes
+            # (the variance behind an error bar cancels: 1e-9 of the peak)
+            assert np.max(np.abs(o[key] - outs[0][key])) <= 1e-9 * peak, key
