@@ -320,8 +320,8 @@ ss_status ss_inject_timeout(ss_plan_t plan, int on);
  * warp per frame (T <= 1024), or transforms one frame at a time; K2 uses 4 x 4
  * micro-tiles in CTAs of 256 threads (4 stages, or 3 stages with three CTAs per
  * SM), 8 x 4 micro-tiles in CTAs of 128 threads with 2 or 3 pipeline stages, or
- * (one channel) 8 x 4 micro-tiles in warps that each take their own 32 x 32
- * sub-tiles and stage their own frames, with no block barrier.
+ * (84w, what a new plan has) 8 x 4 micro-tiles on 32 x 32 sub-tiles in warps that
+ * stage their own frames, each a quarter of an item's groups.
  *
  * ss_autotune   -- time every form of K1 and K2 on this plan's shapes on this
  *                  GPU (a synthetic Gaussian record of about 64 x SMs groups,

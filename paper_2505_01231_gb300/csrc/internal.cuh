@@ -49,6 +49,15 @@ struct SampleSource {
   int dtype;  // SS_F32 or SS_I16
 };
 
+// The centred spectra K1 writes: bin 0 of channel c's frame row r is at
+// rows + c * chan_stride + r * stride.  Mp bins from there on are written (zeros
+// past M - 1); with mirror, also the conjugates at the bins -(M - 1) .. -1 before.
+struct SpecRows {
+  float2* rows;
+  long long chan_stride;
+  int stride, mirror;
+};
+
 // One channel combination of one order; channels as in the ABI records.
 struct Combo {
   int order;
@@ -108,8 +117,8 @@ enum { kK1Auto = 0, kK1Resident96 = 1, kK1Frames = 2, kK1Warp = 3, kK1Modes = 4 
 // Kernel launchers (each returns the launch status; all work on `stream`).
 cudaError_t launch_k1_spectra(const SampleSource& src, long long sample0, int G, int C, int T,
                               int m, int M, int Mp, const float* win, const float2* tw,
-                              float2* spec, long long spec_chan_stride, const int* s2_auto,
-                              double* acc2, int n_s2, float pref2, int grid, cudaStream_t stream,
+                              const SpecRows& spec, const int* s2_auto, double* acc2, int n_s2,
+                              float pref2, int grid, cudaStream_t stream,
                               const OperandImage& oi = OperandImage(), double* acc1 = nullptr,
                               int mode = kK1Auto);
 
@@ -129,9 +138,8 @@ cudaError_t launch_k1_cross_s2(const float2* spec, long long chan_stride, int G,
 // K2 tilings (the autotuner's choice per plan): 4 x 4 micro-tiles in CTAs of 256
 // threads with 4 stages (two CTAs per SM) or 3 stages (three CTAs per SM, 85
 // registers), or 8 x 4 micro-tiles in CTAs of 128 threads with 2 or 3 stages;
-// all take the same 64 x 64 tiles and give the same sums.  kK2Warp84 (one channel;
-// the plan takes kK2Tile84Stages2 for several) runs k2_bispec84w: 8 x 4 micro-tiles
-// in warps that work independently on 32 x 32 sub-tiles, each with its own stages.
+// all take the same 64 x 64 tiles and give the same sums.  kK2Warp84, the default, runs
+// k2_bispec84w: 8 x 4 micro-tiles on 32 x 32 sub-tiles, a ring of stages per warp.
 enum { kK2Tile44 = 0, kK2Tile84Stages2 = 1, kK2Tile84Stages3 = 2, kK2Tile44Stages3 = 3,
        kK2Warp84 = 4, kK2Variants = 5 };
 cudaError_t launch_k2_bispec(const CUtensorMap& tm64, const CUtensorMap& tm128,
@@ -223,15 +231,50 @@ cudaError_t launch_k5_complex(const float2* spec, long long chan_stride, int G, 
                               bool natural, double* acc, long long plane, int nsm,
                               cudaStream_t stream);
 
-// K2 for isolated grid points of one channel (pts: n_pts (k, l) pairs)
-// One channel: independent warps on 32 x 32 sub-tiles (the plan's list of those
-// with more than 8 points of the domain; k2_points takes the others' points).
-// tm32 / tm64w: boxes of 2 / 4 blocks (32 / 64 bins) x kFrames84w frame rows.
+// Groups of an item of k2_bispec84w, for blocks of G groups times
+// `tiles` (tiles, combinations and blocks).  Estimated, in clocks: a group takes a warp
+// `group` with the SM's 16 warps at work (1.6 times less work gets done in that time
+// where a warp has its scheduler to itself), an item 1500 more, and its `adds` float64
+// additions are taken by the L2 at about 200 a clock over the whole GPU.  A warp takes
+// a quarter of the groups, at most kMaxFp32Groups of them.  Measured (ms, K2 alone)
+// for 4 / 16 / 64 groups: T = 1024, m = 10, 2^28 samples 10.21 / 7.34 / 6.75; T = 128,
+// m = 32, 2^23 samples 0.113 / 0.130 / 0.166 (8 groups: 0.108); T = 256, m = 10, 2^20
+// samples 0.033 / 0.040 / 0.062.
+inline int warp_item_groups(int G, long long tiles, int nsm, double group, int adds) {
+  int best = 1;
+  double tb = 1e300;
+  const int top = G < 4 * kMaxFp32Groups ? G : 4 * kMaxFp32Groups;
+  for (int gc = 1; gc <= top; ++gc) {
+    const long long items = (long long)((G + gc - 1) / gc) * tiles;
+    const double item = ((gc + 3) / 4) * group + 1500.0;
+    const long long full = (items + nsm - 1) / nsm;  // items of the busiest SM
+    const double rounds = full <= 4 ? (double)full : (double)items / nsm + 1.0;
+    const double alone = full == 1 ? 1.6 : full == 2 ? 1.1 : 1.0;
+    const double t = rounds * item * alone + (double)items * (adds / 200.0);
+    if (t < tb) {
+      tb = t;
+      best = gc;
+    }
+  }
+  return best;
+}
+
+// Independent warps on 32 x 32 sub-tiles, every combination in one launch: combos
+// is a device array of n_combos channel triples (x, y, z) whose sums start
+// combo_stride doubles apart; channel c's rows start at c * chan_rows.  tm32 /
+// tm64w: boxes of 2 / 4 blocks (32 / 64 bins) x kFrames84w frame rows of the
+// spectra, bin 0 in block zblk of a row.  One channel: the plan's list of
+// sub-tiles with more than 8 points of the domain (k2_points takes the others'
+// points) or of all; several: every sub-tile that touches the domain.  Groups form
+// blocks of block_groups (0: one block) whose sums are block_stride doubles apart.
 constexpr int kFrames84w = 4;
-cudaError_t launch_k2_bispec84w(const CUtensorMap& tm32, const CUtensorMap& tm64w, int row0,
-                                int G, int m, int M, const TileInfo* tiles, int n_tiles,
-                                float pref3, double* acc, long long plane, int nsm, int* counter,
+cudaError_t launch_k2_bispec84w(const CUtensorMap& tm32, const CUtensorMap& tm64w, int chan_rows,
+                                int zblk, int G, int m, int M, const TileInfo* tiles, int n_tiles,
+                                const int4* combos, int n_combos, int cross, float pref3,
+                                double* acc, long long plane, long long combo_stride,
+                                int block_groups, long long block_stride, int nsm, int* counter,
                                 int* status, int inject_timeout, cudaStream_t stream);
+// K2 for isolated grid points of one channel (pts: n_pts (k, l) pairs)
 cudaError_t launch_k2_points(const float2* spec, int Mp, int G, int m, const int2* pts,
                              int n_pts, int M, float pref3, double* acc, long long plane,
                              cudaStream_t stream);

@@ -635,34 +635,63 @@ k2_bispec84(const __grid_constant__ CUtensorMap tm64, const __grid_constant__ CU
 }
 
 // ---------------------------------------------------------------------------
-// K2 with independent warps (k2_bispec84w, one channel).  Each warp of a
-// 128-thread CTA is a worker of its own: it takes (group chunk, 32 x 32
-// sub-tile) items from the queue, stages the item's frame rows kFS84w at a
-// time into its own ring of kSt84w stages (a: 32 bins, b: 32 bins, c: 64 bins
-// per frame, three 3-D TMA boxes with 128-byte swizzling, refilled by its lane
-// 0 as soon as the warp leaves a stage) and evaluates 8 x 4 micro-tiles as
-// k2_bispec84 does, with the same lane layout (conflict-free for these 256- and
-// 512-byte frame rows too, checked with a bank model).  No block barrier: a warp
-// never waits for another.  The frames of an item's groups are contiguous rows,
-// so the stages run across group boundaries and a group ends at the frame where
-// its m-th row is consumed.  Per-item sums: 128 TMEM columns of the warp's lane
-// quadrant; four CTAs per SM fill the 512 columns.
+// K2 with independent warps (k2_bispec84w).  A 128-thread CTA takes (group chunk,
+// combination, 32 x 32 sub-tile) items from the queue and each of its warps a quarter
+// of the item's groups.  A warp stages its frame rows kFS84w at a time into its own
+// ring of kSt84w stages (a: 32 bins, b: 32 bins, c: 64 bins per frame, three 3-D
+// TMA boxes with 128-byte swizzling, refilled by its lane 0 as soon as the warp
+// leaves a stage) and evaluates 8 x 4 micro-tiles as k2_bispec84 does, with the
+// same lane layout (conflict-free for these 256- and 512-byte frame rows too,
+// checked with a bank model).  No warp waits for another before the item's end.
+// The frames of a warp's groups are contiguous rows, so the stages run across
+// group boundaries and a group ends at the frame where its m-th row is consumed.
+// Per-item sums: 128 TMEM columns of the warp's lane quadrant; four CTAs per SM
+// fill the 512 columns.
+//
+// Several channels: the spectra's rows hold the conjugate half at negative bins
+// too (K1 writes both), so every sub-tile of the domain |k + l| <= M - 1 is three
+// TMA boxes and all combinations go in one launch.
+//
+// At an item's end the four warps' float32 sums meet in shared memory (the warps'
+// rings, free by then; 32 x 32 floats a warp and part, chunk XOR keeps the exchange
+// free of bank conflicts), are added in float64 and go to the accumulators a row of
+// 32 consecutive doubles per warp instruction.  What this is for is the number of
+// float64 atomics, of which the L2 takes about 200 a clock: an item's 4096 cost as
+// much as 1.4 groups of m = 10 frames of one warp.  With an item per warp instead
+// (each flushing its own sums), T = 1024, m = 10: 6.95 ms for 2^28 samples, 0.93 ms
+// for 2^25; now 6.75 and 0.88 ms.  2^20 samples at T = 256: 0.099 ms with 64 x 64
+// tiles, one group an item, and now 0.033 ms.  Four channels, 2^21 samples, T = 512,
+// m = 20, 20 combinations: 10.5 ms in 20 launches of 64 x 64 tiles (the half with
+// negative bins staged by the threads), now 3.3 ms.
 constexpr int kThreads84w = 128;
 constexpr int kFS84w = kFrames84w;  // frames per stage
 constexpr int kSt84w = 3;   // stages per warp
 constexpr uint32_t kStage84w = kFS84w * (256u + 256u + 512u);  // a | b | c
 constexpr uint32_t kRing84w = kSt84w * kStage84w;
+static_assert(kRing84w >= 32 * 32 * sizeof(float), "the flush exchanges one part in the ring");
+
+// A warp's current item, kept in shared memory: the copies' coordinates (lane 0) and
+// the place of the sums, which would otherwise hold registers through the frame loop.
+struct Item84w {
+  int ya, yb, yc, ra, rb, rc;  // 16-bin blocks and first frame rows of a, b, c
+  int k0, l0;
+  long long acc_off;           // of the sub-tile's row k0, column l0
+};
 
 __global__ void __launch_bounds__(kThreads84w, 4)
 k2_bispec84w(const __grid_constant__ CUtensorMap tm32, const __grid_constant__ CUtensorMap tm64,
-             int row0, int m, int M, int G, const TileInfo* __restrict__ tiles, WorkQueue wq,
-             float pref3, double* __restrict__ acc, long long plane, int* __restrict__ status,
-             int inject_timeout) {
+             int m, int M, int G, int zblk, const TileInfo* __restrict__ tiles,
+             const int4* __restrict__ combos, int chan_rows, long long combo_stride, WarpQueue wq,
+             int cross, float pref3, double* __restrict__ acc, long long plane,
+             int* __restrict__ status, int inject_timeout) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];  // + 1024 spare bytes
   __shared__ __align__(8) uint64_t full[kThreads84w / 32][kSt84w];
   __shared__ __align__(8) uint64_t never;  // completed by nothing (timeout test)
   __shared__ uint32_t tmem_slot;
+  __shared__ Item84w items[kThreads84w / 32];
+  __shared__ int s_next;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  Item84w& it = items[warp];
   unsigned char* ring = align1024<unsigned char>(smem_raw) + (size_t)warp * kRing84w;
   const int tx = lane & 3;
   const int ty = ((lane >> 3) & 1) | (((lane >> 2) & 1) << 1) | (((lane >> 4) & 1) << 2);
@@ -696,41 +725,63 @@ k2_bispec84w(const __grid_constant__ CUtensorMap tm32, const __grid_constant__ C
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tsum = tmem_slot + ((uint32_t)(32 * warp) << 16);
-  {
-    float z[32];
-#pragma unroll
-    for (int i = 0; i < 32; ++i) z[i] = 0.f;
-#pragma unroll
-    for (int part = 0; part < 4; ++part) tmem_st32(tsum + 32 * part, z);
-  }
   uint32_t qb = 0;  // stages this warp has consumed (stage = q % kSt84w)
+  int next = 0;     // thread 0: the item after the current one, drawn while it runs
+  if (tid == 0) next = atomicAdd(wq.counter, 1);
   for (;;) {
-    int item = 0;
-    if (lane == 0) item = atomicAdd(wq.counter, 1);
-    item = __shfl_sync(0xffffffffu, item, 0);
+    if (tid == 0) s_next = next;
+    __syncthreads();
+    const int item = s_next;
     if (item >= wq.n_items) break;
-    const int t = item % wq.n_tiles;
-    const int ga = (item / wq.n_tiles) * wq.group_chunk;
-    const int gb = min(G, ga + wq.group_chunk);
-    const int k0 = tiles[t].k0, l0 = tiles[t].l0;
-    const int rows = (gb - ga) * m;  // the item's frames, consecutive rows from r0
-    const int r0 = row0 + ga * m;
+    if (tid == 0) next = atomicAdd(wq.counter, 1);
+    int rows;  // the warp's frames of the item, consecutive rows
+    {
+      const int per_chunk = wq.n_tiles * wq.n_combos;
+      const int chunk = item / per_chunk, rest = item - chunk * per_chunk;
+      const int combo = rest / wq.n_tiles, t = rest - combo * wq.n_tiles;
+      const int blk = chunk / wq.chunks_per_block;
+      int ga = blk * wq.block_groups + (chunk - blk * wq.chunks_per_block) * wq.group_chunk;
+      int ng = min(min(G, (blk + 1) * wq.block_groups), ga + wq.group_chunk) - ga;
+      const int w0 = ng * warp / 4;
+      ng = ng * (warp + 1) / 4 - w0;
+      ga += w0;
+      rows = ng * m;
+      if (lane == 0) {
+        const int k0 = tiles[t].k0, l0 = tiles[t].l0;
+        const int4 cb = combos[combo];
+        it.ya = zblk + (k0 >> 4);
+        it.yb = zblk + (l0 >> 4);
+        it.yc = zblk + ((k0 + l0) >> 4);
+        it.ra = cb.x * chan_rows + ga * m;
+        it.rb = cb.y * chan_rows + ga * m;
+        it.rc = cb.z * chan_rows + ga * m;
+        it.k0 = k0;
+        it.l0 = l0;
+        it.acc_off = blk * wq.block_stride + combo * combo_stride +
+                     (long long)(k0 + (cross ? M - 1 : 0)) * M + l0;
+      }
+    }
     const int nst = (rows + kFS84w - 1) / kFS84w;
-    auto issue = [&](int i) {  // lane 0: stage of step i (kFS84w rows from r0 + i kFS84w)
+    auto issue = [&](int i) {  // lane 0: stage of step i (kFS84w rows from row i kFS84w)
       const int s = (int)((qb + i) % kSt84w);
       unsigned char* st = ring + (size_t)s * kStage84w;
-      const int r = r0 + i * kFS84w;
+      const int r = i * kFS84w;
       mbar_arrive_expect_tx(&full[warp][s], kStage84w);
-      tma_load_3d(st, &tm32, 0, k0 >> 4, r, &full[warp][s]);
-      tma_load_3d(st + kFS84w * 256, &tm32, 0, l0 >> 4, r, &full[warp][s]);
-      tma_load_3d(st + kFS84w * 512, &tm64, 0, (k0 + l0) >> 4, r, &full[warp][s]);
+      tma_load_3d(st, &tm32, 0, it.ya, it.ra + r, &full[warp][s]);
+      tma_load_3d(st + kFS84w * 256, &tm32, 0, it.yb, it.rb + r, &full[warp][s]);
+      tma_load_3d(st + kFS84w * 512, &tm64, 0, it.yc, it.rc + r, &full[warp][s]);
     };
     float ar[32], ai[32];
 #pragma unroll
     for (int i = 0; i < 32; ++i) ar[i] = ai[i] = 0.f;
-    if (lane == 0) {
-      fence_async_smem();
+    if (lane == 0)
       for (int i = 0; i < kSt84w && i < nst; ++i) issue(i);
+    {
+      float z[32];
+#pragma unroll
+      for (int i = 0; i < 32; ++i) z[i] = 0.f;
+#pragma unroll
+      for (int part = 0; part < 4; ++part) tmem_st32(tsum + 32 * part, z);
     }
     __syncwarp();
     bool ok = true;
@@ -830,22 +881,42 @@ k2_bispec84w(const __grid_constant__ CUtensorMap tm32, const __grid_constant__ C
         issue(i + kSt84w);
       }
     }
-    if (!ok) break;
+    if (__syncthreads_or(!ok)) break;
     qb += nst;
-    // end of the item: the sums of each part go to the float64 accumulators
+    // end of the item: the sums of each part go to the float64 accumulators.  The
+    // rings hold no copy in flight now; lane (tx, ty) writes its four columns of row
+    // kt + a as 16-byte chunk ty ^ perm(tx), perm = {0, 1, 4, 5}
+    float* ex = reinterpret_cast<float*>(ring);
+    const int wchunk = 4 * (ty ^ ((tx & 1) | ((tx & 2) << 1)));
+    const int k0 = it.k0, l = it.l0 + lane;
+    double* arow = acc + it.acc_off + lane;
 #pragma unroll 1
     for (int part = 0; part < 4; ++part) {
-      float tt[32], z[32];
+      float tt[32];
       tmem_ld32(tsum + 32 * part, tt);
-      double* dst = acc + (long long)part * plane;
 #pragma unroll
-      for (int q = 0; q < 32; ++q) {
-        const int k = k0 + kt + (q >> 2), l = l0 + lt + (q & 3);
-        if (in_domain3(k, l, M, 0)) atomicAdd(dst + (long long)k * M + l, (double)tt[q]);
-        z[q] = 0.f;
+      for (int a = 0; a < 8; ++a)
+        *reinterpret_cast<float4*>(ex + (kt + a) * 32 + wchunk) =
+            make_float4(tt[4 * a], tt[4 * a + 1], tt[4 * a + 2], tt[4 * a + 3]);
+      double* dst = arow + part * plane;
+      __syncthreads();
+      // the CTA's four sums of the rows 8 warp .. 8 warp + 7
+      const float* exs = reinterpret_cast<const float*>(align1024<unsigned char>(smem_raw));
+      const int perm = (warp & 1) | ((warp & 2) << 1);
+      const float* col = exs + 4 * ((lane >> 2) ^ perm) + (lane & 3);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int r = 8 * warp + i;
+        double v = 0.0;
+#pragma unroll
+        for (int w = 0; w < 4; ++w) v += (double)col[w * (kRing84w / 4) + r * 32];
+        if (in_domain3(k0 + r, l, M, cross)) atomicAdd(dst + (long long)r * M, v);
       }
-      tmem_st32(tsum + 32 * part, z);
+      __syncthreads();
     }
+    // the exchange's accesses come before the next item's copies into the ring
+    fence_async_smem();
+    __syncwarp();
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
@@ -1004,11 +1075,25 @@ cudaError_t launch_k2_fc(const CUtensorMap& tm64, const CUtensorMap& tm128, cons
 
 }  // namespace
 
-cudaError_t launch_k2_bispec84w(const CUtensorMap& tm32, const CUtensorMap& tm64w, int row0,
-                                int G, int m, int M, const TileInfo* tiles, int n_tiles,
-                                float pref3, double* acc, long long plane, int nsm, int* counter,
+cudaError_t launch_k2_bispec84w(const CUtensorMap& tm32, const CUtensorMap& tm64w, int chan_rows,
+                                int zblk, int G, int m, int M, const TileInfo* tiles, int n_tiles,
+                                const int4* combos, int n_combos, int cross, float pref3,
+                                double* acc, long long plane, long long combo_stride,
+                                int block_groups, long long block_stride, int nsm, int* counter,
                                 int* status, int inject_timeout, cudaStream_t stream) {
-  if (G <= 0 || n_tiles <= 0) return cudaSuccess;
+  if (G <= 0 || n_tiles <= 0 || n_combos <= 0) return cudaSuccess;
+  WarpQueue wq;
+  wq.counter = counter;
+  wq.n_tiles = n_tiles;
+  wq.n_combos = n_combos;
+  if (block_groups <= 0 || block_groups > G) block_groups = G;
+  wq.block_groups = block_groups;
+  wq.block_stride = block_stride;
+  const long long n_blocks = (G + block_groups - 1) / block_groups;
+  wq.group_chunk = warp_item_groups(block_groups, n_blocks * n_tiles * n_combos, nsm,
+                                    400.0 * m + 500.0, 4 * 1024);
+  wq.chunks_per_block = (block_groups + wq.group_chunk - 1) / wq.group_chunk;
+  const long long n_items = n_blocks * wq.chunks_per_block * n_tiles * n_combos;
   const size_t smem = (size_t)(kThreads84w / 32) * kRing84w + 1024;
   cudaError_t e = cudaFuncSetAttribute(k2_bispec84w, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)smem);
@@ -1020,18 +1105,14 @@ cudaError_t launch_k2_bispec84w(const CUtensorMap& tm32, const CUtensorMap& tm64
   int occ = 1;
   e = ctas_per_sm(k2_bispec84w, kThreads84w, smem, 4, &occ);
   if (e != cudaSuccess) return e;
-  const int n_cta = nsm * occ;
-  WorkQueue wq;  // items per warp
-  wq.counter = counter;
-  wq.n_tiles = n_tiles;
-  // about 8 items per warp (half the pair kernels' 16): each item ends with a
-  // flush of its warp's 32 x 32 sub-tile, so longer items halve the atomics
-  wq.group_chunk = work_group_chunk(G, n_tiles, n_cta * (kThreads84w / 32) / 2);
-  wq.n_items = n_tiles * ((G + wq.group_chunk - 1) / wq.group_chunk);
+  if (n_items > 0x7ffffff0ll - 4ll * nsm * occ) return cudaErrorInvalidValue;
+  wq.n_items = (int)n_items;
+  const int n_cta = (int)std::min<long long>((long long)nsm * occ, n_items);
   e = cudaMemsetAsync(counter, 0, sizeof(int), stream);
   if (e != cudaSuccess) return e;
-  k2_bispec84w<<<n_cta, kThreads84w, smem, stream>>>(tm32, tm64w, row0, m, M, G, tiles, wq,
-                                                     pref3, acc, plane, status, inject_timeout);
+  k2_bispec84w<<<n_cta, kThreads84w, smem, stream>>>(
+      tm32, tm64w, m, M, G, zblk, tiles, combos, chan_rows, combo_stride, wq, cross, pref3, acc,
+      plane, status, inject_timeout);
   return cudaGetLastError();
 }
 

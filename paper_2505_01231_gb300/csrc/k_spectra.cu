@@ -181,6 +181,14 @@ __device__ __forceinline__ float f16_row_scale(float bound) {
   return ldexpf(1.f, 14 - e);
 }
 
+// Coefficient of bin k of a spectra row (bin 0 at row[0]); with mirror, also its
+// conjugate at bin -k (several channels: K2 reads whole rows of signed bins).
+__device__ __forceinline__ void put_coef(float2* __restrict__ row, int k, int M, float2 d,
+                                         int mirror) {
+  row[k] = d;
+  if (mirror && k > 0 && k < M) row[-k] = make_float2(d.x, -d.y);
+}
+
 template <int DTYPE>
 __device__ __forceinline__ float load_sample(const SampleSource& s, int c, long long idx) {
   if (idx < s.carry_n) {
@@ -312,7 +320,7 @@ template <int DTYPE, int FMT>
 __global__ void __launch_bounds__(kThreadsK1)
 k1_spectra(SampleSource src, long long sample0, int G, int C, int T, int m, int M, int Mp,
            const float* __restrict__ win, const float2* __restrict__ tw,
-           float2* __restrict__ spec, long long chan_stride, const int* __restrict__ s2_auto,
+           SpecRows sp, const int* __restrict__ s2_auto,
            double* __restrict__ acc2, int n_s2, float pref2, OperandImage oi,
            double* __restrict__ acc1) {
   extern __shared__ float4 smem_raw[];
@@ -330,7 +338,7 @@ k1_spectra(SampleSource src, long long sample0, int G, int C, int T, int m, int 
   int ngroups = 0;  // groups in the float32 sums since the last flush
   for (int g = blockIdx.x; g < G; g += gridDim.x) {
     for (int c = 0; c < C; ++c) {
-      float2* grow = spec + (long long)c * chan_stride + (long long)g * m * Mp;
+      float2* grow = sp.rows + (long long)c * sp.chan_stride + (long long)g * m * sp.stride;
       for (int k = threadIdx.x; k < M; k += blockDim.x) gsum[k] = make_float2(0.f, 0.f);
       for (int j = 0; j < m; ++j) {
         const long long s0 = sample0 + ((long long)g * m + j) * T;
@@ -360,7 +368,7 @@ k1_spectra(SampleSource src, long long sample0, int G, int C, int T, int m, int 
           float2* t = x; x = y; y = t;
         }
         // x holds Y_n; X_k = 1/2 [(Y_k + Y*_{N-k}) - j w^k (Y_k - Y*_{N-k})], w = e^{+2 pi j/T}
-        float2* row = grow + (long long)j * Mp;
+        float2* row = grow + (long long)j * sp.stride;
         for (int k = threadIdx.x; k < M; k += blockDim.x) {
           const float2 yk = x[k == N ? 0 : k];
           const float2 yr = x[k == 0 ? 0 : N - k];
@@ -383,8 +391,8 @@ k1_spectra(SampleSource src, long long sample0, int G, int C, int T, int m, int 
         if (k == 0) add_s1(s1s[c], mean);
         centre_bin<FMT>(
             k, valid, mean, m, c, g, Mp, oi,
-            [&](int j) { return grow[(long long)j * Mp + k]; },
-            [&](int j, float2 d) { grow[(long long)j * Mp + k] = d; },
+            [&](int j) { return grow[(long long)j * sp.stride + k]; },
+            [&](int j, float2 d) { put_coef(grow + (long long)j * sp.stride, k, M, d, sp.mirror); },
             ia >= 0 ? s2sum + c * M : nullptr, ia >= 0 ? s2sq + c * M : nullptr, pref2);
       }
     }
@@ -434,7 +442,8 @@ __device__ __forceinline__ void stockham_pass_batch(const float2* __restrict__ x
 // sums and, with an operand image, write the bin's weighted Gram products and its
 // ps value.
 template <int FMT>
-__device__ __forceinline__ void centre_resident(float2* Xs, float2* __restrict__ grow, int c, int g,
+__device__ __forceinline__ void centre_resident(float2* Xs, float2* __restrict__ grow,
+                                                int row_stride, int mirror, int c, int g,
                                                 int m, int M, int Mp, const OperandImage& oi,
                                                 int ia, float* s2sum, float* s2sq, float* s1,
                                                 float pref2) {
@@ -452,7 +461,7 @@ __device__ __forceinline__ void centre_resident(float2* Xs, float2* __restrict__
     for (int j = 0; j < m; ++j) {
       const float2 d = valid ? csub(Xs[j * Mp + k], mean) : make_float2(0.f, 0.f);
       Xs[j * Mp + k] = d;
-      grow[(long long)j * Mp + k] = d;
+      put_coef(grow + (long long)j * row_stride, k, M, d, mirror);
       const float pj = fmaf(d.x, d.x, d.y * d.y);
       p += pj;
       mx = fmaxf(mx, pj);
@@ -524,7 +533,7 @@ template <int DTYPE, int FMT>
 __global__ void __launch_bounds__(kThreadsK1, 3)
 k1_spectra_res(SampleSource src, long long sample0, int G, int C, int T, int m, int M, int Mp,
                int FB, const float* __restrict__ win, const float2* __restrict__ tw,
-               float2* __restrict__ spec, long long chan_stride, const int* __restrict__ s2_auto,
+               SpecRows sp, const int* __restrict__ s2_auto,
                double* __restrict__ acc2, int n_s2, float pref2, OperandImage oi,
            double* __restrict__ acc1) {
   extern __shared__ float4 smem_raw[];
@@ -569,7 +578,7 @@ k1_spectra_res(SampleSource src, long long sample0, int G, int C, int T, int m, 
   int ngroups = 0;  // groups in the float32 sums since the last flush
   for (int g = blockIdx.x; g < G; g += gridDim.x) {
     for (int c = 0; c < C; ++c) {
-      float2* grow = spec + (long long)c * chan_stride + (long long)g * m * Mp;
+      float2* grow = sp.rows + (long long)c * sp.chan_stride + (long long)g * m * sp.stride;
       for (int j0 = 0; j0 < m; j0 += FB) {
         const int nf = min(FB, m - j0);
         const long long s0 = sample0 + ((long long)g * m + j0) * T;  // first sample of the batch
@@ -666,7 +675,7 @@ k1_spectra_res(SampleSource src, long long sample0, int G, int C, int T, int m, 
         }
       }
       __syncthreads();  // the group's coefficients are in shared memory
-      centre_resident<FMT>(Xs, grow, c, g, m, M, Mp, oi, s2_auto[c], s2sum, s2sq, s1s[c], pref2);
+      centre_resident<FMT>(Xs, grow, sp.stride, sp.mirror, c, g, m, M, Mp, oi, s2_auto[c], s2sum, s2sq, s1s[c], pref2);
     }
     if (++ngroups == kMaxFp32Groups) {
       flush_k1_sums(C, M, s2_auto, acc2, n_s2, s2sum, s2sq, s1s, acc1);
@@ -723,7 +732,7 @@ template <int DTYPE, int FMT>
 __global__ void __launch_bounds__(kThreadsK1, 2)
 k1_spectra_warp(SampleSource src, long long sample0, int G, int C, int T, int m, int M, int Mp,
                 const float* __restrict__ win, const float2* __restrict__ tw,
-                float2* __restrict__ spec, long long chan_stride, const int* __restrict__ s2_auto,
+                SpecRows sp, const int* __restrict__ s2_auto,
                 double* __restrict__ acc2, int n_s2, float pref2, OperandImage oi,
                 double* __restrict__ acc1) {
   extern __shared__ float4 smem_raw[];
@@ -751,7 +760,7 @@ k1_spectra_warp(SampleSource src, long long sample0, int G, int C, int T, int m,
   int ngroups = 0;  // groups in the float32 sums since the last flush
   for (int g = blockIdx.x; g < G; g += gridDim.x) {
     for (int c = 0; c < C; ++c) {
-      float2* grow = spec + (long long)c * chan_stride + (long long)g * m * Mp;
+      float2* grow = sp.rows + (long long)c * sp.chan_stride + (long long)g * m * sp.stride;
       for (int j = warp; j < m; j += kWarps) {
         // the frame's samples times the window, packed as N complex points
         const long long s0 = sample0 + ((long long)g * m + j) * T;
@@ -804,7 +813,7 @@ k1_spectra_warp(SampleSource src, long long sample0, int G, int C, int T, int m,
         __syncwarp();  // the buffer is free for the warp's next frame
       }
       __syncthreads();  // the group's coefficients are in shared memory
-      centre_resident<FMT>(Xs, grow, c, g, m, M, Mp, oi, s2_auto[c], s2sum, s2sq, s1s[c], pref2);
+      centre_resident<FMT>(Xs, grow, sp.stride, sp.mirror, c, g, m, M, Mp, oi, s2_auto[c], s2sum, s2sq, s1s[c], pref2);
       __syncthreads();  // Xs is free for the next channel or group
     }
     if (++ngroups == kMaxFp32Groups) {
@@ -897,8 +906,8 @@ cudaError_t k1_occupancy(Kern kern, size_t smem, int* occ) {
 
 template <int DTYPE, int FMT>
 cudaError_t launch_k1_t(const SampleSource& src, long long sample0, int G, int C, int T, int m,
-                        int M, int Mp, const float* win, const float2* tw, float2* spec,
-                        long long spec_chan_stride, const int* s2_auto, double* acc2, int n_s2,
+                        int M, int Mp, const float* win, const float2* tw, const SpecRows& spec,
+                        const int* s2_auto, double* acc2, int n_s2,
                         float pref2, const OperandImage& oi, int grid, size_t smem,
                         cudaStream_t stream, double* acc1, int mode) {
   // a group whose coefficients fit beside a batch of FFT buffers stays resident
@@ -925,8 +934,7 @@ cudaError_t launch_k1_t(const SampleSource& src, long long sample0, int G, int C
     if (e != cudaSuccess) return e;
     const int rgrid = std::max(1, std::min(G, nsm * occ));
     kern<<<rgrid, kThreadsK1, wsmem, stream>>>(src, sample0, G, C, T, m, M, Mp, win, tw, spec,
-                                               spec_chan_stride, s2_auto, acc2, n_s2, pref2, oi,
-                                               acc1);
+                                               s2_auto, acc2, n_s2, pref2, oi, acc1);
     return cudaGetLastError();
   }
   const size_t budget = mode == kK1Frames ? 0
@@ -959,7 +967,7 @@ cudaError_t launch_k1_t(const SampleSource& src, long long sample0, int G, int C
     const int occ = std::max(1, std::min(std::min(by_smem, by_regs), 2048 / kThreadsK1));
     const int rgrid = std::max(1, std::min(G, nsm * occ));
     kern<<<rgrid, kThreadsK1, rsmem, stream>>>(
-        src, sample0, G, C, T, m, M, Mp, FB, win, tw, spec, spec_chan_stride, s2_auto, acc2, n_s2,
+        src, sample0, G, C, T, m, M, Mp, FB, win, tw, spec, s2_auto, acc2, n_s2,
         pref2, oi, acc1);
     return cudaGetLastError();
   }
@@ -967,14 +975,13 @@ cudaError_t launch_k1_t(const SampleSource& src, long long sample0, int G, int C
   cudaError_t e = set_smem_limit(k1_spectra<DTYPE, FMT>, kK1MaxSmem);
   if (e != cudaSuccess) return e;
   k1_spectra<DTYPE, FMT><<<grid, kThreadsK1, smem, stream>>>(src, sample0, G, C, T, m, M, Mp, win,
-                                                             tw, spec, spec_chan_stride, s2_auto,
-                                                             acc2, n_s2, pref2, oi, acc1);
+                                                             tw, spec, s2_auto, acc2, n_s2, pref2, oi, acc1);
   return cudaGetLastError();
 }
 
 cudaError_t launch_k1_spectra(const SampleSource& src, long long sample0, int G, int C, int T,
                               int m, int M, int Mp, const float* win, const float2* tw,
-                              float2* spec, long long spec_chan_stride, const int* s2_auto,
+                              const SpecRows& spec, const int* s2_auto,
                               double* acc2, int n_s2, float pref2, int grid, cudaStream_t stream,
                               const OperandImage& oi, double* acc1, int mode) {
   if (G <= 0) return cudaSuccess;
@@ -982,7 +989,7 @@ cudaError_t launch_k1_spectra(const SampleSource& src, long long sample0, int G,
   const size_t smem = k1_smem(T, C);
   if (grid > G) grid = G;
   const bool f32 = src.dtype == SS_F32;
-#define K1_ARGS src, sample0, G, C, T, m, M, Mp, win, tw, spec, spec_chan_stride, s2_auto, acc2, \
+#define K1_ARGS src, sample0, G, C, T, m, M, Mp, win, tw, spec, s2_auto, acc2, \
                 n_s2, pref2, oi, grid, smem, stream, acc1, mode
   switch (oi.fmt) {
     case kImageGramTF32:

@@ -151,6 +151,17 @@ struct WorkQueue {
   int n_items;
 };
 
+// Dynamic work queue of the independent-warp K2: item i is (group chunk, channel
+// combination, sub-tile), chunk-major.  The batch's groups form blocks of
+// block_groups groups (one block unless the spectra of consecutive blocks are kept
+// apart); a block has chunks_per_block chunks of group_chunk groups, the last one
+// shorter, and its sums start block_stride doubles after those of the block before.
+struct WarpQueue {
+  int* counter;
+  int n_tiles, n_combos, group_chunk, n_items, block_groups, chunks_per_block;
+  long long block_stride;
+};
+
 // Returns the next item for the calling CTA (all threads receive it) or -1.
 __device__ __forceinline__ int next_item(const WorkQueue& q, int* s_slot) {
   __syncthreads();  // the previous item's readers of *s_slot are done

@@ -184,23 +184,32 @@ void build_tiles(int M, bool cross, std::vector<TileInfo>& t3, std::vector<TileI
     }
 }
 
-// One channel, k2_bispec84w: the 32 x 32 sub-tiles that hold more than
-// kIsolatedPoints points of the S3 domain (0 <= k <= l, k + l <= M - 1), and the
-// points of the others (where the edge k + l = M - 1 passes a sub-tile corner),
-// which k2_points evaluates.
-void build_warp_tiles(int M, std::vector<TileInfo>& t, std::vector<int2>& pts) {
+// k2_bispec84w.  One channel: the 32 x 32 sub-tiles that hold more than
+// kIsolatedPoints points of the S3 domain (0 <= k <= l, k + l <= M - 1), *n_main of
+// them, then those that hold fewer (where the edge k + l = M - 1 passes a sub-tile
+// corner), and the points of the latter, which k2_points can evaluate instead.
+// Several channels: every sub-tile that touches the domain |k + l| <= M - 1.
+void build_warp_tiles(int M, bool cross, std::vector<TileInfo>& t, std::vector<int2>& pts,
+                      int* n_main) {
   constexpr int kW = 32;
-  for (int k0 = 0; k0 < M; k0 += kW)
+  std::vector<TileInfo> few;
+  const int kmin = cross ? -((M - 1 + kW - 1) / kW) * kW : 0;
+  const size_t isolated = cross ? 0 : kIsolatedPoints;
+  for (int k0 = kmin; k0 < M; k0 += kW)
     for (int l0 = 0; l0 < M; l0 += kW) {
       std::vector<int2> in;
-      for (int a = 0; a < kW && (int)in.size() <= kIsolatedPoints; ++a)
-        for (int b = 0; b < kW && (int)in.size() <= kIsolatedPoints; ++b)
-          if (in_domain3(k0 + a, l0 + b, M, 0)) in.push_back(make_int2(k0 + a, l0 + b));
-      if ((int)in.size() > kIsolatedPoints)
+      for (int a = 0; a < kW && in.size() <= isolated; ++a)
+        for (int b = 0; b < kW && in.size() <= isolated; ++b)
+          if (in_domain3(k0 + a, l0 + b, M, cross)) in.push_back(make_int2(k0 + a, l0 + b));
+      if (in.size() > isolated) {
         t.push_back(TileInfo{k0, l0, 1, kW});
-      else
+      } else if (!in.empty()) {
+        few.push_back(TileInfo{k0, l0, 1, kW});
         pts.insert(pts.end(), in.begin(), in.end());
+      }
     }
+  *n_main = (int)t.size();
+  t.insert(t.end(), few.begin(), few.end());
 }
 
 void record(ss_plan_s* p, int stage, cudaStream_t s, bool start) {
@@ -290,7 +299,8 @@ ss_status process_device(ss_plan_s* p, const void* ptr, long long n, long long s
     src.chunk = ptr;
     src.chunk_stride = stride;
     src.dtype = p->dtype;
-    const long long chan_stride = (long long)p->Gb_max * p->m * p->Mp;
+    const long long chan_stride = (long long)p->Gb_max * p->m * p->Ms;
+    float2* const spec = p->d_spec + p->Z;  // bin 0 of the first row
     // prefactors of c2, c3 and the two parts of c4 over the centred sums: the
     // k-statistics (Eq. 32-34, 85) or the natural estimators
     const double md = p->m;
@@ -307,43 +317,47 @@ ss_status process_device(ss_plan_s* p, const void* ptr, long long n, long long s
       const int cnt = (int)take;
       record(p, 0, p->stream, true);
       SS_TRY(p, launch_k1_spectra(src, g0 * per_group, cnt, p->C, p->T, p->m, p->M, p->Mp,
-                                  p->d_win, p->d_tw, p->d_spec, chan_stride, p->d_s2auto,
-                                  p->d_acc2, (int)p->c2.size(), pref2, 4 * p->nsm, p->stream,
+                                  p->d_win, p->d_tw,
+                                  SpecRows{spec, chan_stride, p->Ms, p->mirror ? 1 : 0},
+                                  p->d_s2auto, p->d_acc2, (int)p->c2.size(), pref2, 4 * p->nsm, p->stream,
                                   p->oi, p->d_acc1, p->k1_mode));
       if (p->n_s2cross > 0)
-        SS_TRY(p, launch_k1_cross_s2(p->d_spec, chan_stride, cnt, p->m, p->M, p->Mp,
+        SS_TRY(p, launch_k1_cross_s2(spec, chan_stride, cnt, p->m, p->M, p->Ms,
                                      p->d_s2cross, p->n_s2cross, pref2, p->d_acc2,
                                      (long long)p->c2.size() * p->M, p->nsm, p->stream));
       record(p, 0, p->stream, false);
       if (!p->c3.empty()) {
         record(p, 1, p->stream, true);
         const long long plane = (long long)p->c3.size() * p->rows3 * p->M;
+        const int row_stride = p->Gb_max * p->m;
+        const long long combo_stride = (long long)p->rows3 * p->M;
+        const bool warps = p->k2_variant == kK2Warp84;
+        // Independent warps: with few items the sub-tiles that hold isolated points are
+        // taken as items too, which costs them less than the point kernel's launch
+        // (T = 256, 409 groups: 8 sub-tiles instead of 6 and a launch of 7.5 us)
+        const bool all = warps && (long long)cnt * p->n_tiles3a <= 16ll * p->nsm * 4;
+        if (warps)
+          SS_TRY(p, launch_k2_bispec84w(p->tm32w, p->tm64w, row_stride, p->Z / 16, cnt, p->m,
+                                        p->M, p->d_tiles3w, all ? p->n_tiles3a : p->n_tiles3w,
+                                        p->d_c3, (int)p->c3.size(), p->C > 1 ? 1 : 0, pref3,
+                                        p->d_acc3, plane, combo_stride, 0, 0, p->nsm,
+                                        p->d_counter, p->d_status, p->inject_timeout, p->stream));
         for (size_t i = 0; i < p->c3.size(); ++i) {
           const Combo& cb = p->c3[i];
-          const int row_stride = p->Gb_max * p->m;
-          double* acc3 = p->d_acc3 + (long long)i * p->rows3 * p->M;
-          const bool warps = p->k2_variant == kK2Warp84 && p->C == 1;
-          if (warps)
-            SS_TRY(p, launch_k2_bispec84w(p->tm32w, p->tm64w, cb.c[0] * row_stride, cnt, p->m,
-                                          p->M, p->d_tiles3w, p->n_tiles3w, pref3, acc3, plane,
-                                          p->nsm, p->d_counter, p->d_status, p->inject_timeout,
-                                          p->stream));
-          else
-            SS_TRY(p, launch_k2_bispec(p->tm64, p->tm128, p->d_spec + cb.c[0] * chan_stride,
-                                       p->d_spec + cb.c[1] * chan_stride,
-                                       p->d_spec + cb.c[2] * chan_stride, cb.c[0] * row_stride,
-                                       cb.c[1] * row_stride, cb.c[2] * row_stride, cnt, p->m,
-                                       p->FC, p->M, p->Mp, p->d_tiles3, p->n_tiles3,
-                                       p->C > 1 ? 1 : 0, pref3, acc3, plane, p->rows3, p->nsm,
-                                       p->d_counter, p->d_status, p->inject_timeout,
-                                       p->k2_variant == kK2Warp84 ? kK2Tile84Stages2
-                                                                  : p->k2_variant,
-                                       p->stream));
+          double* acc3 = p->d_acc3 + (long long)i * combo_stride;
+          if (!warps)
+            SS_TRY(p, launch_k2_bispec(p->tm64, p->tm128, spec + cb.c[0] * chan_stride,
+                                       spec + cb.c[1] * chan_stride, spec + cb.c[2] * chan_stride,
+                                       cb.c[0] * row_stride, cb.c[1] * row_stride,
+                                       cb.c[2] * row_stride, cnt, p->m, p->FC, p->M, p->Ms,
+                                       p->d_tiles3, p->n_tiles3, p->C > 1 ? 1 : 0, pref3, acc3,
+                                       plane, p->rows3, p->nsm, p->d_counter, p->d_status,
+                                       p->inject_timeout, p->k2_variant, p->stream));
           const int2* pts = warps ? p->d_pts3w : p->d_pts3;
           const int npts = warps ? p->n_pts3w : p->n_pts3;
-          if (p->C == 1 && npts > 0)
-            SS_TRY(p, launch_k2_points(p->d_spec + cb.c[0] * chan_stride, p->Mp, cnt, p->m, pts,
-                                       npts, p->M, pref3, acc3, plane, p->stream));
+          if (p->C == 1 && npts > 0 && !all)
+            SS_TRY(p, launch_k2_points(spec + cb.c[0] * chan_stride, p->Ms, cnt, p->m, pts, npts,
+                                       p->M, pref3, acc3, plane, p->stream));
         }
         record(p, 1, p->stream, false);
       }
@@ -351,7 +365,7 @@ ss_status process_device(ss_plan_s* p, const void* ptr, long long n, long long s
         record(p, 2, p->stream, true);
         const long long plane = (long long)p->c4.size() * p->rows4 * p->M;
         if (p->C > 1 && p->precision == SS_PREC_FP32)
-          SS_TRY(p, launch_k3_trispec_cross(p->d_spec, chan_stride, cnt, p->m, p->M, p->Mp,
+          SS_TRY(p, launch_k3_trispec_cross(spec, chan_stride, cnt, p->m, p->M, p->Ms,
                                             p->d_c4cross, (int)p->c4.size(), p->d_acc4, plane,
                                             p->nsm, nat, p->stream));
         else if (p->C > 1) {
@@ -381,7 +395,7 @@ ss_status process_device(ss_plan_s* p, const void* ptr, long long n, long long s
                                            p->d_acc4 + (long long)i * p->rows4 * p->M, plane,
                                            p->nsm, p->d_counter, p->d_status, p->stream));
           if (p->precision != SS_PREC_FP32 && p->col4)
-            SS_TRY(p, launch_k3_column(p->d_spec + cb.c[0] * chan_stride, p->Mp, cnt, p->m,
+            SS_TRY(p, launch_k3_column(spec + cb.c[0] * chan_stride, p->Ms, cnt, p->m,
                                        p->M, pref4a, pref4b,
                                        p->d_acc4 + (long long)i * p->rows4 * p->M, plane,
                                        p->stream));
@@ -394,7 +408,7 @@ ss_status process_device(ss_plan_s* p, const void* ptr, long long n, long long s
         record(p, 2, p->stream, true);
         const int n_cx = (int)(p->cx_ops[o].size() / (o + 2));
         const long long cplane = (long long)p->n_cx_acc[o] / kPlanes;
-        SS_TRY(p, launch_k5_complex(p->d_spec, chan_stride, cnt, p->m, p->M, p->Mp, o + 2,
+        SS_TRY(p, launch_k5_complex(spec, chan_stride, cnt, p->m, p->M, p->Ms, o + 2,
                                     p->d_cx_ops[o], n_cx, p->cx_shift, nat, p->d_cx_acc[o],
                                     cplane, p->nsm, p->stream));
         record(p, 2, p->stream, false);
@@ -548,13 +562,14 @@ ss_status encode_maps(ss_plan_s* p) {
   }
   const cuuint64_t rows = (cuuint64_t)p->C * p->Gb_max * p->m;
   const cuuint64_t dims[3] = {16, (cuuint64_t)p->Mp / 16, rows};
-  const cuuint64_t strides[2] = {16 * sizeof(float2), (cuuint64_t)p->Mp * sizeof(float2)};
+  const cuuint64_t strides[2] = {16 * sizeof(float2), (cuuint64_t)p->Ms * sizeof(float2)};
+  const cuuint64_t wdims[3] = {16, (cuuint64_t)p->Ms / 16, rows};  // with the bins below 0
   const cuuint32_t estr[3] = {1, 1, 1};
   for (int blocks : {3, 4, 8}) {
     const cuuint32_t box[3] = {16, (cuuint32_t)blocks, (cuuint32_t)p->FC};
     CUtensorMap* map = blocks == 3 ? &p->tm48 : blocks == 4 ? &p->tm64 : &p->tm128;
     CUresult r = encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 3,
-                        p->d_spec, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                        p->d_spec + p->Z, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                         CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS)
@@ -563,7 +578,7 @@ ss_status encode_maps(ss_plan_s* p) {
   for (int blocks : {2, 4}) {  // boxes of kFrames84w rows for k2_bispec84w
     const cuuint32_t box[3] = {16, (cuuint32_t)blocks, (cuuint32_t)kFrames84w};
     CUresult r = encode(blocks == 2 ? &p->tm32w : &p->tm64w, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 3,
-                        p->d_spec, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                        p->d_spec, wdims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                         CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS)
@@ -575,14 +590,14 @@ ss_status encode_maps(ss_plan_s* p) {
     // (c and d); the widths differ between the two forms
     const cuuint32_t fr = p->precision == SS_PREC_FP16X3 ? 8 : 4;
     const cuuint64_t d2[2] = {(cuuint64_t)p->Mp, rows};
-    const cuuint64_t s2[1] = {(cuuint64_t)p->Mp * sizeof(float2)};
+    const cuuint64_t s2[1] = {(cuuint64_t)p->Ms * sizeof(float2)};
     const cuuint32_t e2[2] = {1, 1};
     const bool h = p->precision == SS_PREC_FP16X3;
     const cuuint32_t bab[2] = {(cuuint32_t)std::min(h ? kCrossBoxBinsH : kCrossBoxBins, p->Mp), fr};
     const cuuint32_t bcd[2] = {(cuuint32_t)(h ? kCrossColBoxH : kCrossColBox), fr};
     for (int i = 0; i < 2; ++i) {
       CUresult r = encode(i == 0 ? &p->tmx_ab : &p->tmx_cd, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 2,
-                          p->d_spec, d2, s2, i == 0 ? bab : bcd, e2,
+                          p->d_spec + p->Z, d2, s2, i == 0 ? bab : bcd, e2,
                           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
                           CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
       if (r != CUDA_SUCCESS)
@@ -661,7 +676,7 @@ ss_status alloc_spec(ss_plan_s* p) {
       ptr = nullptr;
     }
   };
-  const size_t spec_group = (size_t)p->C * p->m * p->Mp * sizeof(float2);
+  const size_t spec_group = (size_t)p->C * p->m * p->Ms * sizeof(float2);
   const bool image = p->C == 1 && !p->c4.empty() && p->precision != SS_PREC_FP32;
   // Gram image: ceil(m/16) diagonal chunks, then ceil((m(m-1)/2 + 1) / 16) chunks
   // of the pairs and ps
@@ -700,6 +715,8 @@ ss_status alloc_spec(ss_plan_s* p) {
   if ((long long)p->C * gb * p->m > max_rows) gb = (int)(max_rows / ((long long)p->C * p->m));
   p->Gb_max = gb;
   SS_TRY(p, dev_alloc(p, &p->d_spec, spec_group * gb));
+  // the bins below -(M - 1) of mirrored rows are read (as zeros) but never written
+  if (p->mirror) SS_TRY(p, cudaMemsetAsync(p->d_spec, 0, spec_group * gb, p->stream));
   p->oi = OperandImage();
   if (image) {
     SS_TRY(p, dev_alloc(p, &p->oi.img, img_group * gb));
@@ -757,6 +774,7 @@ void destroy(ss_plan_s* p) {
   cudaFree(p->d_pts3);
   cudaFree(p->d_tiles3w);
   cudaFree(p->d_pts3w);
+  cudaFree(p->d_c3);
   cudaFree(p->d_tiles4);
   cudaFree(p->d_tiles4tc);
   cudaFree(p->d_c4cross);
@@ -857,6 +875,9 @@ static ss_status plan_create(ss_plan_t* out, int channels, int T, double dt, int
     return fail(nullptr, SS_EUNSUPPORTED,
                 "the tensor-core S4 precisions take m <= 32 frames per group; use fp32");
   }
+  p->mirror = channels > 1 && !p->c3.empty();
+  p->Z = p->mirror ? (p->M - 1 + 31) & ~31 : 0;  // whole sub-tiles of 32 bins below bin 0
+  p->Ms = p->Z + p->Mp;
   p->rows3 = channels == 1 ? p->M : 2 * p->M - 1;
   p->rows4 = channels == 1 ? p->M : 2 * p->M - 1;
 
@@ -921,11 +942,11 @@ static ss_status plan_create(ss_plan_t* out, int channels, int T, double dt, int
   if (p->c4.empty() || channels > 1) t4.clear();  // several channels: k3_trispec_cross
   std::vector<TileInfo> t3w;
   std::vector<int2> pts3w;
-  if (channels == 1 && !p->c3.empty()) build_warp_tiles(p->M, t3w, pts3w);
+  if (!p->c3.empty()) build_warp_tiles(p->M, channels > 1, t3w, pts3w, &p->n_tiles3w);
   p->n_tiles3 = (int)t3.size();
   p->n_tiles4 = (int)t4.size();
   p->n_pts3 = (int)pts3.size();
-  p->n_tiles3w = (int)t3w.size();
+  p->n_tiles3a = (int)t3w.size();
   p->n_pts3w = (int)pts3w.size();
 
 #define PLAN_TRY(call)                           \
@@ -957,6 +978,12 @@ static ss_status plan_create(ss_plan_t* out, int channels, int T, double dt, int
   if (!pts3w.empty()) PLAN_TRY(dev_alloc(p, &p->d_pts3w, pts3w.size() * sizeof(int2)));
   if (!t4.empty()) PLAN_TRY(dev_alloc(p, &p->d_tiles4, t4.size() * sizeof(TileInfo)));
   if (!t4tc.empty()) PLAN_TRY(dev_alloc(p, &p->d_tiles4tc, t4tc.size() * sizeof(TileInfo)));
+  if (!p->c3.empty()) {
+    std::vector<int4> c3x;
+    for (const Combo& cb : p->c3) c3x.push_back(make_int4(cb.c[0], cb.c[1], cb.c[2], 0));
+    PLAN_TRY(dev_alloc(p, &p->d_c3, c3x.size() * sizeof(int4)));
+    PLAN_TRY(cudaMemcpy(p->d_c3, c3x.data(), c3x.size() * sizeof(int4), cudaMemcpyHostToDevice));
+  }
   std::vector<int4> c4x;
   if (channels > 1)
     for (const Combo& cb : p->c4) c4x.push_back(make_int4(cb.c[0], cb.c[1], cb.c[2], cb.c[3]));
@@ -1395,7 +1422,9 @@ ss_status ss_query(ss_plan_t p, ss_info* info) {
   info->groups_per_batch = p->Gb_max;
   info->device_bytes = p->device_bytes;
   info->kernels_per_batch = 1 + (p->n_s2cross > 0 ? 1 : 0) +
-                            (int)p->c3.size() * (1 + (p->C == 1 && p->n_pts3 > 0 ? 1 : 0)) +
+                            (p->k2_variant == kK2Warp84
+                                 ? (p->c3.empty() ? 0 : 1 + (p->n_pts3w > 0 ? (int)p->c3.size() : 0))
+                                 : (int)p->c3.size() * (1 + (p->C == 1 && p->n_pts3 > 0 ? 1 : 0))) +
                             (p->C > 1 ? (p->c4.empty() ? 0 : p->precision == SS_PREC_FP32 ? 1 : 2)
                                       : (int)p->c4.size() *
                                             (1 + (p->precision != SS_PREC_FP32 && p->col4 ? 1 : 0)));
@@ -1442,8 +1471,7 @@ ss_status ss_layout_warps(int T, int* tiles, int max_tiles, int* n, int* points,
   if (!n || !np) return fail(nullptr, SS_EINVAL, "NULL count argument");
   std::vector<TileInfo> t;
   std::vector<int2> pts;
-  build_warp_tiles(T / 2 + 1, t, pts);
-  *n = (int)t.size();
+  build_warp_tiles(T / 2 + 1, false, t, pts, n);
   *np = (int)pts.size();
   for (int i = 0; i < *n && i < max_tiles && tiles; ++i) {
     tiles[2 * i] = t[i].k0;

@@ -31,7 +31,11 @@ struct ss_plan_s {
   float2* d_tw = nullptr;
   void* d_carry = nullptr;
   long long carry_n = 0;
+  // rows of Ms coefficients, bin 0 at column Z; Z = 0 and Ms = Mp, or with mirrored
+  // rows (several channels with S3) the bins -(M - 1) .. -1 before it
   float2* d_spec = nullptr;
+  int Z = 0, Ms = 0;
+  bool mirror = false;
   int Gb_max = 0, Gb_user = 0;
   double *d_acc1 = nullptr, *d_acc2 = nullptr, *d_acc3 = nullptr, *d_acc4 = nullptr;
   size_t n_acc1 = 0, n_acc2 = 0, n_acc3 = 0, n_acc4 = 0;
@@ -48,7 +52,7 @@ struct ss_plan_s {
   ss::TileInfo *d_tiles3 = nullptr, *d_tiles4 = nullptr;
   int* d_status = nullptr;
   int inject_timeout = 0;          // timeout test: K2 runs one bounded wait out
-  int k2_variant = ss::kK2Tile84Stages2;  // K2 tiling (set by the autotuner or ss_set_tuning)
+  int k2_variant = ss::kK2Warp84;  // K2 tiling (set by the autotuner or ss_set_tuning)
   int k1_mode = ss::kK1Auto;              // K1 form (likewise)
   float tune_ms[ss::kK1Modes + ss::kK2Variants] = {};  // last ss_autotune: pass ms per form
   // sequential spectra (Sec. 8): every seq_B groups, the block's means and errors
@@ -82,7 +86,9 @@ struct ss_plan_s {
   // the independent-warp K2 form: its 32 x 32 sub-tiles and their isolated points
   ss::TileInfo* d_tiles3w = nullptr;
   int2* d_pts3w = nullptr;
-  int n_tiles3w = 0, n_pts3w = 0;
+  // (the sub-tiles of the isolated points follow the others: n_tiles3a of all)
+  int n_tiles3w = 0, n_tiles3a = 0, n_pts3w = 0;
+  int4* d_c3 = nullptr;  // channel triples of the S3 combinations
   bool col4 = false;       // the S4 column l = M - 1 is left to k3_column
   int n_pts3 = 0;
   long long pairs3 = 0, pairs4 = 0;
