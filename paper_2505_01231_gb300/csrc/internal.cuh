@@ -87,13 +87,23 @@ struct Combo {
 // largest entry (at most max(max(sd, so) max_j |d_jk|^2, sp Sk)) below 2^14, so
 // that hi and lo stay inside the FP16 range; rsc holds 1/s_k per group and bin,
 // and the kernel divides D by s_k and by s_l (exactly: powers of two).
-enum { kImageNone = 0, kImageGramTF32 = 1, kImageGramBF16 = 2, kImageGramF16 = 3 };
+// F32 (k3_trispec_gram, CUDA cores): the entries unsplit and unscaled, one row of Mp
+// bins per entry, rows rows a group: the pairs, ps, the diagonal, then zeros up to a
+// multiple of kGram32Rows.
+enum { kImageNone = 0, kImageGramTF32 = 1, kImageGramBF16 = 2, kImageGramF16 = 3,
+       kImageGramF32 = 4 };
+constexpr int kGram32Rows = 8;   // entry rows of a stage of k3_trispec_gram
+// Largest m of k3_trispec_gram; K1 and S4 with it against k3_trispec at T = 1024, 2^24
+// samples (ms): m = 5 0.58 / 1.56, 10 0.72 / 1.21, 14 0.91 / 1.13, 16 0.99 / 1.09 (m = 17
+// with k3_trispec 1.24).
+constexpr int kGram32MaxM = 16;
 constexpr int kMaxGramM = 32;  // largest m of the tensor-core S4 path
 struct OperandImage {
   void* img = nullptr;
   float* rsc = nullptr;       // FP16: per group and bin, 1 / the bin's row scale
   int fmt = kImageNone;
   int nkc = 0, ndc = 0;       // K chunks, of which diagonal
+  int rows = 0;               // F32: entry rows of a group
   float sd = 0.f, so = 0.f, sp = 0.f;
   long long rg_bytes = 0;     // nkc * 2 * CB
   long long group_bytes = 0;  // (Mp / 8) * rg_bytes
@@ -153,6 +163,16 @@ cudaError_t launch_k3_trispec(const CUtensorMap& tm64, int row0, int G, int m, i
                               const TileInfo* tiles, int n_tiles, float pref4a, float pref4b,
                               double* acc, long long plane, int nsm, int* counter, int* status,
                               cudaStream_t stream);
+
+// The FP32 form for groups of at most kGram32MaxM frames: K1's F32 operand image
+// through 2-D views [group x rows][Mp] with boxes of 32 (tm32) and 64 (tm64) bins x
+// kGram32Rows rows; tiles of 32 x 64 (k, l) bins below lim, sums stored at [k][l].
+// Blocks of groups as for launch_k2_bispec84w.
+cudaError_t launch_k3_trispec_gram(const CUtensorMap& tm32, const CUtensorMap& tm64,
+                                   const OperandImage& oi, int G, int m, int M, int lim,
+                                   const TileInfo* tiles, int n_tiles, double* acc,
+                                   long long plane, int block_groups, long long block_stride,
+                                   int nsm, int* counter, int* status, cudaStream_t stream);
 
 // Tensor-core form of K3 (SS_PREC_TF32X3, SS_PREC_BF16X3, SS_PREC_BF16): tiles of
 // 128 x 128 (k, l) bins, the weighted frame-Gram contraction fed from K1's
@@ -231,26 +251,29 @@ cudaError_t launch_k5_complex(const float2* spec, long long chan_stride, int G, 
                               bool natural, double* acc, long long plane, int nsm,
                               cudaStream_t stream);
 
-// Groups of an item of k2_bispec84w, for blocks of G groups times
+// Groups of an item of k2_bispec84w or k3_trispec_gram, for blocks of G groups times
 // `tiles` (tiles, combinations and blocks).  Estimated, in clocks: a group takes a warp
-// `group` with the SM's 16 warps at work (1.6 times less work gets done in that time
-// where a warp has its scheduler to itself), an item 1500 more, and its `adds` float64
-// additions are taken by the L2 at about 200 a clock over the whole GPU.  A warp takes
-// a quarter of the groups, at most kMaxFp32Groups of them.  Measured (ms, K2 alone)
-// for 4 / 16 / 64 groups: T = 1024, m = 10, 2^28 samples 10.21 / 7.34 / 6.75; T = 128,
-// m = 32, 2^23 samples 0.113 / 0.130 / 0.166 (8 groups: 0.108); T = 256, m = 10, 2^20
-// samples 0.033 / 0.040 / 0.062.
+// `group` with the SM full, up to 1.75 times that with fewer items on an SM than it
+// holds; an item 1500 more; the last items of an SM end unevenly; and the `adds`
+// float64 additions of an item are taken by the L2 at about 200 a clock over the whole
+// GPU.  At most kMaxFp32Groups (a warp takes a quarter).  Measured (ms, K2 alone) for
+// 4 / 8 / 16 / 64 groups: T = 1024, m = 10, 2^28 samples 10.21 / 8.20 / 7.34 / 6.75;
+// T = 128, m = 32, 2^23 samples 0.113 / 0.108 / 0.130 / 0.166; T = 256, m = 10, 2^20
+// samples 0.033 / 0.033 / 0.040 / 0.062.
 inline int warp_item_groups(int G, long long tiles, int nsm, double group, int adds) {
   int best = 1;
   double tb = 1e300;
-  const int top = G < 4 * kMaxFp32Groups ? G : 4 * kMaxFp32Groups;
+  const int top = G < kMaxFp32Groups ? G : kMaxFp32Groups;
   for (int gc = 1; gc <= top; ++gc) {
     const long long items = (long long)((G + gc - 1) / gc) * tiles;
     const double item = ((gc + 3) / 4) * group + 1500.0;
     const long long full = (items + nsm - 1) / nsm;  // items of the busiest SM
-    const double rounds = full <= 4 ? (double)full : (double)items / nsm + 1.0;
-    const double alone = full == 1 ? 1.6 : full == 2 ? 1.1 : 1.0;
-    const double t = rounds * item * alone + (double)items * (adds / 200.0);
+    const double rounds = full == 1   ? 1.75
+                          : full == 2 ? 2 * 1.5
+                          : full == 3 ? 3 * 1.3
+                          : full == 4 ? 4 * 1.1
+                                      : (double)items / nsm + 1.0;
+    const double t = rounds * item + (double)items * (adds / 200.0);
     if (t < tb) {
       tb = t;
       best = gc;
@@ -279,9 +302,10 @@ cudaError_t launch_k2_points(const float2* spec, int Mp, int G, int m, const int
                              int n_pts, int M, float pref3, double* acc, long long plane,
                              cudaStream_t stream);
 
-// the one-channel S4 cut at l = M - 1 for every k, stored at [l][k]
+// the one-channel S4 cut at l = M - 1 for every k, stored at acc[k * sk + l * sl]
 cudaError_t launch_k3_column(const float2* spec, int Mp, int G, int m, int M, float pref4a,
-                             float pref4b, double* acc, long long plane, cudaStream_t stream);
+                             float pref4b, double* acc, long long plane, int sk, int sl,
+                             cudaStream_t stream);
 
 // dynamic shared memory of the pair kernels for FC frames per stage
 size_t k2_smem_bytes(int FC);

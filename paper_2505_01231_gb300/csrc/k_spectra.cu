@@ -250,7 +250,19 @@ __device__ __forceinline__ void centre_bin(int k, bool valid, float2 mean, int m
     const float sd = oi.sd * sc, so = oi.so * sc, sps = oi.sp * p * sc;
     const int npair = m * (m - 1) / 2;
     int pj = 0, pk = 1;  // next off-diagonal pair (j, j'), lexicographic
-    if (k < oi.img_bins) {  // rows the tensor-core S4 reads
+    if (FMT == kImageGramF32) {
+      if (k < oi.img_bins) {
+        float* e = static_cast<float*>(oi.img) + (size_t)g * oi.rows * Mp + k;
+        const int nd = npair + 1;
+        for (int j = 0; j < m; ++j) {
+          for (int q = j + 1; q < m; ++q, e += Mp) *e = so * fmaf(dr[j], dr[q], di[j] * di[q]);
+        }
+        *e = sps;
+        e += Mp;
+        for (int j = 0; j < m; ++j, e += Mp) *e = sd * fmaf(dr[j], dr[j], di[j] * di[j]);
+        for (int r = nd + m; r < oi.rows; ++r, e += Mp) *e = 0.f;
+      }
+    } else if (k < oi.img_bins) {  // rows the tensor-core S4 reads
       constexpr int kChunkBytes = FMT == kImageGramTF32 ? 1024 : 512;  // 2 CB
       unsigned char* rbase = static_cast<unsigned char*>(oi.img) + (size_t)c * oi.chan_bytes +
                              (size_t)g * oi.group_bytes + (size_t)(k >> 3) * oi.rg_bytes +
@@ -468,7 +480,26 @@ __device__ __forceinline__ void centre_resident(float2* Xs, float2* __restrict__
     }
     // several channels in FP16X3: the bin's row scale
     if (oi.rmax) oi.rmax[(long long)c * oi.chan_rmax + (long long)g * Mp + k] = cross_row_scale(mx);
-    if (FMT != kImageNone && k < oi.img_bins) {  // rows the tensor-core S4 reads
+    if (FMT == kImageGramF32 && k < oi.img_bins) {
+      // the bin's column of entry rows: pairs, ps, diagonal, zeros
+      float* e = static_cast<float*>(oi.img) + (size_t)g * oi.rows * Mp + k;
+      for (int j = 0; j < m; ++j) {
+        const float2 dj = Xs[j * Mp + k];
+#pragma unroll 4
+        for (int q = j + 1; q < m; ++q) {
+          const float2 dq = Xs[q * Mp + k];
+          *e = oi.so * fmaf(dj.x, dq.x, dj.y * dq.y);
+          e += Mp;
+        }
+      }
+      *e = oi.sp * p;
+      e += Mp;
+      for (int j = 0; j < m; ++j, e += Mp) {
+        const float2 dj = Xs[j * Mp + k];
+        *e = oi.sd * fmaf(dj.x, dj.x, dj.y * dj.y);
+      }
+      for (int r = m * (m + 1) / 2 + 1; r < oi.rows; ++r, e += Mp) *e = 0.f;
+    } else if (FMT != kImageNone && k < oi.img_bins) {  // rows the tensor-core S4 reads
       const float sc =
         FMT == kImageGramF16 ? f16_row_scale(fmaxf(fmaxf(oi.sd, oi.so) * mx, oi.sp * p)) : 1.f;
       const float sd = oi.sd * sc, so = oi.so * sc, sps = oi.sp * p * sc;
@@ -998,6 +1029,9 @@ cudaError_t launch_k1_spectra(const SampleSource& src, long long sample0, int G,
     case kImageGramBF16:
       return f32 ? launch_k1_t<SS_F32, kImageGramBF16>(K1_ARGS)
                  : launch_k1_t<SS_I16, kImageGramBF16>(K1_ARGS);
+    case kImageGramF32:
+      return f32 ? launch_k1_t<SS_F32, kImageGramF32>(K1_ARGS)
+                 : launch_k1_t<SS_I16, kImageGramF32>(K1_ARGS);
     case kImageGramF16:
       return f32 ? launch_k1_t<SS_F32, kImageGramF16>(K1_ARGS)
                  : launch_k1_t<SS_I16, kImageGramF16>(K1_ARGS);

@@ -230,13 +230,12 @@ cudaError_t launch_k3_trispec(const CUtensorMap& tm64, int row0, int G, int m, i
 // tiles leave it out when it is the only column of its block): one thread per
 // k, the same five length-m sums as above per group, reading the centred
 // coefficients from global memory (consecutive k are consecutive addresses; the
-// bin-l values are the same address across a warp).  Written at [l][k], the
-// layout of the tensor-core kernel's accumulators.
+// bin-l values are the same address across a warp).
 constexpr int kColThreads = 128;
 
 __global__ void __launch_bounds__(kColThreads)
 k3_column(const float2* __restrict__ spec, int Mp, int G, int m, int M, float pref_a,
-          float pref_b, double* __restrict__ acc, long long plane) {
+          float pref_b, double* __restrict__ acc, long long plane, int sk_out, int sl_out) {
   const int k = blockIdx.x * kColThreads + threadIdx.x;
   const int l = M - 1;
   if (k >= M) return;
@@ -263,19 +262,20 @@ k3_column(const float2* __restrict__ spec, int Mp, int G, int m, int M, float pr
     sum += c4;
     sq = fmaf(c4, c4, sq);
   }
-  const long long o = (long long)l * M + k;
+  const long long o = (long long)l * sl_out + (long long)k * sk_out;
   atomicAdd(acc + o, (double)sum);
   atomicAdd(acc + 2 * plane + o, (double)sq);
 }
 
 cudaError_t launch_k3_column(const float2* spec, int Mp, int G, int m, int M, float pref4a,
-                             float pref4b, double* acc, long long plane, cudaStream_t stream) {
+                             float pref4b, double* acc, long long plane, int sk, int sl,
+                             cudaStream_t stream) {
   if (G <= 0 || M <= 0) return cudaSuccess;
   const int gx = (M + kColThreads - 1) / kColThreads;
   // at most kMaxFp32Groups groups in a thread's float32 sums (grid y <= 65535)
   const int gy = std::min(G, std::min(65535, std::max(1024, (G + kMaxFp32Groups - 1) / kMaxFp32Groups)));
   k3_column<<<dim3((unsigned)gx, (unsigned)gy), kColThreads, 0, stream>>>(
-      spec, Mp, G, m, M, pref4a, pref4b, acc, plane);
+      spec, Mp, G, m, M, pref4a, pref4b, acc, plane, sk, sl);
   return cudaGetLastError();
 }
 

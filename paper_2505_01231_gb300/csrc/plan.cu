@@ -137,6 +137,18 @@ std::vector<TileInfo> build_tc_tiles(int M, bool* last_col) {
   return t;
 }
 
+// Tiles of k3_trispec_gram: 32 k-bins by 64 l-bins that touch the upper triangle
+// k <= l.  A last column block that holds only l = M - 1 (T >= 128) is left to
+// k3_column (*last_col = true).
+std::vector<TileInfo> build_gram_tiles(int M, bool* last_col) {
+  std::vector<TileInfo> t;
+  *last_col = (M - 1) % 64 == 0;
+  const int lim = *last_col ? M - 1 : M;
+  for (int l0 = 0; l0 < lim; l0 += 64)
+    for (int k0 = 0; k0 < lim && k0 <= l0 + 63; k0 += 32) t.push_back(TileInfo{k0, l0, 4, 64});
+  return t;
+}
+
 // Tiles of 64 x 64 grid points that touch the domain, with the number of
 // their 32 x 16 warp sub-tiles that touch it (the kernels skip the others).
 // A one-channel S3 tile holding at most this many domain points (the corner
@@ -383,7 +395,13 @@ ss_status process_device(ss_plan_s* p, const void* ptr, long long n, long long s
         }
         for (size_t i = 0; i < p->c4.size() && p->C == 1; ++i) {
           const Combo& cb = p->c4[i];
-          if (p->precision == SS_PREC_FP32)
+          if (p->gram32)
+            SS_TRY(p, launch_k3_trispec_gram(
+                          p->tm_g32, p->tm_g64, p->oi, cnt, p->m, p->M,
+                          p->col4 ? p->M - 1 : p->M, p->d_tiles4g, p->n_tiles4g,
+                          p->d_acc4 + (long long)i * p->rows4 * p->M, plane, 0, 0, p->nsm,
+                          p->d_counter, p->d_status, p->stream));
+          else if (p->precision == SS_PREC_FP32)
             SS_TRY(p, launch_k3_trispec(p->tm64, cb.c[0] * p->Gb_max * p->m, cnt, p->m, p->FC,
                                         p->M, p->d_tiles4, p->n_tiles4, pref4a, pref4b,
                                         p->d_acc4 + (long long)i * p->rows4 * p->M, plane,
@@ -394,11 +412,11 @@ ss_status process_device(ss_plan_s* p, const void* ptr, long long n, long long s
                                            p->d_tiles4tc, p->n_tiles4tc, p->precision,
                                            p->d_acc4 + (long long)i * p->rows4 * p->M, plane,
                                            p->nsm, p->d_counter, p->d_status, p->stream));
-          if (p->precision != SS_PREC_FP32 && p->col4)
+          if (p->col4)
             SS_TRY(p, launch_k3_column(spec + cb.c[0] * chan_stride, p->Ms, cnt, p->m,
                                        p->M, pref4a, pref4b,
                                        p->d_acc4 + (long long)i * p->rows4 * p->M, plane,
-                                       p->stream));
+                                       p->gram32 ? p->M : 1, p->gram32 ? 1 : p->M, p->stream));
         }
         record(p, 2, p->stream, false);
       }
@@ -622,7 +640,22 @@ ss_status encode_maps(ss_plan_s* p) {
                     "cuTensorMapEncodeTiled (cross maxima) failed with code " + std::to_string(r));
     }
   }
-  if (p->oi.img) {
+  if (p->oi.fmt == kImageGramF32) {
+    // F32 operand image as [group x entry row][Mp] floats
+    const cuuint64_t gdims[2] = {(cuuint64_t)p->Mp, (cuuint64_t)p->Gb_max * p->oi.rows};
+    const cuuint64_t gstr[1] = {(cuuint64_t)p->Mp * sizeof(float)};
+    const cuuint32_t e2[2] = {1, 1};
+    for (int bins : {32, 64}) {
+      const cuuint32_t gbox[2] = {(cuuint32_t)bins, (cuuint32_t)kGram32Rows};
+      CUresult r = encode(bins == 32 ? &p->tm_g32 : &p->tm_g64, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2,
+                          p->oi.img, gdims, gstr, gbox, e2, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                          CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+      if (r != CUDA_SUCCESS)
+        return fail(p, SS_ECUDA,
+                    "cuTensorMapEncodeTiled (F32 image) failed with code " + std::to_string(r));
+    }
+  } else if (p->oi.img) {
     // Gram operand image of each channel as [group][row group][chunk][2 CB bytes]
     // in 8-byte elements; a box is the stage's chunks of 16 row groups of one group
     const cuuint64_t cbytes = p->oi.rg_bytes / p->oi.nkc;  // 2 CB
@@ -677,14 +710,17 @@ ss_status alloc_spec(ss_plan_s* p) {
     }
   };
   const size_t spec_group = (size_t)p->C * p->m * p->Ms * sizeof(float2);
-  const bool image = p->C == 1 && !p->c4.empty() && p->precision != SS_PREC_FP32;
+  const bool image = p->C == 1 && !p->c4.empty() && (p->precision != SS_PREC_FP32 || p->gram32);
   // Gram image: ceil(m/16) diagonal chunks, then ceil((m(m-1)/2 + 1) / 16) chunks
   // of the pairs and ps
   const int ndc = (p->m + 15) / 16;
   const int nkc = ndc + (p->m * (p->m - 1) / 2 + 16) / 16;
   const size_t cb = p->precision == SS_PREC_TF32X3 ? 512 : 256;
   const size_t rg_bytes = (size_t)nkc * 2 * cb;
-  const size_t group_bytes = (size_t)(p->Mp / 8) * rg_bytes;
+  // F32 image: the entries in rows of Mp floats, a multiple of kGram32Rows rows
+  const int grows = (p->m * (p->m + 1) / 2 + kGram32Rows) / kGram32Rows * kGram32Rows;
+  const size_t group_bytes = p->gram32 ? (size_t)grows * p->Mp * sizeof(float)
+                                       : (size_t)(p->Mp / 8) * rg_bytes;
   const size_t img_group = image ? (size_t)p->C * group_bytes : 0;
   // FP16: the bins' row scales per group
   const bool scaled = image && p->precision == SS_PREC_FP16X3;
@@ -710,9 +746,10 @@ ss_status alloc_spec(ss_plan_s* p) {
     // about 4 GiB of per-batch scratch, at least one group
     gb = (int)std::max<size_t>(1, (size_t)(4096ull << 20) / per_group);
   }
-  // the 3-D views index rows with 32-bit coordinates
+  // the views index rows with 32-bit coordinates
   const long long max_rows = (1ll << 31) - 1;
-  if ((long long)p->C * gb * p->m > max_rows) gb = (int)(max_rows / ((long long)p->C * p->m));
+  const long long group_rows = std::max((long long)p->C * p->m, p->gram32 ? (long long)grows : 0ll);
+  if (gb * group_rows > max_rows) gb = (int)(max_rows / group_rows);
   p->Gb_max = gb;
   SS_TRY(p, dev_alloc(p, &p->d_spec, spec_group * gb));
   // the bins below -(M - 1) of mirrored rows are read (as zeros) but never written
@@ -721,7 +758,9 @@ ss_status alloc_spec(ss_plan_s* p) {
   if (image) {
     SS_TRY(p, dev_alloc(p, &p->oi.img, img_group * gb));
     if (scaled) SS_TRY(p, dev_alloc(p, &p->oi.rsc, rsc_group * gb));
-    p->oi.fmt = p->precision == SS_PREC_TF32X3   ? kImageGramTF32
+    p->oi.rows = p->gram32 ? grows : 0;
+    p->oi.fmt = p->gram32                        ? kImageGramF32
+                : p->precision == SS_PREC_TF32X3 ? kImageGramTF32
                 : p->precision == SS_PREC_FP16X3 ? kImageGramF16
                                                  : kImageGramBF16;
     p->oi.nkc = nkc;
@@ -775,6 +814,7 @@ void destroy(ss_plan_s* p) {
   cudaFree(p->d_tiles3w);
   cudaFree(p->d_pts3w);
   cudaFree(p->d_c3);
+  cudaFree(p->d_tiles4g);
   cudaFree(p->d_tiles4);
   cudaFree(p->d_tiles4tc);
   cudaFree(p->d_c4cross);
@@ -935,11 +975,15 @@ static ss_status plan_create(ss_plan_t* out, int channels, int T, double dt, int
   if (channels == 1 && !p->c4.empty() && precision != SS_PREC_FP32)
     t4tc = build_tc_tiles(p->M, &p->col4);
   p->n_tiles4tc = (int)t4tc.size();
+  std::vector<TileInfo> t4g;
+  p->gram32 = channels == 1 && !p->c4.empty() && precision == SS_PREC_FP32 && m <= kGram32MaxM;
+  if (p->gram32) t4g = build_gram_tiles(p->M, &p->col4);
+  p->n_tiles4g = (int)t4g.size();
   if (p->c3.empty()) {
     t3.clear();
     pts3.clear();
   }
-  if (p->c4.empty() || channels > 1) t4.clear();  // several channels: k3_trispec_cross
+  if (p->c4.empty() || channels > 1 || p->gram32) t4.clear();  // several channels: k3_trispec_cross
   std::vector<TileInfo> t3w;
   std::vector<int2> pts3w;
   if (!p->c3.empty()) build_warp_tiles(p->M, channels > 1, t3w, pts3w, &p->n_tiles3w);
@@ -978,6 +1022,11 @@ static ss_status plan_create(ss_plan_t* out, int channels, int T, double dt, int
   if (!pts3w.empty()) PLAN_TRY(dev_alloc(p, &p->d_pts3w, pts3w.size() * sizeof(int2)));
   if (!t4.empty()) PLAN_TRY(dev_alloc(p, &p->d_tiles4, t4.size() * sizeof(TileInfo)));
   if (!t4tc.empty()) PLAN_TRY(dev_alloc(p, &p->d_tiles4tc, t4tc.size() * sizeof(TileInfo)));
+  if (!t4g.empty()) {
+    PLAN_TRY(dev_alloc(p, &p->d_tiles4g, t4g.size() * sizeof(TileInfo)));
+    PLAN_TRY(cudaMemcpy(p->d_tiles4g, t4g.data(), t4g.size() * sizeof(TileInfo),
+                        cudaMemcpyHostToDevice));
+  }
   if (!p->c3.empty()) {
     std::vector<int4> c3x;
     for (const Combo& cb : p->c3) c3x.push_back(make_int4(cb.c[0], cb.c[1], cb.c[2], 0));
@@ -1427,7 +1476,7 @@ ss_status ss_query(ss_plan_t p, ss_info* info) {
                                  : (int)p->c3.size() * (1 + (p->C == 1 && p->n_pts3 > 0 ? 1 : 0))) +
                             (p->C > 1 ? (p->c4.empty() ? 0 : p->precision == SS_PREC_FP32 ? 1 : 2)
                                       : (int)p->c4.size() *
-                                            (1 + (p->precision != SS_PREC_FP32 && p->col4 ? 1 : 0)));
+                                            (1 + (p->col4 ? 1 : 0)));
   return SS_OK;
 }
 
@@ -1765,7 +1814,11 @@ ss_status ss_plan_many(ss_many_t* out, int n_rec, const int* T, const size_t* ma
       return many_fail(nullptr, SS_EINVAL,
                        "recording " + std::to_string(i) + " holds fewer than two groups");
     const int Mp = ((T[i] / 2 + 1) + 15) & ~15;
-    total += (double)groups[i] * m * Mp * 8.0 * (precision == SS_PREC_FP32 ? 1.0 : 5.0);
+    // spectra and, with S4 of small groups or on tensor cores, the operand image
+    const double per_bin = precision != SS_PREC_FP32               ? 40.0 * m
+                           : (orders & SS_ORDER4) && m <= kGram32MaxM ? 8.0 * m + 2.0 * m * (m + 1) + 32.0
+                                                                      : 8.0 * m;
+    total += (double)groups[i] * Mp * per_bin;
   }
   ss_many_s* mp = new ss_many_s();
   mp->stream = static_cast<cudaStream_t>(stream);

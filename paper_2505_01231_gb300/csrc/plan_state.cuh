@@ -76,10 +76,15 @@ struct ss_plan_s {
   CUtensorMap tm32w{}, tm64w{};          // the same with boxes of kFrames84w rows (k2_bispec84w)
   CUtensorMap tmx_ab{}, tmx_cd{};        // 2-D views [rows][Mp] (several channels, tensor cores)
   CUtensorMap tmx_sab{}, tmx_scd{};      // FP16X3: views of the bins' maxima [rows][Mp]
+  CUtensorMap tm_g32{}, tm_g64{};        // 2-D views of the F32 operand image (k3_trispec_gram)
   CUtensorMap tm_img[4]{};               // 4-D views of each channel's Gram operand image
   ss::TileInfo* d_tiles4tc = nullptr;  // tiles of the tensor-core S4 kernel (one channel)
   int4* d_c4cross = nullptr;       // (a, b, c, d) of each S4 combination (several channels)
   int n_tiles4tc = 0;
+  // FP32 S4 of one channel with m <= kGram32MaxM: the tiles of k3_trispec_gram
+  bool gram32 = false;
+  ss::TileInfo* d_tiles4g = nullptr;
+  int n_tiles4g = 0;
   ss::OperandImage oi;                 // K1's second output for the tensor-core S4 kernel
   int n_tiles3 = 0, n_tiles4 = 0;
   int2* d_pts3 = nullptr;  // isolated S3 grid points of one channel (k2_points)
