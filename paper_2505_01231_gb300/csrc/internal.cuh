@@ -52,10 +52,11 @@ struct SampleSource {
 // The centred spectra K1 writes: bin 0 of channel c's frame row r is at
 // rows + c * chan_stride + r * stride.  Mp bins from there on are written (zeros
 // past M - 1); with mirror, also the conjugates at the bins -(M - 1) .. -1 before.
+// Without store, nothing reads the spectra (S2 alone) and they need not be written.
 struct SpecRows {
   float2* rows;
   long long chan_stride;
-  int stride, mirror;
+  int stride, mirror, store;
 };
 
 // One channel combination of one order; channels as in the ABI records.
@@ -123,6 +124,35 @@ struct OperandImage {
 // the 96 KB budget (kK1Resident96); one frame at a time (kK1Frames); resident
 // groups with a warp per frame (kK1Warp, T <= 1024 and the group within 96 KB).
 enum { kK1Auto = 0, kK1Resident96 = 1, kK1Frames = 2, kK1Warp = 3, kK1Modes = 4 };
+
+// Radix of the next pass of K1's Stockham transform with `rem` still to go (N = T/2 is
+// a power of two).
+__host__ __device__ inline int fft_radix(int rem) {
+  return rem % 8 == 0 && rem != 16 ? 8 : rem % 4 == 0 ? 4 : 2;
+}
+// K1's twiddles, e^{+2 pi j a/T} at a = twiddle_angle(T, i) for entry i: first a = 0 ..
+// N/2 (the split into the real frame's coefficients), then per pass of radix R over
+// sub-transforms of length Ns > 1 the factors r k T/(Ns R), r = 1 .. R - 1, as R - 1
+// rows of Ns entries k, so that a warp's loads are consecutive.  (Indexed by r k T/(Ns R)
+// in one table of T entries, a warp's 7 loads of a radix-8 pass fell on one bank up to
+// 16 times: most of the passes' shared-memory time.)
+inline __host__ __device__ int twiddle_count(int T) { return (3 * T / 4 + 2) & ~1; }
+inline __host__ __device__ int twiddle_angle(int T, int i) {
+  const int N = T / 2;
+  if (i <= N / 2) return i;
+  int off = N / 2 + 1, Ns = 1;
+  for (int rem = N; rem > 1;) {
+    const int R = fft_radix(rem);
+    if (Ns > 1) {
+      const int cnt = (R - 1) * Ns;
+      if (i < off + cnt) return ((i - off) / Ns + 1) * ((i - off) % Ns) * (T / (Ns * R));
+      off += cnt;
+    }
+    Ns *= R;
+    rem /= R;
+  }
+  return 0;  // padding
+}
 
 // Kernel launchers (each returns the launch status; all work on `stream`).
 cudaError_t launch_k1_spectra(const SampleSource& src, long long sample0, int G, int C, int T,

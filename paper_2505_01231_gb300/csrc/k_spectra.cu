@@ -74,28 +74,32 @@ __device__ __forceinline__ void dft<8>(float2 (&v)[8]) {
   v[3] = cadd(e3, o3); v[7] = csub(e3, o3);
 }
 
+// Where point i of a frame lies in a shared-memory buffer or coefficient row: its place
+// within 16 points is XOR-ed with bits of i, so that the strided stores of the first
+// passes (8 points apart, then 8 within 64) fall on distinct banks like the consecutive
+// loads.  Blocks of 16 points stay in place.
+__device__ __forceinline__ int swz(int i) { return i ^ ((i >> 4) & 7) ^ ((i >> 3) & 8); }
+
 // One Stockham pass: sub-transforms of length Ns are combined R at a time into
-// length Ns*R.  x, y: N complex points in shared memory; tw[a] = e^{+2 pi j a/T}.
+// length Ns*R.  x, y: N complex points in shared memory; twp: the pass's twiddles
+// (twiddle_angle).
 template <int R>
 __device__ __forceinline__ void stockham_pass(const float2* __restrict__ x, float2* __restrict__ y,
-                                              int N, int Ns, const float2* __restrict__ tw,
-                                              int T) {
+                                              int N, int Ns, const float2* __restrict__ twp) {
   const int NR = N / R;
-  const int tw_scale = T / (Ns * R);
   for (int j = threadIdx.x; j < NR; j += blockDim.x) {
     const int k = j & (Ns - 1);
     float2 v[R];
 #pragma unroll
-    for (int r = 0; r < R; ++r) v[r] = x[j + r * NR];
+    for (int r = 0; r < R; ++r) v[r] = x[swz(j + r * NR)];
     if (Ns > 1) {
-      const int step = k * tw_scale;
 #pragma unroll
-      for (int r = 1; r < R; ++r) v[r] = cmul(v[r], __ldg(&tw[r * step]));
+      for (int r = 1; r < R; ++r) v[r] = cmul(v[r], __ldg(&twp[(r - 1) * Ns + k]));
     }
     dft<R>(v);
     const int base = (j - k) * R + k;
 #pragma unroll
-    for (int q = 0; q < R; ++q) y[base + q * Ns] = v[q];
+    for (int q = 0; q < R; ++q) y[swz(base + q * Ns)] = v[q];
   }
 }
 
@@ -103,6 +107,13 @@ __device__ __forceinline__ uint32_t to_tf32(float x) {
   uint32_t t;
   asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(t) : "f"(x));
   return t;
+}
+
+// e^{+2 pi j k/T} for k = 0 .. N = T/2 from the entries 0 .. N/2 (w^{N-k} = -conj w^k)
+template <class At>
+__device__ __forceinline__ float2 split_twiddle(At at, int k, int N) {
+  const float2 w = at(2 * k <= N ? k : N - k);
+  return 2 * k <= N ? w : make_float2(-w.x, w.y);
 }
 
 // Write one bin's row of one K chunk (16 entries) of the Gram operand image:
@@ -358,35 +369,37 @@ k1_spectra(SampleSource src, long long sample0, int G, int C, int T, int m, int 
         for (int n = threadIdx.x; n < N; n += blockDim.x) {
           const float x0 = load_sample<DTYPE>(src, c, s0 + 2 * n);
           const float x1 = load_sample<DTYPE>(src, c, s0 + 2 * n + 1);
-          bufA[n] = make_float2(x0 * __ldg(&win[2 * n]), x1 * __ldg(&win[2 * n + 1]));
+          bufA[swz(n)] = make_float2(x0 * __ldg(&win[2 * n]), x1 * __ldg(&win[2 * n + 1]));
         }
         __syncthreads();
         float2* x = bufA;
         float2* y = bufB;
         int Ns = 1;
         int rem = N;
+        const float2* twp = tw + N / 2 + 1;
         while (rem > 1) {
-          if (rem % 8 == 0 && rem != 16) {
-            stockham_pass<8>(x, y, N, Ns, tw, T);
-            Ns *= 8; rem /= 8;
-          } else if (rem % 4 == 0) {
-            stockham_pass<4>(x, y, N, Ns, tw, T);
-            Ns *= 4; rem /= 4;
-          } else {
-            stockham_pass<2>(x, y, N, Ns, tw, T);
-            Ns *= 2; rem /= 2;
-          }
+          const int R = fft_radix(rem);
+          if (R == 8)
+            stockham_pass<8>(x, y, N, Ns, twp);
+          else if (R == 4)
+            stockham_pass<4>(x, y, N, Ns, twp);
+          else
+            stockham_pass<2>(x, y, N, Ns, twp);
+          if (Ns > 1) twp += (R - 1) * Ns;
+          Ns *= R;
+          rem /= R;
           __syncthreads();
           float2* t = x; x = y; y = t;
         }
         // x holds Y_n; X_k = 1/2 [(Y_k + Y*_{N-k}) - j w^k (Y_k - Y*_{N-k})], w = e^{+2 pi j/T}
         float2* row = grow + (long long)j * sp.stride;
         for (int k = threadIdx.x; k < M; k += blockDim.x) {
-          const float2 yk = x[k == N ? 0 : k];
-          const float2 yr = x[k == 0 ? 0 : N - k];
+          const float2 yk = x[swz(k == N ? 0 : k)];
+          const float2 yr = x[swz(k == 0 ? 0 : N - k)];
           const float2 yc = make_float2(yr.x, -yr.y);
           const float2 s = cadd(yk, yc);
-          const float2 wd = cmul(__ldg(&tw[k]), csub(yk, yc));
+          const float2 wk = split_twiddle([&](int i) { return __ldg(&tw[i]); }, k, N);
+          const float2 wd = cmul(wk, csub(yk, yc));
           const float2 X = make_float2(0.5f * (s.x + wd.y), 0.5f * (s.y - wd.x));
           row[k] = X;
           gsum[k] = cadd(gsum[k], X);
@@ -417,16 +430,22 @@ k1_spectra(SampleSource src, long long sample0, int G, int C, int T, int m, int 
   if (ngroups) flush_k1_sums(C, M, s2_auto, acc2, n_s2, s2sum, s2sq, s1s, acc1);
 }
 
+// The points n, n + 1 (n even) of a row as one 16-byte store (they stay a pair under swz)
+__device__ __forceinline__ void put_pair(float2* row, int n, float4 v) {
+  const int p = swz(n);
+  if (p & 1) v = make_float4(v.z, v.w, v.x, v.y);
+  *reinterpret_cast<float4*>(row + (p & ~1)) = v;
+}
+
 // Stockham pass over a batch of FB frames of N points (frame f at x + f sx, its
 // output at y + f sy); all threads share the FB * N/R butterflies of the pass.
 template <int R>
 __device__ __forceinline__ void stockham_pass_batch(const float2* __restrict__ x,
                                                     float2* __restrict__ y, int N, int Ns,
-                                                    const float2* __restrict__ tw, int T, int FB,
+                                                    const float2* __restrict__ twp, int FB,
                                                     int sx, int sy) {
   const int NR = N / R;
   const int lg = __ffs(NR) - 1;  // NR is a power of two
-  const int tw_scale = T / (Ns * R);
   for (int idx = threadIdx.x; idx < FB * NR; idx += blockDim.x) {
     const int f = idx >> lg, j = idx & (NR - 1);
     const float2* xf = x + f * sx;
@@ -434,115 +453,125 @@ __device__ __forceinline__ void stockham_pass_batch(const float2* __restrict__ x
     const int k = j & (Ns - 1);
     float2 v[R];
 #pragma unroll
-    for (int r = 0; r < R; ++r) v[r] = xf[j + r * NR];
+    for (int r = 0; r < R; ++r) v[r] = xf[swz(j + r * NR)];
     if (Ns > 1) {
-      const int step = k * tw_scale;
 #pragma unroll
-      for (int r = 1; r < R; ++r) v[r] = cmul(v[r], tw[r * step]);
+      for (int r = 1; r < R; ++r) v[r] = cmul(v[r], twp[(r - 1) * Ns + k]);
     }
     dft<R>(v);
     const int base = (j - k) * R + k;
 #pragma unroll
-    for (int q = 0; q < R; ++q) yf[base + q * Ns] = v[q];
+    for (int q = 0; q < R; ++q) yf[swz(base + q * Ns)] = v[q];
   }
 }
 
-// K1, resident forms: with the group's m coefficient rows of channel c in shared
-// memory (Xs, [m][Mp]), thread = bin: subtract the bin's group mean (the centred
-// samples of the factorised k-statistics, App. H, Eq. 85), write the centred
-// column to the spectra once, add the per-group S2 estimate to the CTA's float32
-// sums and, with an operand image, write the bin's weighted Gram products and its
-// ps value.
+// K1: with bin k's m coefficients in shared memory (frame j's at col[j * cs], the
+// thread's own): subtract the bin's group mean (the centred samples of the factorised
+// k-statistics, App. H, Eq. 85), write the centred column to the spectra (with store),
+// and, with an operand image, the bin's weighted Gram products and its ps value.  Adds
+// the group's S1 (s1, if any) and returns sum_j |d_j|^2.
 template <int FMT>
-__device__ __forceinline__ void centre_resident(float2* Xs, float2* __restrict__ grow,
-                                                int row_stride, int mirror, int c, int g,
+__device__ __forceinline__ float centre_column(float2* col, int cs, float2* __restrict__ grow,
+                                               int row_stride, int mirror, int store, int k, int c,
+                                               int g, int m, int M, int Mp,
+                                               const OperandImage& oi, float* s1) {
+  const float inv_m = 1.0f / (float)m;
+  const bool valid = k < M;
+  float2 mean = make_float2(0.f, 0.f);
+  if (valid) {
+    for (int j = 0; j < m; ++j) mean = cadd(mean, col[j * cs]);
+    mean = make_float2(mean.x * inv_m, mean.y * inv_m);
+  }
+  if (k == 0 && s1) add_s1(s1, mean);
+  float p = 0.f, mx = 0.f;  // sum and max over j of |d_j|^2
+  for (int j = 0; j < m; ++j) {
+    const float2 d = valid ? csub(col[j * cs], mean) : make_float2(0.f, 0.f);
+    col[j * cs] = d;
+    if (store) put_coef(grow + (long long)j * row_stride, k, M, d, mirror);
+    const float pj = fmaf(d.x, d.x, d.y * d.y);
+    p += pj;
+    mx = fmaxf(mx, pj);
+  }
+  // several channels in FP16X3: the bin's row scale
+  if (oi.rmax) oi.rmax[(long long)c * oi.chan_rmax + (long long)g * Mp + k] = cross_row_scale(mx);
+  if (FMT == kImageGramF32 && k < oi.img_bins) {
+    // the bin's column of entry rows: pairs, ps, diagonal, zeros
+    float* e = static_cast<float*>(oi.img) + (size_t)g * oi.rows * Mp + k;
+    for (int j = 0; j < m; ++j) {
+      const float2 dj = col[j * cs];
+#pragma unroll 4
+      for (int q = j + 1; q < m; ++q) {
+        const float2 dq = col[q * cs];
+        *e = oi.so * fmaf(dj.x, dq.x, dj.y * dq.y);
+        e += Mp;
+      }
+    }
+    *e = oi.sp * p;
+    e += Mp;
+    for (int j = 0; j < m; ++j, e += Mp) {
+      const float2 dj = col[j * cs];
+      *e = oi.sd * fmaf(dj.x, dj.x, dj.y * dj.y);
+    }
+    for (int r = m * (m + 1) / 2 + 1; r < oi.rows; ++r, e += Mp) *e = 0.f;
+  } else if (FMT != kImageNone && k < oi.img_bins) {  // rows the tensor-core S4 reads
+    const float sc =
+        FMT == kImageGramF16 ? f16_row_scale(fmaxf(fmaxf(oi.sd, oi.so) * mx, oi.sp * p)) : 1.f;
+    const float sd = oi.sd * sc, so = oi.so * sc, sps = oi.sp * p * sc;
+    // weighted Gram products of the bin in K order, read from the centred column
+    const int npair = m * (m - 1) / 2;
+    int pj = 0, pk = 1;
+    float2 dj = col[0];
+    constexpr int kChunkBytes = FMT == kImageGramTF32 ? 1024 : 512;  // 2 CB
+    unsigned char* rbase = static_cast<unsigned char*>(oi.img) + (size_t)c * oi.chan_bytes +
+                           (size_t)g * oi.group_bytes + (size_t)(k >> 3) * oi.rg_bytes +
+                           (k & 7) * 16;
+    for (int ch = 0; ch < oi.nkc; ++ch) {
+      float e[16];
+      if (ch < oi.ndc) {
+#pragma unroll
+        for (int t = 0; t < 16; ++t) {
+          const int j = ch * 16 + t;
+          const float2 d = j < m ? col[j * cs] : make_float2(0.f, 0.f);
+          e[t] = sd * fmaf(d.x, d.x, d.y * d.y);
+        }
+      } else {
+        const int p0 = (ch - oi.ndc) * 16;
+#pragma unroll
+        for (int t = 0; t < 16; ++t) {
+          if (p0 + t < npair) {
+            const float2 d2 = col[pk * cs];
+            e[t] = so * fmaf(dj.x, d2.x, dj.y * d2.y);
+            if (++pk == m) {
+              ++pj;
+              pk = pj + 1;
+              dj = col[pj * cs];
+            }
+          } else {
+            e[t] = p0 + t == npair ? sps : 0.f;  // ps after the pairs (negated with them)
+          }
+        }
+      }
+      write_gram_row<FMT>(rbase + ch * kChunkBytes, e);
+    }
+    if (FMT == kImageGramF16)  // exact: a power of two
+      oi.rsc[(long long)c * oi.chan_rsc + (long long)g * Mp + k] = 1.f / sc;
+  }
+  return p;
+}
+
+// K1, resident forms: the group's m coefficient rows of channel c in shared memory (Xs,
+// [m][Mp], swizzled within 16), thread = bin; adds the per-group S2 estimate to the
+// CTA's float32 sums.
+template <int FMT>
+__device__ __forceinline__ void centre_resident(float2* Xs, const SpecRows& sp, int c, int g,
                                                 int m, int M, int Mp, const OperandImage& oi,
                                                 int ia, float* s2sum, float* s2sq, float* s1,
                                                 float pref2) {
-  const float inv_m = 1.0f / (float)m;
+  float2* grow = sp.rows + (long long)c * sp.chan_stride + (long long)g * m * sp.stride;
   for (int k = threadIdx.x; k < Mp; k += blockDim.x) {
-    // thread = bin: centre the column in place, write it out once
-    const bool valid = k < M;
-    float2 mean = make_float2(0.f, 0.f);
-    if (valid) {
-      for (int j = 0; j < m; ++j) mean = cadd(mean, Xs[j * Mp + k]);
-      mean = make_float2(mean.x * inv_m, mean.y * inv_m);
-    }
-    if (k == 0) add_s1(s1, mean);
-    float p = 0.f, mx = 0.f;  // sum and max over j of |d_j|^2
-    for (int j = 0; j < m; ++j) {
-      const float2 d = valid ? csub(Xs[j * Mp + k], mean) : make_float2(0.f, 0.f);
-      Xs[j * Mp + k] = d;
-      put_coef(grow + (long long)j * row_stride, k, M, d, mirror);
-      const float pj = fmaf(d.x, d.x, d.y * d.y);
-      p += pj;
-      mx = fmaxf(mx, pj);
-    }
-    // several channels in FP16X3: the bin's row scale
-    if (oi.rmax) oi.rmax[(long long)c * oi.chan_rmax + (long long)g * Mp + k] = cross_row_scale(mx);
-    if (FMT == kImageGramF32 && k < oi.img_bins) {
-      // the bin's column of entry rows: pairs, ps, diagonal, zeros
-      float* e = static_cast<float*>(oi.img) + (size_t)g * oi.rows * Mp + k;
-      for (int j = 0; j < m; ++j) {
-        const float2 dj = Xs[j * Mp + k];
-#pragma unroll 4
-        for (int q = j + 1; q < m; ++q) {
-          const float2 dq = Xs[q * Mp + k];
-          *e = oi.so * fmaf(dj.x, dq.x, dj.y * dq.y);
-          e += Mp;
-        }
-      }
-      *e = oi.sp * p;
-      e += Mp;
-      for (int j = 0; j < m; ++j, e += Mp) {
-        const float2 dj = Xs[j * Mp + k];
-        *e = oi.sd * fmaf(dj.x, dj.x, dj.y * dj.y);
-      }
-      for (int r = m * (m + 1) / 2 + 1; r < oi.rows; ++r, e += Mp) *e = 0.f;
-    } else if (FMT != kImageNone && k < oi.img_bins) {  // rows the tensor-core S4 reads
-      const float sc =
-        FMT == kImageGramF16 ? f16_row_scale(fmaxf(fmaxf(oi.sd, oi.so) * mx, oi.sp * p)) : 1.f;
-      const float sd = oi.sd * sc, so = oi.so * sc, sps = oi.sp * p * sc;
-      // weighted Gram products of the bin in K order, read from the centred column
-      const int npair = m * (m - 1) / 2;
-      int pj = 0, pk = 1;
-      float2 dj = Xs[k];
-      constexpr int kChunkBytes = FMT == kImageGramTF32 ? 1024 : 512;  // 2 CB
-      unsigned char* rbase = static_cast<unsigned char*>(oi.img) + (size_t)c * oi.chan_bytes +
-                             (size_t)g * oi.group_bytes + (size_t)(k >> 3) * oi.rg_bytes +
-                             (k & 7) * 16;
-      for (int ch = 0; ch < oi.nkc; ++ch) {
-        float e[16];
-        if (ch < oi.ndc) {
-#pragma unroll
-          for (int t = 0; t < 16; ++t) {
-            const int j = ch * 16 + t;
-            const float2 d = j < m ? Xs[j * Mp + k] : make_float2(0.f, 0.f);
-            e[t] = sd * fmaf(d.x, d.x, d.y * d.y);
-          }
-        } else {
-          const int p0 = (ch - oi.ndc) * 16;
-#pragma unroll
-          for (int t = 0; t < 16; ++t) {
-            if (p0 + t < npair) {
-              const float2 d2 = Xs[pk * Mp + k];
-              e[t] = so * fmaf(dj.x, d2.x, dj.y * d2.y);
-              if (++pk == m) {
-                ++pj;
-                pk = pj + 1;
-                dj = Xs[pj * Mp + k];
-              }
-            } else {
-              e[t] = p0 + t == npair ? sps : 0.f;  // ps after the pairs (negated with them)
-            }
-          }
-        }
-        write_gram_row<FMT>(rbase + ch * kChunkBytes, e);
-      }
-      if (FMT == kImageGramF16)  // exact: a power of two
-        oi.rsc[(long long)c * oi.chan_rsc + (long long)g * Mp + k] = 1.f / sc;
-    }
-    if (valid && ia >= 0) {
+    const float p = centre_column<FMT>(Xs + swz(k), Mp, grow, sp.stride, sp.mirror, sp.store, k, c,
+                                       g, m, M, Mp, oi, s1);
+    if (k < M && ia >= 0) {
       const float c2 = p * pref2;
       s2sum[c * M + k] += c2;
       s2sq[c * M + k] = fmaf(c2, c2, s2sq[c * M + k]);
@@ -571,8 +600,8 @@ k1_spectra_res(SampleSource src, long long sample0, int G, int C, int T, int m, 
   const int N = T / 2;
   float2* buf = reinterpret_cast<float2*>(smem_raw);  // [FB][N]
   float2* Xs = buf + FB * N;                          // [m][Mp]
-  float2* tws = Xs + m * Mp;                           // [T] twiddles e^{+2 pi j a/T}
-  float* wins = reinterpret_cast<float*>(tws + T);     // [T] window / sqrt(sum g^2)
+  float2* tws = Xs + m * Mp;                           // [twiddle_count(T)] twiddles
+  float* wins = reinterpret_cast<float*>(tws + twiddle_count(T));  // [T] window / sqrt(sum g^2)
   float* s2sum = wins + T;                             // [C][M]
   float* s2sq = s2sum + C * M;                         // [C][M]
   constexpr int kVec = DTYPE == SS_F32 ? 16 : 8;        // bytes per vector load (4 samples)
@@ -581,7 +610,7 @@ k1_spectra_res(SampleSource src, long long sample0, int G, int C, int T, int m, 
   for (int i = threadIdx.x; i < 2 * C * M; i += blockDim.x) s2sum[i] = 0.f;
   if (threadIdx.x < 16) s1s[threadIdx.x >> 2][threadIdx.x & 3] = 0.f;
   for (int i = threadIdx.x; i < T; i += blockDim.x) {
-    tws[i] = __ldg(&tw[i]);
+    if (i < twiddle_count(T)) tws[i] = __ldg(&tw[i]);
     wins[i] = __ldg(&win[i]);
   }
 
@@ -609,7 +638,6 @@ k1_spectra_res(SampleSource src, long long sample0, int G, int C, int T, int m, 
   int ngroups = 0;  // groups in the float32 sums since the last flush
   for (int g = blockIdx.x; g < G; g += gridDim.x) {
     for (int c = 0; c < C; ++c) {
-      float2* grow = sp.rows + (long long)c * sp.chan_stride + (long long)g * m * sp.stride;
       for (int j0 = 0; j0 < m; j0 += FB) {
         const int nf = min(FB, m - j0);
         const long long s0 = sample0 + ((long long)g * m + j0) * T;  // first sample of the batch
@@ -624,9 +652,8 @@ k1_spectra_res(SampleSource src, long long sample0, int G, int C, int T, int m, 
             if (q < nf * T / 4) {
               const int i = (4 * q) & (T - 1), f = (4 * q) / T;
               const float4 w = *reinterpret_cast<const float4*>(wins + i);
-              float2* d = Xs + (j0 + f) * Mp + i / 2;
-              d[0] = make_float2(pre[r].x * w.x, pre[r].y * w.y);
-              d[1] = make_float2(pre[r].z * w.z, pre[r].w * w.w);
+              put_pair(Xs + (j0 + f) * Mp, i / 2,
+                       make_float4(pre[r].x * w.x, pre[r].y * w.y, pre[r].z * w.z, pre[r].w * w.w));
             }
           }
         } else if (off >= 0 && ((uintptr_t)cbase % kVec) == 0) {
@@ -641,15 +668,14 @@ k1_spectra_res(SampleSource src, long long sample0, int G, int C, int T, int m, 
               x0 = v.x; x1 = v.y; x2 = v.z; x3 = v.w;
             }
             const float4 w = *reinterpret_cast<const float4*>(wins + i);
-            float2* d = Xs + (j0 + f) * Mp + i / 2;
-            d[0] = make_float2(x0 * w.x, x1 * w.y);
-            d[1] = make_float2(x2 * w.z, x3 * w.w);
+            put_pair(Xs + (j0 + f) * Mp, i / 2,
+                     make_float4(x0 * w.x, x1 * w.y, x2 * w.z, x3 * w.w));
           }
         } else {
           for (int q = threadIdx.x; q < nf * N; q += blockDim.x) {
             const int f = q / N, n = q - f * N;
             const long long si = s0 + (long long)f * T + 2 * n;
-            Xs[(j0 + f) * Mp + n] = make_float2(load_sample<DTYPE>(src, c, si) * wins[2 * n],
+            Xs[(j0 + f) * Mp + swz(n)] = make_float2(load_sample<DTYPE>(src, c, si) * wins[2 * n],
                                                 load_sample<DTYPE>(src, c, si + 1) * wins[2 * n + 1]);
           }
         }
@@ -671,17 +697,18 @@ k1_spectra_res(SampleSource src, long long sample0, int G, int C, int T, int m, 
         int sx = Mp, sy = N;
         int Ns = 1;
         int rem = N;
+        const float2* twp = tws + N / 2 + 1;
         while (rem > 1) {
-          if (rem % 8 == 0 && rem != 16) {
-            stockham_pass_batch<8>(x, y, N, Ns, tws, T, nf, sx, sy);
-            Ns *= 8; rem /= 8;
-          } else if (rem % 4 == 0) {
-            stockham_pass_batch<4>(x, y, N, Ns, tws, T, nf, sx, sy);
-            Ns *= 4; rem /= 4;
-          } else {
-            stockham_pass_batch<2>(x, y, N, Ns, tws, T, nf, sx, sy);
-            Ns *= 2; rem /= 2;
-          }
+          const int R = fft_radix(rem);
+          if (R == 8)
+            stockham_pass_batch<8>(x, y, N, Ns, twp, nf, sx, sy);
+          else if (R == 4)
+            stockham_pass_batch<4>(x, y, N, Ns, twp, nf, sx, sy);
+          else
+            stockham_pass_batch<2>(x, y, N, Ns, twp, nf, sx, sy);
+          if (Ns > 1) twp += (R - 1) * Ns;
+          Ns *= R;
+          rem /= R;
           __syncthreads();
           float2* t = x; x = y; y = t;
           const int ts = sx; sx = sy; sy = ts;
@@ -692,7 +719,7 @@ k1_spectra_res(SampleSource src, long long sample0, int G, int C, int T, int m, 
         auto split = [&](float2 yk, float2 yr, int k) {
           const float2 yc = make_float2(yr.x, -yr.y);
           const float2 sm = cadd(yk, yc);
-          const float2 wd = cmul(tws[k], csub(yk, yc));
+          const float2 wd = cmul(split_twiddle([&](int i) { return tws[i]; }, k, N), csub(yk, yc));
           return make_float2(0.5f * (sm.x + wd.y), 0.5f * (sm.y - wd.x));
         };
         const int NH = N / 2 + 1;  // pairs per frame
@@ -700,13 +727,13 @@ k1_spectra_res(SampleSource src, long long sample0, int G, int C, int T, int m, 
           const int f = idx / NH, k = idx - f * NH;
           const float2* xf = x + f * sx;
           float2* xr = rows + f * Mp;
-          const float2 a = xf[k], b = xf[k == 0 ? 0 : N - k];
-          xr[k] = split(a, b, k);
-          xr[N - k] = split(b, a, N - k);
+          const float2 a = xf[swz(k)], b = xf[swz(k == 0 ? 0 : N - k)];
+          xr[swz(k)] = split(a, b, k);
+          xr[swz(N - k)] = split(b, a, N - k);
         }
       }
       __syncthreads();  // the group's coefficients are in shared memory
-      centre_resident<FMT>(Xs, grow, sp.stride, sp.mirror, c, g, m, M, Mp, oi, s2_auto[c], s2sum, s2sq, s1s[c], pref2);
+      centre_resident<FMT>(Xs, sp, c, g, m, M, Mp, oi, s2_auto[c], s2sum, s2sq, s1s[c], pref2);
     }
     if (++ngroups == kMaxFp32Groups) {
       flush_k1_sums(C, M, s2_auto, acc2, n_s2, s2sum, s2sq, s1s, acc1);
@@ -722,17 +749,16 @@ k1_spectra_res(SampleSource src, long long sample0, int G, int C, int T, int m, 
 // N / R <= 32 * (16 / R), i.e. N <= 512: at most 16 points per lane.
 template <int R>
 __device__ __forceinline__ void warp_stockham_pass(float2* buf, int N, int Ns,
-                                                   const float2* __restrict__ tw, int T, int lane) {
+                                                   const float2* __restrict__ twp, int lane) {
   constexpr int kB = 16 / R;  // butterflies per lane
   const int NR = N / R;
-  const int tw_scale = T / (Ns * R);
   float2 v[kB][R];
 #pragma unroll
   for (int b = 0; b < kB; ++b) {
     const int j = lane + 32 * b;
     if (j < NR) {
 #pragma unroll
-      for (int r = 0; r < R; ++r) v[b][r] = buf[j + r * NR];
+      for (int r = 0; r < R; ++r) v[b][r] = buf[swz(j + r * NR)];
     }
   }
   __syncwarp();
@@ -742,14 +768,13 @@ __device__ __forceinline__ void warp_stockham_pass(float2* buf, int N, int Ns,
     if (j < NR) {
       const int k = j & (Ns - 1);
       if (Ns > 1) {
-        const int step = k * tw_scale;
 #pragma unroll
-        for (int r = 1; r < R; ++r) v[b][r] = cmul(v[b][r], tw[r * step]);
+        for (int r = 1; r < R; ++r) v[b][r] = cmul(v[b][r], twp[(r - 1) * Ns + k]);
       }
       dft<R>(v[b]);
       const int base = (j - k) * R + k;
 #pragma unroll
-      for (int q = 0; q < R; ++q) buf[base + q * Ns] = v[b][q];
+      for (int q = 0; q < R; ++q) buf[swz(base + q * Ns)] = v[b][q];
     }
   }
   __syncwarp();
@@ -772,8 +797,8 @@ k1_spectra_warp(SampleSource src, long long sample0, int G, int C, int T, int m,
   constexpr int kWarps = kThreadsK1 / 32;
   float2* Xs = reinterpret_cast<float2*>(smem_raw);  // [m][Mp]
   float2* bufs = Xs + m * Mp;                         // [kWarps][N]
-  float2* tws = bufs + kWarps * N;                    // [T] twiddles e^{+2 pi j a/T}
-  float* wins = reinterpret_cast<float*>(tws + T);   // [T] window / sqrt(sum g^2)
+  float2* tws = bufs + kWarps * N;                    // [twiddle_count(T)] twiddles
+  float* wins = reinterpret_cast<float*>(tws + twiddle_count(T));  // [T] window / sqrt(sum g^2)
   float* s2sum = wins + T;                            // [C][M]
   float* s2sq = s2sum + C * M;                        // [C][M]
   float2* buf = bufs + warp * N;
@@ -783,7 +808,7 @@ k1_spectra_warp(SampleSource src, long long sample0, int G, int C, int T, int m,
   for (int i = threadIdx.x; i < 2 * C * M; i += blockDim.x) s2sum[i] = 0.f;
   if (threadIdx.x < 16) s1s[threadIdx.x >> 2][threadIdx.x & 3] = 0.f;
   for (int i = threadIdx.x; i < T; i += blockDim.x) {
-    tws[i] = __ldg(&tw[i]);
+    if (i < twiddle_count(T)) tws[i] = __ldg(&tw[i]);
     wins[i] = __ldg(&win[i]);
   }
   __syncthreads();
@@ -791,7 +816,6 @@ k1_spectra_warp(SampleSource src, long long sample0, int G, int C, int T, int m,
   int ngroups = 0;  // groups in the float32 sums since the last flush
   for (int g = blockIdx.x; g < G; g += gridDim.x) {
     for (int c = 0; c < C; ++c) {
-      float2* grow = sp.rows + (long long)c * sp.chan_stride + (long long)g * m * sp.stride;
       for (int j = warp; j < m; j += kWarps) {
         // the frame's samples times the window, packed as N complex points
         const long long s0 = sample0 + ((long long)g * m + j) * T;
@@ -809,42 +833,42 @@ k1_spectra_warp(SampleSource src, long long sample0, int G, int C, int T, int m,
               x0 = v.x; x1 = v.y; x2 = v.z; x3 = v.w;
             }
             const float4 w = *reinterpret_cast<const float4*>(wins + 4 * q);
-            buf[2 * q] = make_float2(x0 * w.x, x1 * w.y);
-            buf[2 * q + 1] = make_float2(x2 * w.z, x3 * w.w);
+            put_pair(buf, 2 * q, make_float4(x0 * w.x, x1 * w.y, x2 * w.z, x3 * w.w));
           }
         } else {
           for (int n = lane; n < N; n += 32)
-            buf[n] = make_float2(load_sample<DTYPE>(src, c, s0 + 2 * n) * wins[2 * n],
+            buf[swz(n)] = make_float2(load_sample<DTYPE>(src, c, s0 + 2 * n) * wins[2 * n],
                                  load_sample<DTYPE>(src, c, s0 + 2 * n + 1) * wins[2 * n + 1]);
         }
         __syncwarp();
         int Ns = 1, rem = N;
+        const float2* twp = tws + N / 2 + 1;
         while (rem > 1) {
-          if (rem % 8 == 0 && rem != 16) {
-            warp_stockham_pass<8>(buf, N, Ns, tws, T, lane);
-            Ns *= 8; rem /= 8;
-          } else if (rem % 4 == 0) {
-            warp_stockham_pass<4>(buf, N, Ns, tws, T, lane);
-            Ns *= 4; rem /= 4;
-          } else {
-            warp_stockham_pass<2>(buf, N, Ns, tws, T, lane);
-            Ns *= 2; rem /= 2;
-          }
+          const int R = fft_radix(rem);
+          if (R == 8)
+            warp_stockham_pass<8>(buf, N, Ns, twp, lane);
+          else if (R == 4)
+            warp_stockham_pass<4>(buf, N, Ns, twp, lane);
+          else
+            warp_stockham_pass<2>(buf, N, Ns, twp, lane);
+          if (Ns > 1) twp += (R - 1) * Ns;
+          Ns *= R;
+          rem /= R;
         }
         // X_k = 1/2 [(Y_k + Y*_{N-k}) - j w^k (Y_k - Y*_{N-k})], w = e^{+2 pi j/T}
         float2* xr = Xs + j * Mp;
         for (int k = lane; k < M; k += 32) {
-          const float2 yk = buf[k == N ? 0 : k];
-          const float2 yr = buf[k == 0 ? 0 : N - k];
+          const float2 yk = buf[swz(k == N ? 0 : k)];
+          const float2 yr = buf[swz(k == 0 ? 0 : N - k)];
           const float2 yc = make_float2(yr.x, -yr.y);
           const float2 sm = cadd(yk, yc);
-          const float2 wd = cmul(tws[k], csub(yk, yc));
-          xr[k] = make_float2(0.5f * (sm.x + wd.y), 0.5f * (sm.y - wd.x));
+          const float2 wd = cmul(split_twiddle([&](int i) { return tws[i]; }, k, N), csub(yk, yc));
+          xr[swz(k)] = make_float2(0.5f * (sm.x + wd.y), 0.5f * (sm.y - wd.x));
         }
         __syncwarp();  // the buffer is free for the warp's next frame
       }
       __syncthreads();  // the group's coefficients are in shared memory
-      centre_resident<FMT>(Xs, grow, sp.stride, sp.mirror, c, g, m, M, Mp, oi, s2_auto[c], s2sum, s2sq, s1s[c], pref2);
+      centre_resident<FMT>(Xs, sp, c, g, m, M, Mp, oi, s2_auto[c], s2sum, s2sq, s1s[c], pref2);
       __syncthreads();  // Xs is free for the next channel or group
     }
     if (++ngroups == kMaxFp32Groups) {
@@ -853,6 +877,323 @@ k1_spectra_warp(SampleSource src, long long sample0, int G, int C, int T, int m,
     }
   }
   if (ngroups) flush_k1_sums(C, M, s2_auto, acc2, n_s2, s2sum, s2sq, s1s, acc1);
+}
+
+// ---------------------------------------------------------------------------
+// K1 for long frames (T >= 1024) whose groups do not fit in shared memory, and for
+// power spectra alone.  A 256-thread CTA transforms batches of 2048 complex points
+// (FB = 2048 / N consecutive frames of N = T/2 points), one radix-8 butterfly a thread in
+// the first pass, whose inputs come straight from global memory (two samples each,
+// windowed from shared memory, the next batch's loaded before the current one's passes); the
+// other passes go through two swizzled shared-memory buffers, with one barrier each.
+//
+// kPower: a CTA takes whole groups; thread t owns the bins k = t + 256 s and N - k and
+// keeps each bin's running mean and sum of squared deviations over the group's frames
+// (Welford's update) in registers, so nothing but the sums leaves the SM.  Else
+// the coefficients are written to the spectra as they are, and k1_centre does the rest.
+//
+// HBM bounds the power form in the end (4 bytes a sample in, nothing out); now it is shared
+// memory (LSU 68 %) and issue (68 %).  Measured, S2 alone, T = 2048, m = 16, 2^27 samples:
+// 1.11 ms frame by frame with the spectra written, read, centred and written again, now
+// 0.257 ms (2.07 TB/s); T = 1024, m = 8, 2^26: 0.123 ms; T = 4096, m = 8, 2^26: 0.144 ms.
+// In two kernels, T = 4096, m = 10, int16, 2^24 samples with the FP16 image: 0.246 ms ->
+// 0.117 ms (0.044 transform, 0.069 centring); T = 2048, m = 9, 5e6: 0.095 -> 0.042 ms.
+constexpr int kFftPoints = 2048;
+
+// one pass of radix R over sub-transforms of length NS, compile-time sizes
+template <int R, int NS, int N>
+__device__ __forceinline__ void fixed_pass(const float2* __restrict__ x, float2* __restrict__ y,
+                                           const float2* __restrict__ twp) {
+  constexpr int NR = N / R;
+#pragma unroll
+  for (int i = 0; i < kFftPoints / R / kThreadsK1; ++i) {
+    const int idx = threadIdx.x + i * kThreadsK1;
+    const int f = idx / NR, j = idx % NR, k = j % NS;
+    const float2* xf = x + f * N;
+    float2* yf = y + f * N;
+    float2 v[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) v[r] = xf[swz(j + r * NR)];
+#pragma unroll
+    for (int r = 1; r < R; ++r) v[r] = cmul(v[r], twp[(r - 1) * NS + k]);
+    dft<R>(v);
+    const int base = (j - k) * R + k;
+#pragma unroll
+    for (int q = 0; q < R; ++q) yf[swz(base + q * NS)] = v[q];
+  }
+}
+
+// One bin over a group's frames: running mean and sum of squared deviations.
+struct Welford {
+  float2 mean;
+  float m2;
+  __device__ __forceinline__ void clear() {
+    mean = make_float2(0.f, 0.f);
+    m2 = 0.f;
+  }
+  __device__ __forceinline__ void add(float2 x, float inv_n) {
+    const float2 d = csub(x, mean);
+    mean = make_float2(fmaf(d.x, inv_n, mean.x), fmaf(d.y, inv_n, mean.y));
+    const float2 e = csub(x, mean);
+    m2 = fmaf(d.x, e.x, fmaf(d.y, e.y, m2));
+  }
+};
+
+template <int DTYPE, int N, bool kPower>
+__global__ void __launch_bounds__(kThreadsK1, kPower && N == 2048 ? 2 : 3)  // registers
+k1_fft(SampleSource src, long long sample0, int G, int m, const float* __restrict__ win,
+       const float2* __restrict__ tw, SpecRows sp, const int* __restrict__ s2_auto,
+       double* __restrict__ acc2, int n_s2, float pref2, double* __restrict__ acc1, int C) {
+  constexpr int T = 2 * N, M = N + 1, FB = kFftPoints / N, NR = N / 8;
+  constexpr int kSlots = N / 2 / kThreadsK1;  // bin pairs (k, N - k) of a thread
+  extern __shared__ float4 smem_raw[];
+  float2* bufA = reinterpret_cast<float2*>(smem_raw);
+  float2* bufB = bufA + kFftPoints;
+  float2* tws = bufB + kFftPoints;          // [twiddle_count(T)]
+  float2* wins = tws + twiddle_count(T);     // [N] pairs of the window
+  const int tid = threadIdx.x;
+  const int c = blockIdx.y;
+  for (int i = tid; i < twiddle_count(T); i += kThreadsK1) tws[i] = __ldg(&tw[i]);
+  for (int i = tid; i < N; i += kThreadsK1)
+    wins[i] = __ldg(reinterpret_cast<const float2*>(win) + i);
+  const int pf = tid / NR, pj = tid % NR;  // frame and butterfly of the first pass
+
+  // samples 2 (pj + r NR), + 1 of frame f0 + pf (of nf frames from f0 on)
+  auto load = [&](long long f0, int nf, float2 (&v)[8]) {
+    const long long s0 = sample0 + (f0 + pf) * T + 2 * pj;
+    const long long off = s0 - src.carry_n;
+    constexpr int kVec = DTYPE == SS_F32 ? 8 : 4;  // bytes of two samples
+    const char* p = static_cast<const char*>(src.chunk) +
+                    ((long long)c * src.chunk_stride + off) * (DTYPE == SS_F32 ? 4 : 2);
+    if (pf >= nf) {
+#pragma unroll
+      for (int r = 0; r < 8; ++r) v[r] = make_float2(0.f, 0.f);
+    } else if (off >= 0 && (uintptr_t)p % kVec == 0) {
+#pragma unroll
+      for (int r = 0; r < 8; ++r) {
+        if constexpr (DTYPE == SS_F32) {
+          v[r] = __ldg(reinterpret_cast<const float2*>(p) + r * NR);
+        } else {
+          const short2 q = __ldg(reinterpret_cast<const short2*>(p) + r * NR);
+          v[r] = make_float2((float)q.x, (float)q.y);
+        }
+      }
+    } else {
+#pragma unroll
+      for (int r = 0; r < 8; ++r)
+        v[r] = make_float2(load_sample<DTYPE>(src, c, s0 + 2 * r * NR),
+                           load_sample<DTYPE>(src, c, s0 + 2 * r * NR + 1));
+    }
+  };
+  // the batch's transforms from v; the result is in the returned buffer after a barrier
+  auto transform = [&](float2 (&v)[8]) -> const float2* {
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+      const float2 w = wins[pj + r * NR];
+      v[r] = make_float2(v[r].x * w.x, v[r].y * w.y);
+    }
+    dft<8>(v);
+#pragma unroll
+    for (int q = 0; q < 8; ++q) bufA[pf * N + swz(8 * pj + q)] = v[q];
+    __syncthreads();
+    const float2* t2 = tws + N / 2 + 1;  // NS = 8
+    fixed_pass<8, 8, N>(bufA, bufB, t2);
+    __syncthreads();
+    const float2* t3 = t2 + 7 * 8;  // NS = 64
+    if constexpr (N == 512) {
+      fixed_pass<8, 64, N>(bufB, bufA, t3);
+      __syncthreads();
+      return bufA;
+    } else if constexpr (N == 1024) {
+      fixed_pass<4, 64, N>(bufB, bufA, t3);
+      __syncthreads();
+      fixed_pass<4, 256, N>(bufA, bufB, t3 + 3 * 64);
+      __syncthreads();
+      return bufB;
+    } else {
+      fixed_pass<8, 64, N>(bufB, bufA, t3);
+      __syncthreads();
+      fixed_pass<4, 512, N>(bufA, bufB, t3 + 7 * 64);
+      __syncthreads();
+      return bufB;
+    }
+  };
+  // X_k of Y_k and Y_{N-k} (see k1_spectra_res)
+  auto split = [&](float2 yk, float2 yr, float2 wk) {
+    const float2 yc = make_float2(yr.x, -yr.y);
+    const float2 sm = cadd(yk, yc);
+    const float2 wd = cmul(wk, csub(yk, yc));
+    return make_float2(0.5f * (sm.x + wd.y), 0.5f * (sm.y - wd.x));
+  };
+  // The buffer the result lies in is written again no earlier than after the next
+  // batch's first barrier (N = 512: its first pass writes the result's buffer, so the
+  // split ends with a barrier of its own).
+  float2 pre[8];
+  if constexpr (!kPower) {
+    const long long frames = (long long)G * m, nb = (frames + FB - 1) / FB;
+    float2* base = sp.rows + (long long)c * sp.chan_stride;
+    long long b = blockIdx.x;
+    if (b < nb) load(b * FB, (int)min((long long)FB, frames - b * FB), pre);
+    for (; b < nb; b += gridDim.x) {
+      const int nf = (int)min((long long)FB, frames - b * FB);
+      float2 v[8];
+#pragma unroll
+      for (int r = 0; r < 8; ++r) v[r] = pre[r];
+      const long long bn = b + gridDim.x;
+      if (bn < nb) load(bn * FB, (int)min((long long)FB, frames - bn * FB), pre);
+      if (b == blockIdx.x) __syncthreads();  // the twiddles are in shared memory
+      const float2* Y = transform(v);
+#pragma unroll
+      for (int f = 0; f < FB; ++f) {
+        if (f < nf) {
+          const float2* y = Y + f * N;
+          float2* row = base + (b * FB + f) * (long long)sp.stride;
+#pragma unroll
+          for (int s = 0; s < kSlots; ++s) {
+            const int k = tid + s * kThreadsK1;
+            const float2 a = y[swz(k)], bb = y[swz(k == 0 ? 0 : N - k)];
+            const float2 wk = tws[k];
+            row[k] = split(a, bb, wk);
+            row[N - k] = split(bb, a, make_float2(-wk.x, wk.y));
+          }
+          if (tid == 0) {
+            const float2 a = y[swz(N / 2)];
+            row[N / 2] = split(a, a, tws[N / 2]);
+          }
+        }
+      }
+      if (N == 512) __syncthreads();
+    }
+  } else {
+    const int ia = s2_auto[c];
+    Welford lo[kSlots], hi[kSlots], mid;
+    float sum[2 * kSlots + 1], sq[2 * kSlots + 1];  // c2 and its square over the groups
+    float s1[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int i = 0; i < 2 * kSlots + 1; ++i) sum[i] = sq[i] = 0.f;
+    auto flush = [&]() {
+      const long long plane = (long long)n_s2 * M;
+      auto put = [&](int k, float a, float b) {
+        if (ia < 0) return;
+        atomicAdd(acc2 + (long long)ia * M + k, (double)a);
+        atomicAdd(acc2 + 2 * plane + (long long)ia * M + k, (double)b);
+      };
+#pragma unroll
+      for (int s = 0; s < kSlots; ++s) {
+        const int k = tid + s * kThreadsK1;
+        put(k, sum[2 * s], sq[2 * s]);
+        put(N - k, sum[2 * s + 1], sq[2 * s + 1]);
+      }
+      if (tid == 0) {
+        put(N / 2, sum[2 * kSlots], sq[2 * kSlots]);
+        for (int q = 0; q < 4; ++q) {
+          if (acc1) atomicAdd(acc1 + q * C + c, (double)s1[q]);
+          s1[q] = 0.f;
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < 2 * kSlots + 1; ++i) sum[i] = sq[i] = 0.f;
+    };
+    int g = blockIdx.x, ngroups = 0;
+    if (g < G) load((long long)g * m, min(FB, m), pre);
+    for (; g < G; g += gridDim.x) {
+#pragma unroll
+      for (int s = 0; s < kSlots; ++s) {
+        lo[s].clear();
+        hi[s].clear();
+      }
+      mid.clear();
+      for (int j0 = 0; j0 < m; j0 += FB) {
+        const int nf = min(FB, m - j0);
+        float2 v[8];
+#pragma unroll
+        for (int r = 0; r < 8; ++r) v[r] = pre[r];
+        // the next batch: this group's next frames or the CTA's next group's first
+        const bool more = j0 + FB < m;
+        const long long gn = more ? g : (long long)g + gridDim.x;
+        const int jn = more ? j0 + FB : 0;
+        if (gn < G) load(gn * m + jn, min(FB, m - jn), pre);
+        if (g == (int)blockIdx.x && j0 == 0) __syncthreads();  // the twiddles are there
+        const float2* Y = transform(v);
+#pragma unroll
+        for (int f = 0; f < FB; ++f) {
+          if (f < nf) {
+            const float2* y = Y + f * N;
+            const float inv = 1.0f / (float)(j0 + f + 1);
+#pragma unroll
+            for (int s = 0; s < kSlots; ++s) {
+              const int k = tid + s * kThreadsK1;
+              const float2 a = y[swz(k)], bb = y[swz(k == 0 ? 0 : N - k)];
+              const float2 wk = tws[k];
+              lo[s].add(split(a, bb, wk), inv);
+              hi[s].add(split(bb, a, make_float2(-wk.x, wk.y)), inv);
+            }
+            if (tid == 0) {
+              const float2 a = y[swz(N / 2)];
+              mid.add(split(a, a, tws[N / 2]), inv);
+            }
+          }
+        }
+        if (N == 512) __syncthreads();
+      }
+      auto add = [&](int i, float m2) {
+        const float c2 = m2 * pref2;
+        sum[i] += c2;
+        sq[i] = fmaf(c2, c2, sq[i]);
+      };
+#pragma unroll
+      for (int s = 0; s < kSlots; ++s) {
+        add(2 * s, lo[s].m2);
+        add(2 * s + 1, hi[s].m2);
+      }
+      add(2 * kSlots, mid.m2);
+      if (tid == 0) add_s1(s1, lo[0].mean);
+      if (++ngroups == kMaxFp32Groups) {
+        flush();
+        ngroups = 0;
+      }
+    }
+    if (ngroups) flush();
+  }
+}
+
+// Centring of the spectra that k1_fft wrote (they are still in L2): thread = bin of a
+// block of 256, with its column of the group's m coefficients staged in shared memory
+// (each thread reads and writes its own column only: no barrier); a CTA takes a run of
+// groups and keeps its bins' S2 sums in registers.  Splitting the bins over CTAs instead
+// of one CTA per group gives 9 times the loads in flight at T = 4096.
+template <int FMT>
+__global__ void __launch_bounds__(kThreadsK1)
+k1_centre(int G, int m, int M, int Mp, int groups_per_cta, SpecRows sp,
+          const int* __restrict__ s2_auto, double* __restrict__ acc2, int n_s2, float pref2,
+          OperandImage oi, double* __restrict__ acc1, int C) {
+  extern __shared__ float4 smem_raw[];
+  float2* col = reinterpret_cast<float2*>(smem_raw) + threadIdx.x;  // [m][256]
+  const int k = blockIdx.x * kThreadsK1 + threadIdx.x, c = blockIdx.z;
+  if (k >= Mp) return;
+  const int g0 = blockIdx.y * groups_per_cta, g1 = min(G, g0 + groups_per_cta);
+  float sum = 0.f, sq = 0.f;
+  float s1[4] = {0.f, 0.f, 0.f, 0.f};
+  for (int g = g0; g < g1; ++g) {
+    float2* grow = sp.rows + (long long)c * sp.chan_stride + (long long)g * m * sp.stride;
+    if (k < M) {
+#pragma unroll 8
+      for (int j = 0; j < m; ++j) col[j * kThreadsK1] = grow[(long long)j * sp.stride + k];
+    }
+    const float p = centre_column<FMT>(col, kThreadsK1, grow, sp.stride, sp.mirror, 1, k, c, g, m,
+                                       M, Mp, oi, s1);
+    const float c2 = p * pref2;
+    sum += c2;
+    sq = fmaf(c2, c2, sq);
+  }
+  const int ia = s2_auto[c];
+  if (k < M && ia >= 0) {
+    const long long plane = (long long)n_s2 * M;
+    atomicAdd(acc2 + (long long)ia * M + k, (double)sum);
+    atomicAdd(acc2 + 2 * plane + (long long)ia * M + k, (double)sq);
+  }
+  if (k == 0 && acc1)
+    for (int q = 0; q < 4; ++q) atomicAdd(acc1 + q * C + c, (double)s1[q]);
 }
 
 // Cross-channel S2 (Sec. 7, Eq. 47): c2(a_k, b_k*) = 1/(m-1) sum_j da_jk db_jk*
@@ -935,6 +1276,52 @@ cudaError_t k1_occupancy(Kern kern, size_t smem, int* occ) {
   return cudaSuccess;
 }
 
+// k1_centre keeps a group's columns of 256 bins in shared memory
+constexpr size_t kCentreMaxSmem = 160u << 10;
+
+// k1_fft over whole groups (power) or all frames; N = T/2 is 512, 1024 or 2048
+template <int DTYPE, bool kPower>
+cudaError_t launch_k1_fft(const SampleSource& src, long long sample0, int G, int C, int T, int m,
+                          const float* win, const float2* tw, const SpecRows& spec,
+                          const int* s2_auto, double* acc2, int n_s2, float pref2, double* acc1,
+                          int nsm, cudaStream_t stream) {
+  auto kern = T == 1024   ? k1_fft<DTYPE, 512, kPower>
+              : T == 2048 ? k1_fft<DTYPE, 1024, kPower>
+                          : k1_fft<DTYPE, 2048, kPower>;
+  const size_t smem = (size_t)(2 * kFftPoints + twiddle_count(T) + T / 2) * sizeof(float2);
+  cudaError_t e = set_smem_limit(
+      kern, (size_t)(2 * kFftPoints + twiddle_count(kMaxT) + kMaxT / 2) * sizeof(float2));
+  if (e != cudaSuccess) return e;
+  int occ = 1;
+  e = k1_occupancy(kern, smem, &occ);
+  if (e != cudaSuccess) return e;
+  const int FB = kFftPoints / (T / 2);
+  const long long units = kPower ? G : ((long long)G * m + FB - 1) / FB;
+  const long long wave = std::max(1, nsm * occ / C);
+  kern<<<dim3((unsigned)std::min(units, wave), (unsigned)C), kThreadsK1, smem, stream>>>(
+      src, sample0, G, m, win, tw, spec, s2_auto, acc2, n_s2, pref2, acc1, C);
+  return cudaGetLastError();
+}
+
+template <int FMT>
+cudaError_t launch_k1_centre(int G, int C, int m, int M, int Mp, const SpecRows& spec,
+                             const int* s2_auto, double* acc2, int n_s2, float pref2,
+                             const OperandImage& oi, double* acc1, int nsm, cudaStream_t stream) {
+  const size_t smem = (size_t)m * kThreadsK1 * sizeof(float2);
+  if (smem > kCentreMaxSmem) return cudaErrorInvalidValue;
+  cudaError_t e = set_smem_limit(k1_centre<FMT>, kCentreMaxSmem);
+  if (e != cudaSuccess) return e;
+  const int bx = (Mp + kThreadsK1 - 1) / kThreadsK1;
+  // about eight CTAs per SM, at most kMaxFp32Groups groups in a float32 sum
+  long long gpc = (long long)G * bx * C / (8ll * nsm);
+  gpc = std::max(1ll, std::min<long long>(gpc, kMaxFp32Groups));
+  while ((G + gpc - 1) / gpc > 65535) ++gpc;  // (more than 4 million groups in a batch)
+  k1_centre<FMT><<<dim3((unsigned)bx, (unsigned)((G + gpc - 1) / gpc), (unsigned)C), kThreadsK1,
+                   smem, stream>>>(G, m, M, Mp, (int)gpc, spec, s2_auto, acc2, n_s2, pref2, oi,
+                                   acc1, C);
+  return cudaGetLastError();
+}
+
 template <int DTYPE, int FMT>
 cudaError_t launch_k1_t(const SampleSource& src, long long sample0, int G, int C, int T, int m,
                         int M, int Mp, const float* win, const float2* tw, const SpecRows& spec,
@@ -943,7 +1330,7 @@ cudaError_t launch_k1_t(const SampleSource& src, long long sample0, int G, int C
                         cudaStream_t stream, double* acc1, int mode) {
   // a group whose coefficients fit beside a batch of FFT buffers stays resident
   const size_t fixed = (size_t)m * Mp * sizeof(float2) + (size_t)2 * C * M * sizeof(float) +
-                       (size_t)T * (sizeof(float2) + sizeof(float));  // + twiddles and window
+                       (size_t)twiddle_count(T) * sizeof(float2) + (size_t)T * sizeof(float);
   const size_t per_frame = (size_t)(T / 2) * sizeof(float2);  // one buffer of T/2 points
   // kK1Auto: three CTAs per SM with a smaller batch of frames beat two with a
   // larger one (T = 1024, m = 10: 2.59 vs 2.69 ms per step), else the 96 KB
@@ -967,6 +1354,25 @@ cudaError_t launch_k1_t(const SampleSource& src, long long sample0, int G, int C
     kern<<<rgrid, kThreadsK1, wsmem, stream>>>(src, sample0, G, C, T, m, M, Mp, win, tw, spec,
                                                s2_auto, acc2, n_s2, pref2, oi, acc1);
     return cudaGetLastError();
+  }
+  // Long frames: the power spectrum alone from registers; groups that do not fit in
+  // shared memory (or kK1Frames) as transform and centring in two kernels.
+  if (T >= 1024 && (size_t)m * kThreadsK1 * sizeof(float2) <= kCentreMaxSmem) {
+    const bool two = mode == kK1Frames || fixed + per_frame > kK1ResidentBytes;
+    if (two || (!spec.store && mode == kK1Auto)) {
+      int dev = 0, nsm = 1;
+      cudaError_t e = cudaGetDevice(&dev);
+      if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+      if (e != cudaSuccess) return e;
+      if (!spec.store)
+        return launch_k1_fft<DTYPE, true>(src, sample0, G, C, T, m, win, tw, spec, s2_auto, acc2,
+                                          n_s2, pref2, acc1, nsm, stream);
+      e = launch_k1_fft<DTYPE, false>(src, sample0, G, C, T, m, win, tw, spec, s2_auto, acc2, n_s2,
+                                      pref2, acc1, nsm, stream);
+      if (e != cudaSuccess) return e;
+      return launch_k1_centre<FMT>(G, C, m, M, Mp, spec, s2_auto, acc2, n_s2, pref2, oi, acc1, nsm,
+                                   stream);
+    }
   }
   const size_t budget = mode == kK1Frames ? 0
                         : (mode == kK1Auto && fixed + per_frame <= kK1ResidentBytes3)

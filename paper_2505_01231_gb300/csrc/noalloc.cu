@@ -22,7 +22,7 @@ namespace {
 // spectra of all groups of one call.
 constexpr size_t kTableBytes = 128 << 10;
 constexpr size_t kWinOff = 0;                        // float  [4096]  window / sqrt(sum g^2)
-constexpr size_t kTwOff = 16 << 10;                  // float2 [4096]  e^{+2 pi j a/T}
+constexpr size_t kTwOff = 16 << 10;                  // float2 [4096]  twiddles
 constexpr size_t kAccOff = 48 << 10;                 // double [4][2049] sums over groups
 constexpr size_t kAutoOff = kAccOff + 4 * 2049 * 8;  // int    s2 combination index (0)
 constexpr size_t kSpecOff = kTableBytes;
@@ -50,7 +50,7 @@ bool on_device(const void* ptr) {
   return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
-// The window scaled by 1/sqrt(sum g^2) and the twiddles e^{+2 pi j a/T}, built on
+// The window scaled by 1/sqrt(sum g^2) and the twiddles of K1's passes, built on
 // the device in float64 (the same definitions ss_plan evaluates on the host), so
 // that a call enqueues kernels and memsets only.  One block.
 constexpr int kTableThreads = 256;
@@ -78,9 +78,11 @@ k0_tables(int T, int window, double sigma, float* __restrict__ win, float2* __re
   const double scale = 1.0 / sqrt(red[0]);
   for (int i = threadIdx.x; i < T; i += kTableThreads) {
     win[i] = (float)(g_at(i) * scale);
-    double sn, cs;
-    sincospi(2.0 * i / T, &sn, &cs);
-    tw[i] = make_float2((float)cs, (float)sn);
+    if (i < twiddle_count(T)) {
+      double sn, cs;
+      sincospi(2.0 * twiddle_angle(T, i) / T, &sn, &cs);
+      tw[i] = make_float2((float)cs, (float)sn);
+    }
   }
 }
 
@@ -159,7 +161,7 @@ extern "C" ss_status ss_s2_noalloc(const float* d_signal, size_t n_samples, int 
   src.chunk_stride = (long long)n_samples;
   src.dtype = SS_F32;
   NA_TRY(launch_k1_spectra(src, 0, (int)G, 1, T, m, M, Mp, d_win, d_tw,
-                           SpecRows{d_spec, (long long)G * m * Mp, Mp, 0}, d_auto, d_acc, 1, 1.0f / (float)(m - 1),
+                           SpecRows{d_spec, (long long)G * m * Mp, Mp, 0, 0}, d_auto, d_acc, 1, 1.0f / (float)(m - 1),
                            4 * nsm, s));
   NA_TRY(launch_k4_finalize(d_acc, 1, 1, M, kLayoutVector, G, dt, d_S2, d_S2_err, s));
 #undef NA_TRY

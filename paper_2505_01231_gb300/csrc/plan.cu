@@ -313,6 +313,8 @@ ss_status process_device(ss_plan_s* p, const void* ptr, long long n, long long s
     src.dtype = p->dtype;
     const long long chan_stride = (long long)p->Gb_max * p->m * p->Ms;
     float2* const spec = p->d_spec + p->Z;  // bin 0 of the first row
+    const bool need_spec = !p->c3.empty() || !p->c4.empty() || p->n_s2cross > 0 ||
+                           !p->cx_ops[0].empty() || !p->cx_ops[1].empty() || !p->cx_ops[2].empty();
     // prefactors of c2, c3 and the two parts of c4 over the centred sums: the
     // k-statistics (Eq. 32-34, 85) or the natural estimators
     const double md = p->m;
@@ -330,7 +332,8 @@ ss_status process_device(ss_plan_s* p, const void* ptr, long long n, long long s
       record(p, 0, p->stream, true);
       SS_TRY(p, launch_k1_spectra(src, g0 * per_group, cnt, p->C, p->T, p->m, p->M, p->Mp,
                                   p->d_win, p->d_tw,
-                                  SpecRows{spec, chan_stride, p->Ms, p->mirror ? 1 : 0},
+                                  SpecRows{spec, chan_stride, p->Ms, p->mirror ? 1 : 0,
+                                           need_spec ? 1 : 0},
                                   p->d_s2auto, p->d_acc2, (int)p->c2.size(), pref2, 4 * p->nsm, p->stream,
                                   p->oi, p->d_acc1, p->k1_mode));
       if (p->n_s2cross > 0)
@@ -955,8 +958,10 @@ static ss_status plan_create(ss_plan_t* out, int channels, int T, double dt, int
   std::vector<float> gw(T);
   for (int i = 0; i < T; ++i) gw[i] = (float)(g[i] / std::sqrt(p->sg2));
   std::vector<float2> tw(T);
-  for (int a = 0; a < T; ++a)
-    tw[a] = make_float2((float)std::cos(2.0 * M_PI * a / T), (float)std::sin(2.0 * M_PI * a / T));
+  for (int i = 0; i < twiddle_count(T); ++i) {
+    const double a = 2.0 * M_PI * twiddle_angle(T, i) / T;
+    tw[i] = make_float2((float)std::cos(a), (float)std::sin(a));
+  }
 
   std::vector<int> s2auto(channels, -1);
   std::vector<int4> s2cross;
