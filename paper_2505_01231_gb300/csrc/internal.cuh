@@ -286,14 +286,14 @@ cudaError_t launch_k5_complex(const float2* spec, long long chan_stride, int G, 
 // `group` with the SM full, up to 1.75 times that with fewer items on an SM than it
 // holds; an item 1500 more; the last items of an SM end unevenly; and the `adds`
 // float64 additions of an item are taken by the L2 at about 200 a clock over the whole
-// GPU.  At most kMaxFp32Groups (a warp takes a quarter).  Measured (ms, K2 alone) for
+// GPU.  A warp takes a quarter of the groups, at most kMaxFp32Groups.  Measured (ms, K2 alone) for
 // 4 / 8 / 16 / 64 groups: T = 1024, m = 10, 2^28 samples 10.21 / 8.20 / 7.34 / 6.75;
 // T = 128, m = 32, 2^23 samples 0.113 / 0.108 / 0.130 / 0.166; T = 256, m = 10, 2^20
 // samples 0.033 / 0.033 / 0.040 / 0.062.
 inline int warp_item_groups(int G, long long tiles, int nsm, double group, int adds) {
   int best = 1;
   double tb = 1e300;
-  const int top = G < kMaxFp32Groups ? G : kMaxFp32Groups;
+  const int top = G < 4 * kMaxFp32Groups ? G : 4 * kMaxFp32Groups;
   for (int gc = 1; gc <= top; ++gc) {
     const long long items = (long long)((G + gc - 1) / gc) * tiles;
     const double item = ((gc + 3) / 4) * group + 1500.0;
@@ -346,6 +346,27 @@ size_t k3_smem_bytes(int FC);
 cudaError_t launch_k4_finalize(const double* acc, int n_combos, int rows, int M, int layout,
                                long long G, double norm, double* out, double* err,
                                cudaStream_t stream, const double* prev = nullptr);
+
+// Several grids in one launch, and n_blocks sets of them: set y reads the sums
+// acc_stride y doubles on and writes out_stride y doubles on.  Either of out and err
+// (device memory) may be NULL; launch_k4 drops grids with neither.
+struct K4Job {
+  const double* acc;
+  const double* prev;
+  double* out;
+  double* err;
+  long long plane, acc_stride, out_stride;
+  double mean_scale, sq_scale, mean_sq_scale;
+  int n_combos, rows, M, layout, first_block, wide;
+};
+constexpr int kK4Jobs = 3;
+struct K4Jobs {
+  K4Job job[kK4Jobs];
+  int n;
+};
+K4Job k4_job(const double* acc, int n_combos, int rows, int M, int layout, long long G, double norm,
+             double* out, double* err, const double* prev = nullptr);
+cudaError_t launch_k4(K4Jobs& js, int n_blocks, cudaStream_t stream);
 
 // dst[i] += src[i], i < n (device pointers): merges exported group sums.
 cudaError_t launch_add_f64(double* dst, const double* src, long long n, cudaStream_t stream);

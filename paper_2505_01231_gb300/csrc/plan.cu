@@ -249,6 +249,14 @@ void clear_events(ss_plan_s* p) {
   for (auto& l : p->launches) l = 0;
 }
 
+// how the sums of the S3 and S4 grids are stored
+int layout3(const ss_plan_s* p) { return p->C == 1 ? kLayoutS3Single : kLayoutCross; }
+int layout4(const ss_plan_s* p) {
+  return p->C != 1                      ? kLayoutCross
+         : p->precision == SS_PREC_FP32 ? kLayoutS4Single
+                                        : kLayoutS4Lower;
+}
+
 // Sequential spectra (Sec. 8): the block of seq_B groups that just ended gives
 // its means and standard errors (the sums since the snapshot, over seq_B groups)
 // in the finalize layout at block index seq_blocks of seq_out; then the snapshot
@@ -268,19 +276,15 @@ ss_status emit_block(ss_plan_s* p) {
     const double* q2 = p->d_prev;
     const double* q3 = q2 + p->n_acc2;
     const double* q4 = q3 + p->n_acc3;
-    if (n2)
-      SS_TRY(p, launch_k4_finalize(p->d_acc2, (int)p->c2.size(), 1, p->M, kLayoutVector,
-                                   p->seq_B, p->norm2, o2, e2, p->stream, q2));
-    if (n3)
-      SS_TRY(p, launch_k4_finalize(p->d_acc3, (int)p->c3.size(), p->rows3, p->M,
-                                   p->C == 1 ? kLayoutS3Single : kLayoutCross, p->seq_B,
-                                   p->norm3, o3, e3, p->stream, q3));
-    if (n4)
-      SS_TRY(p, launch_k4_finalize(p->d_acc4, (int)p->c4.size(), p->rows4, p->M,
-                                   p->C != 1                        ? kLayoutCross
-                                   : p->precision == SS_PREC_FP32 ? kLayoutS4Single
-                                                                   : kLayoutS4Lower,
-                                   p->seq_B, p->norm4, o4, e4, p->stream, q4));
+    K4Jobs js{};
+    js.n = 3;
+    js.job[0] = k4_job(p->d_acc2, (int)p->c2.size(), 1, p->M, kLayoutVector, p->seq_B, p->norm2, o2,
+                       e2, q2);
+    js.job[1] = k4_job(p->d_acc3, (int)p->c3.size(), p->rows3, p->M, layout3(p), p->seq_B, p->norm3,
+                       o3, e3, q3);
+    js.job[2] = k4_job(p->d_acc4, (int)p->c4.size(), p->rows4, p->M, layout4(p), p->seq_B, p->norm4,
+                       o4, e4, q4);
+    SS_TRY(p, launch_k4(js, 1, p->stream));
   }
   const std::pair<const double*, size_t> parts[3] = {
       {p->d_acc2, p->n_acc2}, {p->d_acc3, p->n_acc3}, {p->d_acc4, p->n_acc4}};
@@ -1167,46 +1171,60 @@ static ss_status ensure_out(ss_plan_s* p) {
   return SS_OK;
 }
 
-// K4 and the copies to the caller's buffers, stream-ordered (no synchronisation).
+// Device memory of the plan's own GPU: K4 writes it directly (a kernel may not reach
+// another GPU's memory, and managed memory is left to a copy).
+static bool own_device_ptr(const ss_plan_s* p, const void* ptr) {
+  cudaPointerAttributes a;
+  if (cudaPointerGetAttributes(&a, ptr) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return a.type == cudaMemoryTypeDevice && a.device == p->device;
+}
+
+// K4 into the caller's buffers, or into the finalize buffer and from there by copies
+// where a buffer is not memory of this GPU; stream-ordered (no synchronisation).
 static ss_status finalize_launch(ss_plan_s* p, double* S2, double* S3, double* S4,
                                  double* S2_err, double* S3_err, double* S4_err) {
-  ss_status st0 = ensure_out(p);
-  if (st0 != SS_OK) return st0;
   Pooled pl;
-  st0 = pooled(p, &pl);
+  ss_status st0 = pooled(p, &pl);
   if (st0 != SS_OK) return st0;
   const size_t n2 = p->c2.size() * p->M * 2;
   const size_t n3 = p->c3.size() * p->rows3 * p->M * 2;
   const size_t n4 = p->c4.size() * p->rows4 * p->M * 2;
-  double* o2 = p->d_out;
-  double* e2 = o2 + n2;
-  double* o3 = e2 + n2;
-  double* e3 = o3 + n3;
-  double* o4 = e3 + n3;
-  double* e4 = o4 + n4;
-  const bool single = p->C == 1;
+  double* const user[6] = {S2, S2_err, S3, S3_err, S4, S4_err};
+  const size_t cnt[6] = {n2, n2, n3, n3, n4, n4};
+  double* dst[6];
+  bool direct[6], staged = false;
+  for (int i = 0; i < 6; ++i) {
+    dst[i] = cnt[i] ? user[i] : nullptr;
+    direct[i] = !dst[i] || own_device_ptr(p, dst[i]);
+    staged = staged || !direct[i];
+  }
+  if (staged) {
+    st0 = ensure_out(p);
+    if (st0 != SS_OK) return st0;
+    size_t off = 0;
+    for (int i = 0; i < 6; ++i) {
+      if (!direct[i]) dst[i] = p->d_out + off;
+      off += cnt[i];
+    }
+  }
   record(p, 3, p->stream, true);
-  if (n2)
-    SS_TRY(p, launch_k4_finalize(pl.a2, (int)p->c2.size(), 1, p->M, kLayoutVector,
-                                 pl.groups, p->norm2, o2, e2, p->stream));
-  if (n3)
-    SS_TRY(p, launch_k4_finalize(pl.a3, (int)p->c3.size(), p->rows3, p->M,
-                                 single ? kLayoutS3Single : kLayoutCross, pl.groups, p->norm3,
-                                 o3, e3, p->stream));
-  if (n4)
-    SS_TRY(p, launch_k4_finalize(pl.a4, (int)p->c4.size(), p->rows4, p->M,
-                                 !single ? kLayoutCross
-                                 : p->precision == SS_PREC_FP32 ? kLayoutS4Single : kLayoutS4Lower,
-                                 pl.groups, p->norm4,
-                                 o4, e4, p->stream));
+  K4Jobs js{};
+  js.n = 3;
+  js.job[0] = k4_job(pl.a2, (int)p->c2.size(), 1, p->M, kLayoutVector, pl.groups, p->norm2, dst[0],
+                     dst[1]);
+  js.job[1] = k4_job(pl.a3, (int)p->c3.size(), p->rows3, p->M, layout3(p), pl.groups, p->norm3,
+                     dst[2], dst[3]);
+  js.job[2] = k4_job(pl.a4, (int)p->c4.size(), p->rows4, p->M, layout4(p), pl.groups, p->norm4,
+                     dst[4], dst[5]);
+  SS_TRY(p, launch_k4(js, 1, p->stream));
   record(p, 3, p->stream, false);
-  const std::pair<double*, std::pair<const double*, size_t>> copies[6] = {
-      {S2, {o2, n2}}, {S2_err, {e2, n2}}, {S3, {o3, n3}},
-      {S3_err, {e3, n3}}, {S4, {o4, n4}}, {S4_err, {e4, n4}}};
-  for (const auto& c : copies)
-    if (c.first && c.second.second)
-      SS_TRY(p, cudaMemcpyAsync(c.first, c.second.first, c.second.second * sizeof(double),
-                                cudaMemcpyDefault, p->stream));
+  for (int i = 0; i < 6; ++i)
+    if (!direct[i])
+      SS_TRY(p, cudaMemcpyAsync(user[i], dst[i], cnt[i] * sizeof(double), cudaMemcpyDefault,
+                                p->stream));
   return SS_OK;
 }
 
@@ -1370,20 +1388,22 @@ ss_status ss_finalize_complex(ss_plan_t p, double* S, double* S_err) {
   }
   const int nn = 2 * p->M - 1;
   const double norms[3] = {p->norm2, p->norm3, p->norm4};
-  // each order's combinations in one K4 launch over its block of the buffer
+  // each order's combinations over their block of the buffer, one K4 launch
   double* mean[3];
   double* err[3];
   size_t off = 0;
+  K4Jobs js{};
+  js.n = 3;
   for (int o = 0; o < 3; ++o) {
     const size_t combos = p->cx_ops[o].size() / (o + 2);
     const size_t per = 2 * (o == 0 ? (size_t)nn : (size_t)nn * nn);
     mean[o] = p->d_out + off;
     err[o] = p->d_out + total + off;
-    if (combos)
-      SS_TRY(p, launch_k4_finalize(p->d_cx_acc[o], (int)combos, o == 0 ? 1 : nn, nn,
-                                   kLayoutCross, p->groups, norms[o], mean[o], err[o], p->stream));
+    js.job[o] = k4_job(p->d_cx_acc[o], (int)combos, o == 0 ? 1 : nn, nn, kLayoutCross, p->groups,
+                       norms[o], mean[o], err[o]);
     off += combos * per;
   }
+  SS_TRY(p, launch_k4(js, 1, p->stream));
   // to the caller in record order
   size_t seen[3] = {0, 0, 0};
   size_t out_off = 0;
