@@ -49,14 +49,20 @@ struct SampleSource {
   int dtype;  // SS_F32 or SS_I16
 };
 
+// Groups of a block when a batch is one block (its sums in one place).
+constexpr int kOneBlock = 0x7fffffff;
+
 // The centred spectra K1 writes: bin 0 of channel c's frame row r is at
 // rows + c * chan_stride + r * stride.  Mp bins from there on are written (zeros
 // past M - 1); with mirror, also the conjugates at the bins -(M - 1) .. -1 before.
 // Without store, nothing reads the spectra (S2 alone) and they need not be written.
+// The S2 sums of block g / block_groups of the groups go block_stride doubles apart.
 struct SpecRows {
   float2* rows;
   long long chan_stride;
   int stride, mirror, store;
+  int block_groups = kOneBlock;
+  long long block_stride = 0;
 };
 
 // One channel combination of one order; channels as in the ABI records.
@@ -213,8 +219,8 @@ constexpr int kTcTileM = 128, kTcTileN = 128;
 cudaError_t launch_k3_trispec_tc(const CUtensorMap& tm_img, const OperandImage& oi, int channel,
                                  int G, int m, int M, int Mp,
                                  const TileInfo* tiles, int n_tiles, int precision, double* acc,
-                                 long long plane, int nsm, int* counter, int* status,
-                                 cudaStream_t stream);
+                                 long long plane, int block_groups, long long block_stride,
+                                 int nsm, int* counter, int* status, cudaStream_t stream);
 size_t k3tc_smem_bytes(int precision);
 
 // K3 for several channels (FP32 CUDA cores): C4(a_k, b_k*, c_l, d_l*) of every
@@ -335,7 +341,7 @@ cudaError_t launch_k2_points(const float2* spec, int Mp, int G, int m, const int
 // the one-channel S4 cut at l = M - 1 for every k, stored at acc[k * sk + l * sl]
 cudaError_t launch_k3_column(const float2* spec, int Mp, int G, int m, int M, float pref4a,
                              float pref4b, double* acc, long long plane, int sk, int sl,
-                             cudaStream_t stream);
+                             int block_groups, long long block_stride, cudaStream_t stream);
 
 // dynamic shared memory of the pair kernels for FC frames per stage
 size_t k2_smem_bytes(int FC);
@@ -367,6 +373,10 @@ struct K4Jobs {
 K4Job k4_job(const double* acc, int n_combos, int rows, int M, int layout, long long G, double norm,
              double* out, double* err, const double* prev = nullptr);
 cudaError_t launch_k4(K4Jobs& js, int n_blocks, cudaStream_t stream);
+
+// acc[i] += the sum over n_blocks of blk[b * stride + i], and prev[i] = acc[i], i < n
+cudaError_t launch_add_blocks(double* acc, double* prev, const double* blk, long long stride,
+                              int n_blocks, long long n, cudaStream_t stream);
 
 // dst[i] += src[i], i < n (device pointers): merges exported group sums.
 cudaError_t launch_add_f64(double* dst, const double* src, long long n, cudaStream_t stream);

@@ -148,7 +148,28 @@ __global__ void k_add_f64(double* __restrict__ dst, const double* __restrict__ s
     dst[i] += src[i];
 }
 
+__global__ void k_add_blocks(double* __restrict__ acc, double* __restrict__ prev,
+                             const double* __restrict__ blk, long long stride, int n_blocks,
+                             long long n) {
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
+       i += (long long)gridDim.x * blockDim.x) {
+    double s = acc[i];
+#pragma unroll 8
+    for (int b = 0; b < n_blocks; ++b) s += blk[b * stride + i];
+    acc[i] = s;
+    prev[i] = s;
+  }
+}
+
 }  // namespace
+
+cudaError_t launch_add_blocks(double* acc, double* prev, const double* blk, long long stride,
+                              int n_blocks, long long n, cudaStream_t stream) {
+  if (n <= 0) return cudaSuccess;
+  const long long grid = std::min<long long>((n + 255) / 256, 4096);
+  k_add_blocks<<<(int)grid, 256, 0, stream>>>(acc, prev, blk, stride, n_blocks, n);
+  return cudaGetLastError();
+}
 
 cudaError_t launch_add_f64(double* dst, const double* src, long long n, cudaStream_t stream) {
   if (n <= 0) return cudaSuccess;

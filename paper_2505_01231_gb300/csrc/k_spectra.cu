@@ -358,8 +358,15 @@ k1_spectra(SampleSource src, long long sample0, int G, int C, int T, int m, int 
   for (int i = threadIdx.x; i < 2 * C * M; i += blockDim.x) s2sum[i] = 0.f;
   if (threadIdx.x < 16) s1s[threadIdx.x >> 2][threadIdx.x & 3] = 0.f;
 
-  int ngroups = 0;  // groups in the float32 sums since the last flush
+  int ngroups = 0;  // groups in the float32 sums since the last flush, all of block cur
+  int cur = 0;
   for (int g = blockIdx.x; g < G; g += gridDim.x) {
+    if (g / sp.block_groups != cur) {
+      if (ngroups)
+        flush_k1_sums(C, M, s2_auto, acc2 + cur * sp.block_stride, n_s2, s2sum, s2sq, s1s, acc1);
+      ngroups = 0;
+      cur = g / sp.block_groups;
+    }
     for (int c = 0; c < C; ++c) {
       float2* grow = sp.rows + (long long)c * sp.chan_stride + (long long)g * m * sp.stride;
       for (int k = threadIdx.x; k < M; k += blockDim.x) gsum[k] = make_float2(0.f, 0.f);
@@ -422,12 +429,13 @@ k1_spectra(SampleSource src, long long sample0, int G, int C, int T, int m, int 
       }
     }
     if (++ngroups == kMaxFp32Groups) {
-      flush_k1_sums(C, M, s2_auto, acc2, n_s2, s2sum, s2sq, s1s, acc1);
+      flush_k1_sums(C, M, s2_auto, acc2 + cur * sp.block_stride, n_s2, s2sum, s2sq, s1s, acc1);
       ngroups = 0;
     }
   }
   // the CTA's remaining float32 partial sums into the float64 accumulators
-  if (ngroups) flush_k1_sums(C, M, s2_auto, acc2, n_s2, s2sum, s2sq, s1s, acc1);
+  if (ngroups)
+    flush_k1_sums(C, M, s2_auto, acc2 + cur * sp.block_stride, n_s2, s2sum, s2sq, s1s, acc1);
 }
 
 // The points n, n + 1 (n even) of a row as one 16-byte store (they stay a pair under swz)
@@ -635,8 +643,15 @@ k1_spectra_res(SampleSource src, long long sample0, int G, int C, int T, int m, 
     return true;
   };
   bool have = blockIdx.x < G && prefetch(blockIdx.x, 0, 0);  // pre holds the batch's samples
-  int ngroups = 0;  // groups in the float32 sums since the last flush
+  int ngroups = 0;  // groups in the float32 sums since the last flush, all of block cur
+  int cur = 0;
   for (int g = blockIdx.x; g < G; g += gridDim.x) {
+    if (g / sp.block_groups != cur) {
+      if (ngroups)
+        flush_k1_sums(C, M, s2_auto, acc2 + cur * sp.block_stride, n_s2, s2sum, s2sq, s1s, acc1);
+      ngroups = 0;
+      cur = g / sp.block_groups;
+    }
     for (int c = 0; c < C; ++c) {
       for (int j0 = 0; j0 < m; j0 += FB) {
         const int nf = min(FB, m - j0);
@@ -736,11 +751,12 @@ k1_spectra_res(SampleSource src, long long sample0, int G, int C, int T, int m, 
       centre_resident<FMT>(Xs, sp, c, g, m, M, Mp, oi, s2_auto[c], s2sum, s2sq, s1s[c], pref2);
     }
     if (++ngroups == kMaxFp32Groups) {
-      flush_k1_sums(C, M, s2_auto, acc2, n_s2, s2sum, s2sq, s1s, acc1);
+      flush_k1_sums(C, M, s2_auto, acc2 + cur * sp.block_stride, n_s2, s2sum, s2sq, s1s, acc1);
       ngroups = 0;
     }
   }
-  if (ngroups) flush_k1_sums(C, M, s2_auto, acc2, n_s2, s2sum, s2sq, s1s, acc1);
+  if (ngroups)
+    flush_k1_sums(C, M, s2_auto, acc2 + cur * sp.block_stride, n_s2, s2sum, s2sq, s1s, acc1);
 }
 
 // One Stockham pass of a warp's own frame (N points in the warp's shared buffer,
@@ -813,8 +829,15 @@ k1_spectra_warp(SampleSource src, long long sample0, int G, int C, int T, int m,
   }
   __syncthreads();
 
-  int ngroups = 0;  // groups in the float32 sums since the last flush
+  int ngroups = 0;  // groups in the float32 sums since the last flush, all of block cur
+  int cur = 0;
   for (int g = blockIdx.x; g < G; g += gridDim.x) {
+    if (g / sp.block_groups != cur) {
+      if (ngroups)
+        flush_k1_sums(C, M, s2_auto, acc2 + cur * sp.block_stride, n_s2, s2sum, s2sq, s1s, acc1);
+      ngroups = 0;
+      cur = g / sp.block_groups;
+    }
     for (int c = 0; c < C; ++c) {
       for (int j = warp; j < m; j += kWarps) {
         // the frame's samples times the window, packed as N complex points
@@ -872,11 +895,12 @@ k1_spectra_warp(SampleSource src, long long sample0, int G, int C, int T, int m,
       __syncthreads();  // Xs is free for the next channel or group
     }
     if (++ngroups == kMaxFp32Groups) {
-      flush_k1_sums(C, M, s2_auto, acc2, n_s2, s2sum, s2sq, s1s, acc1);
+      flush_k1_sums(C, M, s2_auto, acc2 + cur * sp.block_stride, n_s2, s2sum, s2sq, s1s, acc1);
       ngroups = 0;
     }
   }
-  if (ngroups) flush_k1_sums(C, M, s2_auto, acc2, n_s2, s2sum, s2sq, s1s, acc1);
+  if (ngroups)
+    flush_k1_sums(C, M, s2_auto, acc2 + cur * sp.block_stride, n_s2, s2sum, s2sq, s1s, acc1);
 }
 
 // ---------------------------------------------------------------------------
@@ -1071,12 +1095,13 @@ k1_fft(SampleSource src, long long sample0, int G, int m, const float* __restric
     float s1[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
     for (int i = 0; i < 2 * kSlots + 1; ++i) sum[i] = sq[i] = 0.f;
-    auto flush = [&]() {
+    auto flush = [&](int blk) {
       const long long plane = (long long)n_s2 * M;
+      double* dst = acc2 + blk * sp.block_stride + (long long)ia * M;
       auto put = [&](int k, float a, float b) {
         if (ia < 0) return;
-        atomicAdd(acc2 + (long long)ia * M + k, (double)a);
-        atomicAdd(acc2 + 2 * plane + (long long)ia * M + k, (double)b);
+        atomicAdd(dst + k, (double)a);
+        atomicAdd(dst + 2 * plane + k, (double)b);
       };
 #pragma unroll
       for (int s = 0; s < kSlots; ++s) {
@@ -1094,9 +1119,14 @@ k1_fft(SampleSource src, long long sample0, int G, int m, const float* __restric
 #pragma unroll
       for (int i = 0; i < 2 * kSlots + 1; ++i) sum[i] = sq[i] = 0.f;
     };
-    int g = blockIdx.x, ngroups = 0;
+    int g = blockIdx.x, ngroups = 0, cur = 0;
     if (g < G) load((long long)g * m, min(FB, m), pre);
     for (; g < G; g += gridDim.x) {
+      if (g / sp.block_groups != cur) {
+        if (ngroups) flush(cur);
+        ngroups = 0;
+        cur = g / sp.block_groups;
+      }
 #pragma unroll
       for (int s = 0; s < kSlots; ++s) {
         lo[s].clear();
@@ -1149,11 +1179,11 @@ k1_fft(SampleSource src, long long sample0, int G, int m, const float* __restric
       add(2 * kSlots, mid.m2);
       if (tid == 0) add_s1(s1, lo[0].mean);
       if (++ngroups == kMaxFp32Groups) {
-        flush();
+        flush(cur);
         ngroups = 0;
       }
     }
-    if (ngroups) flush();
+    if (ngroups) flush(cur);
   }
 }
 
@@ -1174,7 +1204,20 @@ k1_centre(int G, int m, int M, int Mp, int groups_per_cta, SpecRows sp,
   const int g0 = blockIdx.y * groups_per_cta, g1 = min(G, g0 + groups_per_cta);
   float sum = 0.f, sq = 0.f;
   float s1[4] = {0.f, 0.f, 0.f, 0.f};
+  const int ia = s2_auto[c];
+  int cur = g0 / sp.block_groups;
+  auto flush = [&]() {
+    if (k >= M || ia < 0) return;
+    double* dst = acc2 + cur * sp.block_stride + (long long)ia * M + k;
+    atomicAdd(dst, (double)sum);
+    atomicAdd(dst + 2 * (long long)n_s2 * M, (double)sq);
+    sum = sq = 0.f;
+  };
   for (int g = g0; g < g1; ++g) {
+    if (g / sp.block_groups != cur) {
+      flush();
+      cur = g / sp.block_groups;
+    }
     float2* grow = sp.rows + (long long)c * sp.chan_stride + (long long)g * m * sp.stride;
     if (k < M) {
 #pragma unroll 8
@@ -1186,12 +1229,7 @@ k1_centre(int G, int m, int M, int Mp, int groups_per_cta, SpecRows sp,
     sum += c2;
     sq = fmaf(c2, c2, sq);
   }
-  const int ia = s2_auto[c];
-  if (k < M && ia >= 0) {
-    const long long plane = (long long)n_s2 * M;
-    atomicAdd(acc2 + (long long)ia * M + k, (double)sum);
-    atomicAdd(acc2 + 2 * plane + (long long)ia * M + k, (double)sq);
-  }
+  flush();
   if (k == 0 && acc1)
     for (int q = 0; q < 4; ++q) atomicAdd(acc1 + q * C + c, (double)s1[q]);
 }

@@ -235,12 +235,14 @@ constexpr int kColThreads = 128;
 
 __global__ void __launch_bounds__(kColThreads)
 k3_column(const float2* __restrict__ spec, int Mp, int G, int m, int M, float pref_a,
-          float pref_b, double* __restrict__ acc, long long plane, int sk_out, int sl_out) {
+          float pref_b, double* __restrict__ acc, long long plane, int sk_out, int sl_out,
+          int block_groups, long long block_stride) {
   const int k = blockIdx.x * kColThreads + threadIdx.x;
   const int l = M - 1;
   if (k >= M) return;
   float sum = 0.f, sq = 0.f;
-  for (int g = blockIdx.y; g < G; g += gridDim.y) {
+  const int ge = min(G, (int)(blockIdx.z + 1) * block_groups);
+  for (int g = blockIdx.z * block_groups + blockIdx.y; g < ge; g += gridDim.y) {
     const float2* row = spec + (long long)g * m * Mp;
     float q = 0.f, sk = 0.f, sl = 0.f, rr = 0.f, ii = 0.f, xx = 0.f, xt = 0.f;
     for (int j = 0; j < m; ++j, row += Mp) {
@@ -262,20 +264,25 @@ k3_column(const float2* __restrict__ spec, int Mp, int G, int m, int M, float pr
     sum += c4;
     sq = fmaf(c4, c4, sq);
   }
-  const long long o = (long long)l * sl_out + (long long)k * sk_out;
+  const long long o = blockIdx.z * block_stride + (long long)l * sl_out + (long long)k * sk_out;
   atomicAdd(acc + o, (double)sum);
   atomicAdd(acc + 2 * plane + o, (double)sq);
 }
 
 cudaError_t launch_k3_column(const float2* spec, int Mp, int G, int m, int M, float pref4a,
                              float pref4b, double* acc, long long plane, int sk, int sl,
-                             cudaStream_t stream) {
+                             int block_groups, long long block_stride, cudaStream_t stream) {
   if (G <= 0 || M <= 0) return cudaSuccess;
+  if (block_groups <= 0 || block_groups > G) block_groups = G;
+  const int n_blocks = (G + block_groups - 1) / block_groups;
   const int gx = (M + kColThreads - 1) / kColThreads;
-  // at most kMaxFp32Groups groups in a thread's float32 sums (grid y <= 65535)
-  const int gy = std::min(G, std::min(65535, std::max(1024, (G + kMaxFp32Groups - 1) / kMaxFp32Groups)));
-  k3_column<<<dim3((unsigned)gx, (unsigned)gy), kColThreads, 0, stream>>>(
-      spec, Mp, G, m, M, pref4a, pref4b, acc, plane, sk, sl);
+  // at most kMaxFp32Groups groups in a thread's float32 sums (grid y, z <= 65535)
+  const int gy = std::min(block_groups,
+                          std::min(65535, std::max(std::max(1, 1024 / n_blocks),
+                                                   (block_groups + kMaxFp32Groups - 1) / kMaxFp32Groups)));
+  if (n_blocks > 65535) return cudaErrorInvalidValue;
+  k3_column<<<dim3((unsigned)gx, (unsigned)gy, (unsigned)n_blocks), kColThreads, 0, stream>>>(
+      spec, Mp, G, m, M, pref4a, pref4b, acc, plane, sk, sl, block_groups, block_stride);
   return cudaGetLastError();
 }
 

@@ -37,6 +37,8 @@
 // at the end of an item they add both to the float64 accumulators.  Tiles of the last l-block are as
 // narrow as the bins left (N a multiple of 16).  Every wait is bounded; on a
 // failure the CTA stops, drains its copies and products and frees its TMEM.
+#include <algorithm>
+
 #include "internal.cuh"
 #include "pipeline.cuh"
 
@@ -145,6 +147,7 @@ __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::
 // Record of a group for the MMA warps and the epilogue (FP16: with its row scales).
 struct GroupRec {
   int k0, l0, n, flags;  // n = tile columns; flags: 1 = last group of its item, 2 = stop
+  long long off;         // doubles to the sums of the group's block
 };
 
 constexpr int kPsSlots = 8;  // ring of per-group records (a power of two)
@@ -155,7 +158,7 @@ template <int kFmt, int kPasses>
 __global__ void __launch_bounds__(kTcThreads, 1)
 k3_trispec_tc(const __grid_constant__ CUtensorMap tm_img, const float* __restrict__ rsc,
               int G, int nkc, int ndc, int M, int Mp,
-              const TileInfo* __restrict__ tiles, WorkQueue wq, double* __restrict__ acc,
+              const TileInfo* __restrict__ tiles, WarpQueue wq, double* __restrict__ acc,
               long long plane, int* __restrict__ status) {
   using F = OpFmt<kFmt>;
   constexpr int S = F::kStages, KC = F::kChunks;
@@ -224,9 +227,10 @@ k3_trispec_tc(const __grid_constant__ CUtensorMap tm_img, const float* __restric
       for (;;) {
         const int item = atomicAdd(wq.counter, 1);
         if (item >= wq.n_items || *(volatile int*)&s_fail) break;
-        const int t = item % wq.n_tiles;
-        const int ga = (item / wq.n_tiles) * wq.group_chunk;
-        const int gb = min(G, ga + wq.group_chunk);
+        const int chunk = item / wq.n_tiles, t = item - chunk * wq.n_tiles;
+        const int blk = chunk / wq.chunks_per_block;
+        const int ga = blk * wq.block_groups + (chunk - blk * wq.chunks_per_block) * wq.group_chunk;
+        const int gb = min(min(G, (blk + 1) * wq.block_groups), ga + wq.group_chunk);
         const TileInfo ti = tiles[t];
         const uint32_t pk = (uint32_t)min(kTM, Mp - ti.k0) * 4u;
         const uint32_t pl = (uint32_t)min(ti.ncols, Mp - ti.l0) * 4u;
@@ -238,7 +242,7 @@ k3_trispec_tc(const __grid_constant__ CUtensorMap tm_img, const float* __restric
             ok = false;
             break;
           }
-          prec[p] = GroupRec{ti.k0, ti.l0, ti.ncols, (g == gb - 1) ? 1 : 0};
+          prec[p] = GroupRec{ti.k0, ti.l0, ti.ncols, (g == gb - 1) ? 1 : 0, blk * wq.block_stride};
           if constexpr (F::kScaled) {
             const float* rg = rsc + (long long)g * Mp;
             mbar_arrive_expect_tx(&psfull[p], pk + pl);
@@ -447,7 +451,7 @@ k3_trispec_tc(const __grid_constant__ CUtensorMap tm_img, const float* __restric
         for (int i = 0; i < kEpiCols; ++i) {
           const int l = r.l0 + col0 + i;
           if (i < 16 * nh && k <= l && l < M) {
-            const long long o = (long long)l * M + k;
+            const long long o = r.off + (long long)l * M + k;
             atomicAdd(acc + o, (double)sm[i]);
             atomicAdd(acc + 2 * plane + o, (double)sq[i]);
           }
@@ -485,8 +489,9 @@ int k3tc_stage_chunks(int precision) {
 
 cudaError_t launch_k3_trispec_tc(const CUtensorMap& tm_img, const OperandImage& oi, int channel,
                                  int G, int m, int M, int Mp, const TileInfo* tiles, int n_tiles,
-                                 int precision, double* acc, long long plane, int nsm,
-                                 int* counter, int* status, cudaStream_t stream) {
+                                 int precision, double* acc, long long plane, int block_groups,
+                                 long long block_stride, int nsm, int* counter, int* status,
+                                 cudaStream_t stream) {
   if (G <= 0 || n_tiles <= 0) return cudaSuccess;
   if (m < 4 || m > kMaxGramM || (Mp & 15)) return cudaErrorInvalidValue;
   const size_t smem = k3tc_smem_bytes(precision);
@@ -498,11 +503,17 @@ cudaError_t launch_k3_trispec_tc(const CUtensorMap& tm_img, const OperandImage& 
   if (e != cudaSuccess) return e;
   // one CTA per SM: each CTA allocates all 512 TMEM columns
   const int n_cta = nsm;
-  WorkQueue wq;
+  WarpQueue wq;
   wq.counter = counter;
   wq.n_tiles = n_tiles;
-  wq.group_chunk = work_group_chunk(G, n_tiles, n_cta);
-  wq.n_items = n_tiles * ((G + wq.group_chunk - 1) / wq.group_chunk);
+  wq.n_combos = 1;
+  if (block_groups <= 0 || block_groups > G) block_groups = G;
+  const int n_blocks = (G + block_groups - 1) / block_groups;
+  wq.block_groups = block_groups;
+  wq.block_stride = block_stride;
+  wq.group_chunk = std::min(block_groups, work_group_chunk(G, n_tiles, n_cta));
+  wq.chunks_per_block = (block_groups + wq.group_chunk - 1) / wq.group_chunk;
+  wq.n_items = n_tiles * wq.chunks_per_block * n_blocks;
   e = cudaMemsetAsync(counter, 0, sizeof(int), stream);
   if (e != cudaSuccess) return e;
   const float* rsc = oi.rsc ? oi.rsc + (size_t)channel * oi.chan_rsc : nullptr;

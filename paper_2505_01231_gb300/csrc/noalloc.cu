@@ -161,7 +161,7 @@ extern "C" ss_status ss_s2_noalloc(const float* d_signal, size_t n_samples, int 
   src.chunk_stride = (long long)n_samples;
   src.dtype = SS_F32;
   NA_TRY(launch_k1_spectra(src, 0, (int)G, 1, T, m, M, Mp, d_win, d_tw,
-                           SpecRows{d_spec, (long long)G * m * Mp, Mp, 0, 0}, d_auto, d_acc, 1, 1.0f / (float)(m - 1),
+                           SpecRows{d_spec, (long long)G * m * Mp, Mp, 0, 0, kOneBlock, 0}, d_auto, d_acc, 1, 1.0f / (float)(m - 1),
                            4 * nsm, s));
   NA_TRY(launch_k4_finalize(d_acc, 1, 1, M, kLayoutVector, G, dt, d_S2, d_S2_err, s));
 #undef NA_TRY

@@ -286,17 +286,46 @@ ss_status emit_block(ss_plan_s* p) {
                        o4, e4, q4);
     SS_TRY(p, launch_k4(js, 1, p->stream));
   }
-  const std::pair<const double*, size_t> parts[3] = {
-      {p->d_acc2, p->n_acc2}, {p->d_acc3, p->n_acc3}, {p->d_acc4, p->n_acc4}};
-  double* q = p->d_prev;
-  for (const auto& pr : parts) {
-    if (pr.second)
-      SS_TRY(p, cudaMemcpyAsync(q, pr.first, pr.second * sizeof(double),
-                                cudaMemcpyDeviceToDevice, p->stream));
-    q += pr.second;
-  }
+  // the sums of orders 2 to 4 are one array
+  const size_t n = p->n_acc2 + p->n_acc3 + p->n_acc4;
+  if (n)
+    SS_TRY(p, cudaMemcpyAsync(p->d_prev, p->d_sums, n * sizeof(double), cudaMemcpyDeviceToDevice,
+                              p->stream));
   return SS_OK;
 }
+
+// A batch that computed n whole blocks into d_blocks: their means and errors in one
+// launch, then their sums into the plan's, where the snapshot moves to.
+ss_status emit_blocks(ss_plan_s* p, int n) {
+  const size_t n2 = p->c2.size() * p->M * 2;
+  const size_t n3 = p->c3.size() * p->rows3 * p->M * 2;
+  const size_t n4 = p->c4.size() * p->rows4 * p->M * 2;
+  const long long rec = 2 * (long long)(n2 + n3 + n4);
+  const long long room = std::max(0ll, p->seq_cap - p->seq_blocks);
+  if (room > 0) {
+    double* o = p->seq_out + p->seq_blocks * rec;
+    const double* q = p->d_blocks;
+    K4Jobs js{};
+    js.n = 3;
+    js.job[0] = k4_job(q, (int)p->c2.size(), 1, p->M, kLayoutVector, p->seq_B, p->norm2, o, o + n2);
+    o += 2 * n2;
+    js.job[1] = k4_job(q + p->n_acc2, (int)p->c3.size(), p->rows3, p->M, layout3(p), p->seq_B,
+                       p->norm3, o, o + n3);
+    o += 2 * n3;
+    js.job[2] = k4_job(q + p->n_acc2 + p->n_acc3, (int)p->c4.size(), p->rows4, p->M, layout4(p),
+                       p->seq_B, p->norm4, o, o + n4);
+    for (K4Job& j : js.job) {
+      j.acc_stride = (long long)p->seq_stride;
+      j.out_stride = rec;
+    }
+    SS_TRY(p, launch_k4(js, (int)std::min<long long>(room, n), p->stream));
+  }
+  SS_TRY(p, launch_add_blocks(p->d_sums, p->d_prev, p->d_blocks, (long long)p->seq_stride, n,
+                              (long long)p->seq_stride, p->stream));
+  p->seq_blocks += n;
+  return SS_OK;
+}
+
 
 // Process n samples per channel that are already on the device (channel c at
 // ptr + c * stride elements).
@@ -330,15 +359,37 @@ ss_status process_device(ss_plan_s* p, const void* ptr, long long n, long long s
     const float pref4b = (float)(nat ? 1.0 / (md * md) : 1.0 / ((md - 2) * (md - 3)));
     for (long long g0 = 0; g0 < Gn;) {
       long long take = std::min(gb, Gn - g0);
-      // sequential spectra: a batch ends where a block of seq_B groups ends
-      if (p->seq_B > 0) take = std::min(take, p->seq_B - (p->groups + g0) % p->seq_B);
+      // sequential spectra: a batch ends where a block of seq_B groups ends, or holds
+      // several whole blocks, whose sums the kernels keep apart (a block at a time was
+      // a dozen launches a block: 32 blocks of 64 groups at T = 128 took 3.8 ms)
+      int n_blocks = 0;
+      if (p->seq_B > 0) {
+        const long long in = (p->groups + g0) % p->seq_B;
+        const long long whole = std::min<long long>({take / p->seq_B, (Gn - g0) / p->seq_B,
+                                                     (long long)p->seq_set});
+        const bool kept_apart = p->k2_variant == kK2Warp84 &&
+                                (p->c4.empty() || p->gram32 || p->precision != SS_PREC_FP32);
+        if (in == 0 && whole >= 2 && p->d_blocks && kept_apart) {
+          n_blocks = (int)whole;
+          take = whole * p->seq_B;
+          SS_TRY(p, cudaMemsetAsync(p->d_blocks, 0, n_blocks * p->seq_stride * sizeof(double),
+                                    p->stream));
+        } else {
+          take = std::min(take, p->seq_B - in);
+        }
+      }
       const int cnt = (int)take;
+      const int bg = n_blocks ? p->seq_B : 0;  // groups of a block (0: one block)
+      const long long bs = n_blocks ? (long long)p->seq_stride : 0;
+      double* const acc2 = n_blocks ? p->d_blocks : p->d_acc2;
+      double* const acc3 = n_blocks ? p->d_blocks + p->n_acc2 : p->d_acc3;
+      double* const acc4 = n_blocks ? p->d_blocks + p->n_acc2 + p->n_acc3 : p->d_acc4;
       record(p, 0, p->stream, true);
       SS_TRY(p, launch_k1_spectra(src, g0 * per_group, cnt, p->C, p->T, p->m, p->M, p->Mp,
                                   p->d_win, p->d_tw,
                                   SpecRows{spec, chan_stride, p->Ms, p->mirror ? 1 : 0,
-                                           need_spec ? 1 : 0},
-                                  p->d_s2auto, p->d_acc2, (int)p->c2.size(), pref2, 4 * p->nsm, p->stream,
+                                           need_spec ? 1 : 0, n_blocks ? bg : kOneBlock, bs},
+                                  p->d_s2auto, acc2, (int)p->c2.size(), pref2, 4 * p->nsm, p->stream,
                                   p->oi, p->d_acc1, p->k1_mode));
       if (p->n_s2cross > 0)
         SS_TRY(p, launch_k1_cross_s2(spec, chan_stride, cnt, p->m, p->M, p->Ms,
@@ -354,29 +405,30 @@ ss_status process_device(ss_plan_s* p, const void* ptr, long long n, long long s
         // Independent warps: with few items the sub-tiles that hold isolated points are
         // taken as items too, which costs them less than the point kernel's launch
         // (T = 256, 409 groups: 8 sub-tiles instead of 6 and a launch of 7.5 us)
-        const bool all = warps && (long long)cnt * p->n_tiles3a <= 16ll * p->nsm * 4;
+        const bool all =
+            warps && (n_blocks || (long long)cnt * p->n_tiles3a <= 16ll * p->nsm * 4);
         if (warps)
           SS_TRY(p, launch_k2_bispec84w(p->tm32w, p->tm64w, row_stride, p->Z / 16, cnt, p->m,
                                         p->M, p->d_tiles3w, all ? p->n_tiles3a : p->n_tiles3w,
                                         p->d_c3, (int)p->c3.size(), p->C > 1 ? 1 : 0, pref3,
-                                        p->d_acc3, plane, combo_stride, 0, 0, p->nsm,
+                                        acc3, plane, combo_stride, bg, bs, p->nsm,
                                         p->d_counter, p->d_status, p->inject_timeout, p->stream));
         for (size_t i = 0; i < p->c3.size(); ++i) {
           const Combo& cb = p->c3[i];
-          double* acc3 = p->d_acc3 + (long long)i * combo_stride;
+          double* acc3i = acc3 + (long long)i * combo_stride;
           if (!warps)
             SS_TRY(p, launch_k2_bispec(p->tm64, p->tm128, spec + cb.c[0] * chan_stride,
                                        spec + cb.c[1] * chan_stride, spec + cb.c[2] * chan_stride,
                                        cb.c[0] * row_stride, cb.c[1] * row_stride,
                                        cb.c[2] * row_stride, cnt, p->m, p->FC, p->M, p->Ms,
-                                       p->d_tiles3, p->n_tiles3, p->C > 1 ? 1 : 0, pref3, acc3,
+                                       p->d_tiles3, p->n_tiles3, p->C > 1 ? 1 : 0, pref3, acc3i,
                                        plane, p->rows3, p->nsm, p->d_counter, p->d_status,
                                        p->inject_timeout, p->k2_variant, p->stream));
           const int2* pts = warps ? p->d_pts3w : p->d_pts3;
           const int npts = warps ? p->n_pts3w : p->n_pts3;
           if (p->C == 1 && npts > 0 && !all)
             SS_TRY(p, launch_k2_points(spec + cb.c[0] * chan_stride, p->Ms, cnt, p->m, pts, npts,
-                                       p->M, pref3, acc3, plane, p->stream));
+                                       p->M, pref3, acc3i, plane, p->stream));
         }
         record(p, 1, p->stream, false);
       }
@@ -406,7 +458,7 @@ ss_status process_device(ss_plan_s* p, const void* ptr, long long n, long long s
             SS_TRY(p, launch_k3_trispec_gram(
                           p->tm_g32, p->tm_g64, p->oi, cnt, p->m, p->M,
                           p->col4 ? p->M - 1 : p->M, p->d_tiles4g, p->n_tiles4g,
-                          p->d_acc4 + (long long)i * p->rows4 * p->M, plane, 0, 0, p->nsm,
+                          acc4 + (long long)i * p->rows4 * p->M, plane, bg, bs, p->nsm,
                           p->d_counter, p->d_status, p->stream));
           else if (p->precision == SS_PREC_FP32)
             SS_TRY(p, launch_k3_trispec(p->tm64, cb.c[0] * p->Gb_max * p->m, cnt, p->m, p->FC,
@@ -417,13 +469,14 @@ ss_status process_device(ss_plan_s* p, const void* ptr, long long n, long long s
             SS_TRY(p, launch_k3_trispec_tc(p->tm_img[cb.c[0]], p->oi, cb.c[0], cnt, p->m, p->M,
                                            p->Mp,
                                            p->d_tiles4tc, p->n_tiles4tc, p->precision,
-                                           p->d_acc4 + (long long)i * p->rows4 * p->M, plane,
+                                           acc4 + (long long)i * p->rows4 * p->M, plane, bg, bs,
                                            p->nsm, p->d_counter, p->d_status, p->stream));
           if (p->col4)
             SS_TRY(p, launch_k3_column(spec + cb.c[0] * chan_stride, p->Ms, cnt, p->m,
                                        p->M, pref4a, pref4b,
-                                       p->d_acc4 + (long long)i * p->rows4 * p->M, plane,
-                                       p->gram32 ? p->M : 1, p->gram32 ? 1 : p->M, p->stream));
+                                       acc4 + (long long)i * p->rows4 * p->M, plane,
+                                       p->gram32 ? p->M : 1, p->gram32 ? 1 : p->M, bg, bs,
+                                       p->stream));
         }
         record(p, 2, p->stream, false);
       }
@@ -440,7 +493,7 @@ ss_status process_device(ss_plan_s* p, const void* ptr, long long n, long long s
       }
       g0 += take;
       if (p->seq_B > 0 && (p->groups + g0) % p->seq_B == 0) {
-        ss_status st = emit_block(p);
+        ss_status st = n_blocks ? emit_blocks(p, n_blocks) : emit_block(p);
         if (st != SS_OK) return st;
       }
     }
@@ -551,11 +604,7 @@ ss_status process_host(ss_plan_s* p, const void* chunk, long long n) {
 }
 
 ss_status zero_state(ss_plan_s* p) {
-  if (p->d_status) SS_TRY(p, cudaMemsetAsync(p->d_status, 0, sizeof(int), p->stream));
-  if (p->d_acc1) SS_TRY(p, cudaMemsetAsync(p->d_acc1, 0, p->n_acc1 * sizeof(double), p->stream));
-  if (p->d_acc2) SS_TRY(p, cudaMemsetAsync(p->d_acc2, 0, p->n_acc2 * sizeof(double), p->stream));
-  if (p->d_acc3) SS_TRY(p, cudaMemsetAsync(p->d_acc3, 0, p->n_acc3 * sizeof(double), p->stream));
-  if (p->d_acc4) SS_TRY(p, cudaMemsetAsync(p->d_acc4, 0, p->n_acc4 * sizeof(double), p->stream));
+  if (p->d_sums) SS_TRY(p, cudaMemsetAsync(p->d_sums, 0, p->sums_bytes, p->stream));
   if (p->d_prev)
     SS_TRY(p, cudaMemsetAsync(p->d_prev, 0,
                               (p->n_acc2 + p->n_acc3 + p->n_acc4) * sizeof(double), p->stream));
@@ -810,10 +859,8 @@ void destroy(ss_plan_s* p) {
   cudaFree(p->oi.img);
   cudaFree(p->oi.rsc);
   cudaFree(p->oi.rmax);
-  cudaFree(p->d_acc1);
-  cudaFree(p->d_acc2);
-  cudaFree(p->d_acc3);
-  cudaFree(p->d_acc4);
+  cudaFree(p->d_sums);
+  cudaFree(p->d_blocks);
   cudaFree(p->d_s2auto);
   cudaFree(p->d_s2cross);
   cudaFree(p->d_tiles3);
@@ -825,8 +872,6 @@ void destroy(ss_plan_s* p) {
   cudaFree(p->d_tiles4);
   cudaFree(p->d_tiles4tc);
   cudaFree(p->d_c4cross);
-  cudaFree(p->d_status);
-  cudaFree(p->d_counter);
   cudaFree(p->d_out);
   cudaFree(p->d_prev);
   for (int o = 0; o < 3; ++o) {
@@ -1021,10 +1066,18 @@ static ss_status plan_create(ss_plan_t* out, int channels, int T, double dt, int
   p->n_acc2 = (size_t)kPlanes * p->c2.size() * p->M;
   p->n_acc3 = (size_t)kPlanes * p->c3.size() * p->rows3 * p->M;
   p->n_acc4 = (size_t)kPlanes * p->c4.size() * p->rows4 * p->M;
-  if (p->n_acc1) PLAN_TRY(dev_alloc(p, &p->d_acc1, p->n_acc1 * sizeof(double)));
-  if (p->n_acc2) PLAN_TRY(dev_alloc(p, &p->d_acc2, p->n_acc2 * sizeof(double)));
-  if (p->n_acc3) PLAN_TRY(dev_alloc(p, &p->d_acc3, p->n_acc3 * sizeof(double)));
-  if (p->n_acc4) PLAN_TRY(dev_alloc(p, &p->d_acc4, p->n_acc4 * sizeof(double)));
+  {
+    // orders 2 to 4 in a row (as in d_prev and d_blocks), then order 1, status, counter
+    const size_t n = p->n_acc2 + p->n_acc3 + p->n_acc4;
+    p->sums_bytes = (n + p->n_acc1) * sizeof(double) + 2 * sizeof(int);
+    PLAN_TRY(dev_alloc(p, &p->d_sums, p->sums_bytes));
+    if (p->n_acc2) p->d_acc2 = p->d_sums;
+    if (p->n_acc3) p->d_acc3 = p->d_sums + p->n_acc2;
+    if (p->n_acc4) p->d_acc4 = p->d_sums + p->n_acc2 + p->n_acc3;
+    if (p->n_acc1) p->d_acc1 = p->d_sums + n;
+    p->d_status = reinterpret_cast<int*>(p->d_sums + n + p->n_acc1);
+    p->d_counter = p->d_status + 1;
+  }
   if (!t3.empty()) PLAN_TRY(dev_alloc(p, &p->d_tiles3, t3.size() * sizeof(TileInfo)));
   if (!pts3.empty()) PLAN_TRY(dev_alloc(p, &p->d_pts3, pts3.size() * sizeof(int2)));
   if (!t3w.empty()) PLAN_TRY(dev_alloc(p, &p->d_tiles3w, t3w.size() * sizeof(TileInfo)));
@@ -1050,8 +1103,6 @@ static ss_status plan_create(ss_plan_t* out, int channels, int T, double dt, int
     PLAN_TRY(cudaMemcpy(p->d_c4cross, c4x.data(), c4x.size() * sizeof(int4),
                         cudaMemcpyHostToDevice));
   }
-  PLAN_TRY(dev_alloc(p, &p->d_status, sizeof(int)));
-  PLAN_TRY(dev_alloc(p, &p->d_counter, sizeof(int)));
   PLAN_TRY(cudaMemcpy(p->d_win, gw.data(), T * sizeof(float), cudaMemcpyHostToDevice));
   PLAN_TRY(cudaMemcpy(p->d_tw, tw.data(), T * sizeof(float2), cudaMemcpyHostToDevice));
   PLAN_TRY(cudaMemcpy(p->d_s2auto, s2auto.data(), channels * sizeof(int),
@@ -1295,6 +1346,13 @@ ss_status ss_set_sequential(ss_plan_t p, int block_groups, double* out, long lon
   p->seq_cap = block_groups > 0 ? max_blocks : 0;
   p->seq_blocks = 0;
   const size_t n = p->n_acc2 + p->n_acc3 + p->n_acc4;
+  if (block_groups > 0 && !p->d_blocks && n && p->C == 1 && p->n_s2cross == 0) {
+    // sums of a set of blocks that one batch computes: at most 256, 128 MB
+    const size_t fit = (128ull << 20) / (n * sizeof(double));
+    p->seq_set = (int)std::min<size_t>(256, fit);
+    p->seq_stride = n;
+    if (p->seq_set >= 2) SS_TRY(p, dev_alloc(p, &p->d_blocks, p->seq_set * n * sizeof(double)));
+  }
   if (block_groups > 0 && !p->d_prev && n) SS_TRY(p, dev_alloc(p, &p->d_prev, n * sizeof(double)));
   if (p->d_prev) SS_TRY(p, cudaMemsetAsync(p->d_prev, 0, n * sizeof(double), p->stream));
   return SS_OK;

@@ -37,6 +37,9 @@ struct ss_plan_s {
   int Z = 0, Ms = 0;
   bool mirror = false;
   int Gb_max = 0, Gb_user = 0;
+  // one allocation: the sums of orders 1 to 4, the status word and the queue counter
+  double* d_sums = nullptr;
+  size_t sums_bytes = 0;
   double *d_acc1 = nullptr, *d_acc2 = nullptr, *d_acc3 = nullptr, *d_acc4 = nullptr;
   size_t n_acc1 = 0, n_acc2 = 0, n_acc3 = 0, n_acc4 = 0;
   int estimator = SS_EST_UNBIASED;
@@ -61,6 +64,10 @@ struct ss_plan_s {
   double* seq_out = nullptr;
   long long seq_cap = 0, seq_blocks = 0;
   double* d_prev = nullptr;  // the S2/S3/S4 sums at the end of the last block
+  // sums of up to seq_set consecutive blocks of one batch (blocks seq_stride doubles apart)
+  double* d_blocks = nullptr;
+  int seq_set = 0;
+  size_t seq_stride = 0;
   // complex-valued signals (App. D) and shifted S4 planes (App. E): per order
   // (index order - 2) the operands of its combinations, their float64 sums, and
   // each record's order and place in the caller's record list
