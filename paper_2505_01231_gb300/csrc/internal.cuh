@@ -131,6 +131,27 @@ struct OperandImage {
 // groups with a warp per frame (kK1Warp, T <= 1024 and the group within 96 KB).
 enum { kK1Auto = 0, kK1Resident96 = 1, kK1Frames = 2, kK1Warp = 3, kK1Modes = 4 };
 
+// What a plan keeps between launches: the GPU's SM count, for each kernel whether its
+// function attributes are set and how many CTAs an SM holds of it with this plan's
+// shared memory (0: not asked yet), and how many items the plan's kernels have drawn
+// from its ticket counter since the last reset (the counter runs on, so a launch needs
+// no memset: its items are the tickets from there on).  A launch without one asks the
+// runtime each time.
+enum { kSlotK1Res74 = 0, kSlotK1Res96, kSlotK1Warp, kSlotK1Frames, kSlotK1Power, kSlotK1Fft,
+       kSlotK1Centre, kSlotK2Warp, kSlotGram, kSlotTc, kSlots };
+struct LaunchCache {
+  int nsm = 0;
+  int occ[kSlots] = {};
+  unsigned drawn = 0;
+};
+// Set a kernel's shared-memory attributes (one fixed limit per kernel, whatever launch
+// comes first) and find its resident CTAs per SM from its registers and shared memory
+// (the occupancy query reports fewer for some of these kernels than both limits allow),
+// at most max_ctas; both once per cache.
+cudaError_t prepare_kernel(const void* kern, int threads, size_t smem, size_t limit, int max_ctas,
+                           LaunchCache* lc, int slot, int* occ);
+cudaError_t sm_count(LaunchCache* lc, int* nsm);
+
 // Radix of the next pass of K1's Stockham transform with `rem` still to go (N = T/2 is
 // a power of two).
 __host__ __device__ inline int fft_radix(int rem) {
@@ -164,7 +185,7 @@ inline __host__ __device__ int twiddle_angle(int T, int i) {
 cudaError_t launch_k1_spectra(const SampleSource& src, long long sample0, int G, int C, int T,
                               int m, int M, int Mp, const float* win, const float2* tw,
                               const SpecRows& spec, const int* s2_auto, double* acc2, int n_s2,
-                              float pref2, int grid, cudaStream_t stream,
+                              float pref2, LaunchCache* lc, cudaStream_t stream,
                               const OperandImage& oi = OperandImage(), double* acc1 = nullptr,
                               int mode = kK1Auto);
 
@@ -208,7 +229,8 @@ cudaError_t launch_k3_trispec_gram(const CUtensorMap& tm32, const CUtensorMap& t
                                    const OperandImage& oi, int G, int m, int M, int lim,
                                    const TileInfo* tiles, int n_tiles, double* acc,
                                    long long plane, int block_groups, long long block_stride,
-                                   int nsm, int* counter, int* status, cudaStream_t stream);
+                                   LaunchCache* lc, unsigned* ticket, int* status,
+                                   cudaStream_t stream);
 
 // Tensor-core form of K3 (SS_PREC_TF32X3, SS_PREC_BF16X3, SS_PREC_BF16): tiles of
 // 128 x 128 (k, l) bins, the weighted frame-Gram contraction fed from K1's
@@ -220,7 +242,8 @@ cudaError_t launch_k3_trispec_tc(const CUtensorMap& tm_img, const OperandImage& 
                                  int G, int m, int M, int Mp,
                                  const TileInfo* tiles, int n_tiles, int precision, double* acc,
                                  long long plane, int block_groups, long long block_stride,
-                                 int nsm, int* counter, int* status, cudaStream_t stream);
+                                 LaunchCache* lc, unsigned* ticket, int* status,
+                                 cudaStream_t stream);
 size_t k3tc_smem_bytes(int precision);
 
 // K3 for several channels (FP32 CUDA cores): C4(a_k, b_k*, c_l, d_l*) of every
@@ -331,8 +354,9 @@ cudaError_t launch_k2_bispec84w(const CUtensorMap& tm32, const CUtensorMap& tm64
                                 int zblk, int G, int m, int M, const TileInfo* tiles, int n_tiles,
                                 const int4* combos, int n_combos, int cross, float pref3,
                                 double* acc, long long plane, long long combo_stride,
-                                int block_groups, long long block_stride, int nsm, int* counter,
-                                int* status, int inject_timeout, cudaStream_t stream);
+                                int block_groups, long long block_stride, LaunchCache* lc,
+                                unsigned* ticket, int* status, int inject_timeout,
+                                cudaStream_t stream);
 // K2 for isolated grid points of one channel (pts: n_pts (k, l) pairs)
 cudaError_t launch_k2_points(const float2* spec, int Mp, int G, int m, const int2* pts,
                              int n_pts, int M, float pref3, double* acc, long long plane,

@@ -727,13 +727,13 @@ k2_bispec84w(const __grid_constant__ CUtensorMap tm32, const __grid_constant__ C
   const uint32_t tsum = tmem_slot + ((uint32_t)(32 * warp) << 16);
   uint32_t qb = 0;  // stages this warp has consumed (stage = q % kSt84w)
   int next = 0;     // thread 0: the item after the current one, drawn while it runs
-  if (tid == 0) next = atomicAdd(wq.counter, 1);
+  if (tid == 0) next = draw_item(wq);
   for (;;) {
     if (tid == 0) s_next = next;
     __syncthreads();
     const int item = s_next;
     if (item >= wq.n_items) break;
-    if (tid == 0) next = atomicAdd(wq.counter, 1);
+    if (tid == 0) next = draw_item(wq);
     int rows;  // the warp's frames of the item, consecutive rows
     {
       const int per_chunk = wq.n_tiles * wq.n_combos;
@@ -1079,37 +1079,34 @@ cudaError_t launch_k2_bispec84w(const CUtensorMap& tm32, const CUtensorMap& tm64
                                 int zblk, int G, int m, int M, const TileInfo* tiles, int n_tiles,
                                 const int4* combos, int n_combos, int cross, float pref3,
                                 double* acc, long long plane, long long combo_stride,
-                                int block_groups, long long block_stride, int nsm, int* counter,
-                                int* status, int inject_timeout, cudaStream_t stream) {
+                                int block_groups, long long block_stride, LaunchCache* lc,
+                                unsigned* ticket, int* status, int inject_timeout,
+                                cudaStream_t stream) {
   if (G <= 0 || n_tiles <= 0 || n_combos <= 0) return cudaSuccess;
   WarpQueue wq;
-  wq.counter = counter;
+  wq.ticket = ticket;
+  wq.base = lc->drawn;
   wq.n_tiles = n_tiles;
   wq.n_combos = n_combos;
   if (block_groups <= 0 || block_groups > G) block_groups = G;
   wq.block_groups = block_groups;
   wq.block_stride = block_stride;
   const long long n_blocks = (G + block_groups - 1) / block_groups;
-  wq.group_chunk = warp_item_groups(block_groups, n_blocks * n_tiles * n_combos, nsm,
+  wq.group_chunk = warp_item_groups(block_groups, n_blocks * n_tiles * n_combos, lc->nsm,
                                     400.0 * m + 500.0, 4 * 1024);
   wq.chunks_per_block = (block_groups + wq.group_chunk - 1) / wq.group_chunk;
   const long long n_items = n_blocks * wq.chunks_per_block * n_tiles * n_combos;
   const size_t smem = (size_t)(kThreads84w / 32) * kRing84w + 1024;
-  cudaError_t e = cudaFuncSetAttribute(k2_bispec84w, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(k2_bispec84w, cudaFuncAttributePreferredSharedMemoryCarveout,
-                           cudaSharedmemCarveoutMaxShared);
-  if (e != cudaSuccess) return e;
   // TMEM: 128 columns per CTA, 512 per SM
   int occ = 1;
-  e = ctas_per_sm(k2_bispec84w, kThreads84w, smem, 4, &occ);
+  cudaError_t e = prepare_kernel((const void*)k2_bispec84w, kThreads84w, smem, smem, 4, lc,
+                                 kSlotK2Warp, &occ);
   if (e != cudaSuccess) return e;
+  const int nsm = lc->nsm;
   if (n_items > 0x7ffffff0ll - 4ll * nsm * occ) return cudaErrorInvalidValue;
   wq.n_items = (int)n_items;
   const int n_cta = (int)std::min<long long>((long long)nsm * occ, n_items);
-  e = cudaMemsetAsync(counter, 0, sizeof(int), stream);
-  if (e != cudaSuccess) return e;
+  lc->drawn += (unsigned)(n_items + n_cta);
   k2_bispec84w<<<n_cta, kThreads84w, smem, stream>>>(
       tm32, tm64w, m, M, G, zblk, tiles, combos, chan_rows, combo_stride, wq, cross, pref3, acc,
       plane, status, inject_timeout);

@@ -1280,40 +1280,6 @@ constexpr size_t k1_smem(int T, int C) {
 }
 constexpr size_t kK1MaxSmem = k1_smem(kMaxT, kMaxChannels);
 
-// The dynamic shared-memory limit of a kernel is an attribute of the function,
-// shared by every plan, stream and captured graph that launches it; each
-// kernel therefore gets one fixed limit, the largest amount any of its
-// launches can ask for, so that no launch depends on which launch set it last.
-template <typename Kern>
-cudaError_t set_smem_limit(Kern kern, size_t limit) {
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)limit);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
-                              cudaSharedmemCarveoutMaxShared);
-}
-
-// resident CTAs per SM of a K1 kernel with `smem` bytes of dynamic shared memory,
-// from its own registers and shared memory (one wave is launched)
-template <typename Kern>
-cudaError_t k1_occupancy(Kern kern, size_t smem, int* occ) {
-  int dev = 0, sm_smem = 0, sm_regs = 0, rsv = 0;
-  cudaFuncAttributes fa;
-  cudaError_t e = cudaFuncGetAttributes(&fa, kern);
-  if (e == cudaSuccess) e = cudaGetDevice(&dev);
-  if (e == cudaSuccess)
-    e = cudaDeviceGetAttribute(&sm_smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
-  if (e == cudaSuccess)
-    e = cudaDeviceGetAttribute(&sm_regs, cudaDevAttrMaxRegistersPerMultiprocessor, dev);
-  if (e == cudaSuccess)
-    e = cudaDeviceGetAttribute(&rsv, cudaDevAttrReservedSharedMemoryPerBlock, dev);
-  if (e != cudaSuccess) return e;
-  const int by_smem = sm_smem / (int)(smem + fa.sharedSizeBytes + rsv);
-  const int by_regs = sm_regs / std::max(1, ((fa.numRegs + 7) & ~7) * kThreadsK1);
-  *occ = std::max(1, std::min(std::min(by_smem, by_regs), 2048 / kThreadsK1));
-  return cudaSuccess;
-}
-
 // k1_centre keeps a group's columns of 256 bins in shared memory
 constexpr size_t kCentreMaxSmem = 160u << 10;
 
@@ -1322,16 +1288,15 @@ template <int DTYPE, bool kPower>
 cudaError_t launch_k1_fft(const SampleSource& src, long long sample0, int G, int C, int T, int m,
                           const float* win, const float2* tw, const SpecRows& spec,
                           const int* s2_auto, double* acc2, int n_s2, float pref2, double* acc1,
-                          int nsm, cudaStream_t stream) {
+                          LaunchCache* lc, int nsm, cudaStream_t stream) {
   auto kern = T == 1024   ? k1_fft<DTYPE, 512, kPower>
               : T == 2048 ? k1_fft<DTYPE, 1024, kPower>
                           : k1_fft<DTYPE, 2048, kPower>;
   const size_t smem = (size_t)(2 * kFftPoints + twiddle_count(T) + T / 2) * sizeof(float2);
-  cudaError_t e = set_smem_limit(
-      kern, (size_t)(2 * kFftPoints + twiddle_count(kMaxT) + kMaxT / 2) * sizeof(float2));
-  if (e != cudaSuccess) return e;
+  const size_t limit = (size_t)(2 * kFftPoints + twiddle_count(kMaxT) + kMaxT / 2) * sizeof(float2);
   int occ = 1;
-  e = k1_occupancy(kern, smem, &occ);
+  cudaError_t e = prepare_kernel((const void*)kern, kThreadsK1, smem, limit, 2048 / kThreadsK1, lc,
+                                 kPower ? kSlotK1Power : kSlotK1Fft, &occ);
   if (e != cudaSuccess) return e;
   const int FB = kFftPoints / (T / 2);
   const long long units = kPower ? G : ((long long)G * m + FB - 1) / FB;
@@ -1344,10 +1309,13 @@ cudaError_t launch_k1_fft(const SampleSource& src, long long sample0, int G, int
 template <int FMT>
 cudaError_t launch_k1_centre(int G, int C, int m, int M, int Mp, const SpecRows& spec,
                              const int* s2_auto, double* acc2, int n_s2, float pref2,
-                             const OperandImage& oi, double* acc1, int nsm, cudaStream_t stream) {
+                             const OperandImage& oi, double* acc1, LaunchCache* lc, int nsm,
+                             cudaStream_t stream) {
   const size_t smem = (size_t)m * kThreadsK1 * sizeof(float2);
   if (smem > kCentreMaxSmem) return cudaErrorInvalidValue;
-  cudaError_t e = set_smem_limit(k1_centre<FMT>, kCentreMaxSmem);
+  int occ = 1;
+  cudaError_t e = prepare_kernel((const void*)k1_centre<FMT>, kThreadsK1, smem, kCentreMaxSmem, 8, lc,
+                                 kSlotK1Centre, &occ);
   if (e != cudaSuccess) return e;
   const int bx = (Mp + kThreadsK1 - 1) / kThreadsK1;
   // about eight CTAs per SM, at most kMaxFp32Groups groups in a float32 sum
@@ -1364,7 +1332,7 @@ template <int DTYPE, int FMT>
 cudaError_t launch_k1_t(const SampleSource& src, long long sample0, int G, int C, int T, int m,
                         int M, int Mp, const float* win, const float2* tw, const SpecRows& spec,
                         const int* s2_auto, double* acc2, int n_s2,
-                        float pref2, const OperandImage& oi, int grid, size_t smem,
+                        float pref2, const OperandImage& oi, LaunchCache* lc, size_t smem,
                         cudaStream_t stream, double* acc1, int mode) {
   // a group whose coefficients fit beside a batch of FFT buffers stays resident
   const size_t fixed = (size_t)m * Mp * sizeof(float2) + (size_t)2 * C * M * sizeof(float) +
@@ -1377,16 +1345,14 @@ cudaError_t launch_k1_t(const SampleSource& src, long long sample0, int G, int C
   // shapes it does not take (T > 1024, or a group beyond 96 KB) use kK1Auto
   const size_t wsmem = fixed + (size_t)(kThreadsK1 / 32) * (T / 2) * sizeof(float2);
   if (mode == kK1Warp && (T > 1024 || wsmem > kK1ResidentBytes)) mode = kK1Auto;
+  int nsm = 1, occ = 1;
+  cudaError_t e = sm_count(lc, &nsm);
+  if (e != cudaSuccess) return e;
+  constexpr int kMaxCtas = 2048 / kThreadsK1;
   if (mode == kK1Warp) {
     auto kern = k1_spectra_warp<DTYPE, FMT>;
-    cudaError_t e = set_smem_limit(kern, kK1ResidentBytes);
-    if (e != cudaSuccess) return e;
-    int occ = 1;
-    e = k1_occupancy(kern, wsmem, &occ);
-    if (e != cudaSuccess) return e;
-    int dev = 0, nsm = 1;
-    e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    e = prepare_kernel((const void*)kern, kThreadsK1, wsmem, kK1ResidentBytes, kMaxCtas, lc,
+                       kSlotK1Warp, &occ);
     if (e != cudaSuccess) return e;
     const int rgrid = std::max(1, std::min(G, nsm * occ));
     kern<<<rgrid, kThreadsK1, wsmem, stream>>>(src, sample0, G, C, T, m, M, Mp, win, tw, spec,
@@ -1398,17 +1364,13 @@ cudaError_t launch_k1_t(const SampleSource& src, long long sample0, int G, int C
   if (T >= 1024 && (size_t)m * kThreadsK1 * sizeof(float2) <= kCentreMaxSmem) {
     const bool two = mode == kK1Frames || fixed + per_frame > kK1ResidentBytes;
     if (two || (!spec.store && mode == kK1Auto)) {
-      int dev = 0, nsm = 1;
-      cudaError_t e = cudaGetDevice(&dev);
-      if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-      if (e != cudaSuccess) return e;
       if (!spec.store)
         return launch_k1_fft<DTYPE, true>(src, sample0, G, C, T, m, win, tw, spec, s2_auto, acc2,
-                                          n_s2, pref2, acc1, nsm, stream);
+                                          n_s2, pref2, acc1, lc, nsm, stream);
       e = launch_k1_fft<DTYPE, false>(src, sample0, G, C, T, m, win, tw, spec, s2_auto, acc2, n_s2,
-                                      pref2, acc1, nsm, stream);
+                                      pref2, acc1, lc, nsm, stream);
       if (e != cudaSuccess) return e;
-      return launch_k1_centre<FMT>(G, C, m, M, Mp, spec, s2_auto, acc2, n_s2, pref2, oi, acc1, nsm,
+      return launch_k1_centre<FMT>(G, C, m, M, Mp, spec, s2_auto, acc2, n_s2, pref2, oi, acc1, lc, nsm,
                                    stream);
     }
   }
@@ -1421,25 +1383,10 @@ cudaError_t launch_k1_t(const SampleSource& src, long long sample0, int G, int C
     const size_t rsmem = fixed + (size_t)FB * per_frame;
     if (rsmem > kK1ResidentBytes) return cudaErrorInvalidValue;  // never: budget <= the limit
     auto kern = k1_spectra_res<DTYPE, FMT>;
-    cudaError_t e = set_smem_limit(kern, kK1ResidentBytes);
+    // one wave: as many CTAs as are resident at once
+    e = prepare_kernel((const void*)kern, kThreadsK1, rsmem, kK1ResidentBytes, kMaxCtas, lc,
+                       budget == kK1ResidentBytes3 ? kSlotK1Res74 : kSlotK1Res96, &occ);
     if (e != cudaSuccess) return e;
-    // one wave: as many CTAs as are resident at once, from the kernel's own
-    // registers and shared memory
-    int dev = 0, nsm = 1, sm_smem = 0, sm_regs = 0, rsv = 0;
-    cudaFuncAttributes fa;
-    e = cudaFuncGetAttributes(&fa, kern);
-    if (e == cudaSuccess) e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess)
-      e = cudaDeviceGetAttribute(&sm_smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
-    if (e == cudaSuccess)
-      e = cudaDeviceGetAttribute(&sm_regs, cudaDevAttrMaxRegistersPerMultiprocessor, dev);
-    if (e == cudaSuccess)
-      e = cudaDeviceGetAttribute(&rsv, cudaDevAttrReservedSharedMemoryPerBlock, dev);
-    if (e != cudaSuccess) return e;
-    const int by_smem = sm_smem / (int)(rsmem + fa.sharedSizeBytes + rsv);
-    const int by_regs = sm_regs / std::max(1, ((fa.numRegs + 7) & ~7) * kThreadsK1);
-    const int occ = std::max(1, std::min(std::min(by_smem, by_regs), 2048 / kThreadsK1));
     const int rgrid = std::max(1, std::min(G, nsm * occ));
     kern<<<rgrid, kThreadsK1, rsmem, stream>>>(
         src, sample0, G, C, T, m, M, Mp, FB, win, tw, spec, s2_auto, acc2, n_s2,
@@ -1447,25 +1394,25 @@ cudaError_t launch_k1_t(const SampleSource& src, long long sample0, int G, int C
     return cudaGetLastError();
   }
   if (smem > kK1MaxSmem) return cudaErrorInvalidValue;
-  cudaError_t e = set_smem_limit(k1_spectra<DTYPE, FMT>, kK1MaxSmem);
+  e = prepare_kernel((const void*)k1_spectra<DTYPE, FMT>, kThreadsK1, smem, kK1MaxSmem, kMaxCtas, lc,
+                     kSlotK1Frames, &occ);
   if (e != cudaSuccess) return e;
-  k1_spectra<DTYPE, FMT><<<grid, kThreadsK1, smem, stream>>>(src, sample0, G, C, T, m, M, Mp, win,
-                                                             tw, spec, s2_auto, acc2, n_s2, pref2, oi, acc1);
+  k1_spectra<DTYPE, FMT><<<std::min(G, 4 * nsm), kThreadsK1, smem, stream>>>(
+      src, sample0, G, C, T, m, M, Mp, win, tw, spec, s2_auto, acc2, n_s2, pref2, oi, acc1);
   return cudaGetLastError();
 }
 
 cudaError_t launch_k1_spectra(const SampleSource& src, long long sample0, int G, int C, int T,
                               int m, int M, int Mp, const float* win, const float2* tw,
                               const SpecRows& spec, const int* s2_auto,
-                              double* acc2, int n_s2, float pref2, int grid, cudaStream_t stream,
+                              double* acc2, int n_s2, float pref2, LaunchCache* lc, cudaStream_t stream,
                               const OperandImage& oi, double* acc1, int mode) {
   if (G <= 0) return cudaSuccess;
   if (mode < kK1Auto || mode >= kK1Modes) return cudaErrorInvalidValue;
   const size_t smem = k1_smem(T, C);
-  if (grid > G) grid = G;
   const bool f32 = src.dtype == SS_F32;
 #define K1_ARGS src, sample0, G, C, T, m, M, Mp, win, tw, spec, s2_auto, acc2, \
-                n_s2, pref2, oi, grid, smem, stream, acc1, mode
+                n_s2, pref2, oi, lc, smem, stream, acc1, mode
   switch (oi.fmt) {
     case kImageGramTF32:
       return f32 ? launch_k1_t<SS_F32, kImageGramTF32>(K1_ARGS)

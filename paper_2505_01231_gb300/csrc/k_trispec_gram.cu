@@ -156,13 +156,13 @@ k3_trispec_gram(const __grid_constant__ CUtensorMap tm32, const __grid_constant_
   const uint32_t tsum = tmem_slot + ((uint32_t)(32 * warp) << 16);
   uint32_t qb = 0;  // stages this warp has consumed (stage = q % kGSt)
   int next = 0;     // thread 0: the item after the current one, drawn while it runs
-  if (tid == 0) next = atomicAdd(wq.counter, 1);
+  if (tid == 0) next = draw_item(wq);
   for (;;) {
     if (tid == 0) s_next = next;
     __syncthreads();
     const int item = s_next;
     if (item >= wq.n_items) break;
-    if (tid == 0) next = atomicAdd(wq.counter, 1);
+    if (tid == 0) next = draw_item(wq);
     int nst;  // stages of the warp's groups, consecutive entry rows
     {
       const int chunk = item / wq.n_tiles, t = item - chunk * wq.n_tiles;
@@ -325,18 +325,21 @@ cudaError_t launch_k3_trispec_gram(const CUtensorMap& tm32, const CUtensorMap& t
                                    const OperandImage& oi, int G, int m, int M, int lim,
                                    const TileInfo* tiles, int n_tiles, double* acc,
                                    long long plane, int block_groups, long long block_stride,
-                                   int nsm, int* counter, int* status, cudaStream_t stream) {
+                                   LaunchCache* lc, unsigned* ticket, int* status,
+                                   cudaStream_t stream) {
   if (G <= 0 || n_tiles <= 0) return cudaSuccess;
   if (oi.fmt != kImageGramF32 || oi.rows % kGRows != 0) return cudaErrorInvalidValue;
   const size_t smem = (size_t)kGWarps * kGRing + 1024;
-  cudaError_t e = cudaFuncSetAttribute(k3_trispec_gram,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // four CTAs per SM: 128 registers a thread, 49 KB of shared memory and 128 TMEM
+  // columns each
+  int occ = 1;
+  cudaError_t e = prepare_kernel((const void*)k3_trispec_gram, kGThreads, smem, smem, 4, lc,
+                                 kSlotGram, &occ);
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(k3_trispec_gram, cudaFuncAttributePreferredSharedMemoryCarveout,
-                           cudaSharedmemCarveoutMaxShared);
-  if (e != cudaSuccess) return e;
+  const int nsm = lc->nsm;
   WarpQueue wq;
-  wq.counter = counter;
+  wq.ticket = ticket;
+  wq.base = lc->drawn;
   wq.n_tiles = n_tiles;
   wq.n_combos = 1;
   if (block_groups <= 0 || block_groups > G) block_groups = G;
@@ -348,15 +351,14 @@ cudaError_t launch_k3_trispec_gram(const CUtensorMap& tm32, const CUtensorMap& t
                                     100.0 * oi.rows + 500.0, 2 * 2048);
   wq.chunks_per_block = (block_groups + wq.group_chunk - 1) / wq.group_chunk;
   const long long n_items = n_blocks * wq.chunks_per_block * n_tiles;
-  // four CTAs per SM: 128 registers a thread, 49 KB of shared memory and 128 TMEM
-  // columns each
-  const long long slots = 4ll * nsm;
+  const long long slots = (long long)occ * nsm;
   if (n_items > 0x7ffffff0ll - slots) return cudaErrorInvalidValue;
   wq.n_items = (int)n_items;
-  e = cudaMemsetAsync(counter, 0, sizeof(int), stream);
-  if (e != cudaSuccess) return e;
-  k3_trispec_gram<<<(int)std::min(slots, n_items), kGThreads, smem, stream>>>(
-      tm32, tm64, oi.rows / kGRows, m * (m - 1) / 2 + 1, G, M, lim, tiles, wq, acc, plane, status);
+  const int n_cta = (int)std::min(slots, n_items);
+  lc->drawn += (unsigned)(n_items + n_cta);
+  k3_trispec_gram<<<n_cta, kGThreads, smem, stream>>>(tm32, tm64, oi.rows / kGRows,
+                                                      m * (m - 1) / 2 + 1, G, M, lim, tiles, wq,
+                                                      acc, plane, status);
   return cudaGetLastError();
 }
 

@@ -225,7 +225,7 @@ k3_trispec_tc(const __grid_constant__ CUtensorMap tm_img, const float* __restric
       uint32_t ph = 0;         // parity of stage s's current use
       bool ok = true;
       for (;;) {
-        const int item = atomicAdd(wq.counter, 1);
+        const int item = draw_item(wq);
         if (item >= wq.n_items || *(volatile int*)&s_fail) break;
         const int chunk = item / wq.n_tiles, t = item - chunk * wq.n_tiles;
         const int blk = chunk / wq.chunks_per_block;
@@ -490,8 +490,8 @@ int k3tc_stage_chunks(int precision) {
 cudaError_t launch_k3_trispec_tc(const CUtensorMap& tm_img, const OperandImage& oi, int channel,
                                  int G, int m, int M, int Mp, const TileInfo* tiles, int n_tiles,
                                  int precision, double* acc, long long plane, int block_groups,
-                                 long long block_stride, int nsm, int* counter, int* status,
-                                 cudaStream_t stream) {
+                                 long long block_stride, LaunchCache* lc, unsigned* ticket,
+                                 int* status, cudaStream_t stream) {
   if (G <= 0 || n_tiles <= 0) return cudaSuccess;
   if (m < 4 || m > kMaxGramM || (Mp & 15)) return cudaErrorInvalidValue;
   const size_t smem = k3tc_smem_bytes(precision);
@@ -499,12 +499,14 @@ cudaError_t launch_k3_trispec_tc(const CUtensorMap& tm_img, const OperandImage& 
               : precision == SS_PREC_BF16X3 ? k3_trispec_tc<kImageGramBF16, 3>
               : precision == SS_PREC_FP16X3 ? k3_trispec_tc<kImageGramF16, 3>
                                             : k3_trispec_tc<kImageGramBF16, 1>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
   // one CTA per SM: each CTA allocates all 512 TMEM columns
-  const int n_cta = nsm;
+  int occ = 1;
+  cudaError_t e = prepare_kernel((const void*)kern, kTcThreads, smem, smem, 1, lc, kSlotTc, &occ);
+  if (e != cudaSuccess) return e;
+  const int n_cta = lc->nsm;
   WarpQueue wq;
-  wq.counter = counter;
+  wq.ticket = ticket;
+  wq.base = lc->drawn;
   wq.n_tiles = n_tiles;
   wq.n_combos = 1;
   if (block_groups <= 0 || block_groups > G) block_groups = G;
@@ -514,8 +516,7 @@ cudaError_t launch_k3_trispec_tc(const CUtensorMap& tm_img, const OperandImage& 
   wq.group_chunk = std::min(block_groups, work_group_chunk(G, n_tiles, n_cta));
   wq.chunks_per_block = (block_groups + wq.group_chunk - 1) / wq.group_chunk;
   wq.n_items = n_tiles * wq.chunks_per_block * n_blocks;
-  e = cudaMemsetAsync(counter, 0, sizeof(int), stream);
-  if (e != cudaSuccess) return e;
+  lc->drawn += (unsigned)(wq.n_items + n_cta);
   const float* rsc = oi.rsc ? oi.rsc + (size_t)channel * oi.chan_rsc : nullptr;
   kern<<<n_cta, kTcThreads, smem, stream>>>(tm_img, rsc, G, oi.nkc, oi.ndc, M, Mp,
                                             tiles, wq, acc, plane, status);

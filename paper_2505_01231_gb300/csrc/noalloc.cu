@@ -51,39 +51,51 @@ bool on_device(const void* ptr) {
 }
 
 // The window scaled by 1/sqrt(sum g^2) and the twiddles of K1's passes, built on
-// the device in float64 (the same definitions ss_plan evaluates on the host), so
-// that a call enqueues kernels and memsets only.  One block.
-constexpr int kTableThreads = 256;
+// the device in float64 (the same definitions ss_plan evaluates on the host), and the
+// cleared sums and combination index, so that a call enqueues kernels only.  A thread an
+// entry over many small blocks: an SM does two float64 operations a clock, and one block
+// took 11 us at T = 256, more than the rest of the call's kernels.  Hann: sum g^2 =
+// 3 T / 8; the confined Gaussian's sum goes through the blocks' partial sums and k0_scale.
+constexpr int kTableThreads = 64;
 
 __global__ void __launch_bounds__(kTableThreads)
-k0_tables(int T, int window, double sigma, float* __restrict__ win, float2* __restrict__ tw) {
-  __shared__ double red[kTableThreads];
-  auto g_at = [&](int i) {
-    if (window == SS_WIN_HANN) return 0.5 - 0.5 * cospi(2.0 * i / T);
+k0_tables(int T, int window, double sigma, float* __restrict__ win, float2* __restrict__ tw,
+          double* __restrict__ g, double* __restrict__ part, double* __restrict__ acc, int n_acc,
+          int* __restrict__ s2_auto) {
+  const int i = blockIdx.x * kTableThreads + threadIdx.x;
+  for (int a = i; a < n_acc; a += gridDim.x * kTableThreads) acc[a] = 0.0;
+  if (i == 0) *s2_auto = 0;
+  if (i < twiddle_count(T)) {
+    double sn, cs;
+    sincospi(2.0 * twiddle_angle(T, i) / T, &sn, &cs);
+    tw[i] = make_float2((float)cs, (float)sn);
+  }
+  if (window == SS_WIN_HANN) {
+    if (i < T) win[i] = (float)((0.5 - 0.5 * cospi(2.0 * i / T)) / sqrt(0.375 * T));
+    return;
+  }
+  double sq = 0.0;
+  if (i < T) {
     const double N = T, c = (N - 1.0) / 2.0, d = 4.0 * N * N * sigma * sigma;
     auto G = [&](double x) { return exp(-(x - c) * (x - c) / d); };
-    return G(i) - G(-0.5) * (G(i + N) + G(i - N)) / (G(-0.5 + N) + G(-0.5 - N));
-  };
-  double s = 0.0;
-  for (int i = threadIdx.x; i < T; i += kTableThreads) {
-    const double g = g_at(i);
-    s += g * g;
+    const double v = G(i) - G(-0.5) * (G(i + N) + G(i - N)) / (G(-0.5 + N) + G(-0.5 - N));
+    g[i] = v;
+    sq = v * v;
   }
-  red[threadIdx.x] = s;
+  __shared__ double red[kTableThreads / 32];
+  for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = sq;
   __syncthreads();
-  for (int h = kTableThreads / 2; h > 0; h >>= 1) {
-    if (threadIdx.x < h) red[threadIdx.x] += red[threadIdx.x + h];
-    __syncthreads();
-  }
-  const double scale = 1.0 / sqrt(red[0]);
-  for (int i = threadIdx.x; i < T; i += kTableThreads) {
-    win[i] = (float)(g_at(i) * scale);
-    if (i < twiddle_count(T)) {
-      double sn, cs;
-      sincospi(2.0 * twiddle_angle(T, i) / T, &sn, &cs);
-      tw[i] = make_float2((float)cs, (float)sn);
-    }
-  }
+  if (threadIdx.x == 0) part[blockIdx.x] = red[0] + red[1];
+}
+
+__global__ void __launch_bounds__(kTableThreads)
+k0_scale(int T, const double* __restrict__ g, const double* __restrict__ part, int n_part,
+         float* __restrict__ win) {
+  double s = 0.0;
+  for (int b = 0; b < n_part; ++b) s += part[b];
+  const int i = blockIdx.x * kTableThreads + threadIdx.x;
+  if (i < T) win[i] = (float)(g[i] / sqrt(s));
 }
 
 }  // namespace
@@ -146,13 +158,17 @@ extern "C" ss_status ss_s2_noalloc(const float* d_signal, size_t n_samples, int 
     cudaError_t e_ = (call);                                                           \
     if (e_ != cudaSuccess) return fail(SS_ECUDA, std::string(#call) + ": " + cudaGetErrorString(e_)); \
   } while (0)
-  k0_tables<<<1, kTableThreads, 0, s>>>(T, window, win_param, d_win, d_tw);
+  // the spectra's part of the array holds the confined Gaussian until it is scaled
+  double* d_g = reinterpret_cast<double*>(base + kSpecOff);
+  double* d_part = d_g + 4096;
+  const int nb = (T + kTableThreads - 1) / kTableThreads;
+  k0_tables<<<nb, kTableThreads, 0, s>>>(T, window, win_param, d_win, d_tw, d_g, d_part, d_acc, 4 * M,
+                                         d_auto);
   NA_TRY(cudaGetLastError());
-  // the array keeps the previous call's contents: clear the sums and the index
-  NA_TRY(cudaMemsetAsync(d_acc, 0, (size_t)4 * M * sizeof(double), s));
-  NA_TRY(cudaMemsetAsync(d_auto, 0, sizeof(int), s));
-  int nsm = 1;
-  NA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+  if (window != SS_WIN_HANN) {
+    k0_scale<<<nb, kTableThreads, 0, s>>>(T, d_g, d_part, nb, d_win);
+    NA_TRY(cudaGetLastError());
+  }
   SampleSource src;
   src.carry = nullptr;
   src.carry_n = 0;
@@ -161,8 +177,8 @@ extern "C" ss_status ss_s2_noalloc(const float* d_signal, size_t n_samples, int 
   src.chunk_stride = (long long)n_samples;
   src.dtype = SS_F32;
   NA_TRY(launch_k1_spectra(src, 0, (int)G, 1, T, m, M, Mp, d_win, d_tw,
-                           SpecRows{d_spec, (long long)G * m * Mp, Mp, 0, 0, kOneBlock, 0}, d_auto, d_acc, 1, 1.0f / (float)(m - 1),
-                           4 * nsm, s));
+                           SpecRows{d_spec, (long long)G * m * Mp, Mp, 0, 0, kOneBlock, 0}, d_auto,
+                           d_acc, 1, 1.0f / (float)(m - 1), nullptr, s));
   NA_TRY(launch_k4_finalize(d_acc, 1, 1, M, kLayoutVector, G, dt, d_S2, d_S2_err, s));
 #undef NA_TRY
   g_err.clear();

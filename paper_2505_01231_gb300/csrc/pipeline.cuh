@@ -156,11 +156,18 @@ struct WorkQueue {
 // block_groups groups (one block unless the spectra of consecutive blocks are kept
 // apart); a block has chunks_per_block chunks of group_chunk groups, the last one
 // shorter, and its sums start block_stride doubles after those of the block before.
+// An item is the ticket drawn minus `base`; every CTA draws until its first ticket past
+// the items, so a launch draws n_items + CTAs of them.
 struct WarpQueue {
-  int* counter;
+  unsigned* ticket;
+  unsigned base;
   int n_tiles, n_combos, group_chunk, n_items, block_groups, chunks_per_block;
   long long block_stride;
 };
+
+__device__ __forceinline__ int draw_item(const WarpQueue& q) {
+  return (int)(atomicAdd(q.ticket, 1u) - q.base);
+}
 
 // Returns the next item for the calling CTA (all threads receive it) or -1.
 __device__ __forceinline__ int next_item(const WorkQueue& q, int* s_slot) {

@@ -389,7 +389,7 @@ ss_status process_device(ss_plan_s* p, const void* ptr, long long n, long long s
                                   p->d_win, p->d_tw,
                                   SpecRows{spec, chan_stride, p->Ms, p->mirror ? 1 : 0,
                                            need_spec ? 1 : 0, n_blocks ? bg : kOneBlock, bs},
-                                  p->d_s2auto, acc2, (int)p->c2.size(), pref2, 4 * p->nsm, p->stream,
+                                  p->d_s2auto, acc2, (int)p->c2.size(), pref2, &p->cache, p->stream,
                                   p->oi, p->d_acc1, p->k1_mode));
       if (p->n_s2cross > 0)
         SS_TRY(p, launch_k1_cross_s2(spec, chan_stride, cnt, p->m, p->M, p->Ms,
@@ -411,8 +411,8 @@ ss_status process_device(ss_plan_s* p, const void* ptr, long long n, long long s
           SS_TRY(p, launch_k2_bispec84w(p->tm32w, p->tm64w, row_stride, p->Z / 16, cnt, p->m,
                                         p->M, p->d_tiles3w, all ? p->n_tiles3a : p->n_tiles3w,
                                         p->d_c3, (int)p->c3.size(), p->C > 1 ? 1 : 0, pref3,
-                                        acc3, plane, combo_stride, bg, bs, p->nsm,
-                                        p->d_counter, p->d_status, p->inject_timeout, p->stream));
+                                        acc3, plane, combo_stride, bg, bs, &p->cache,
+                                        p->d_ticket, p->d_status, p->inject_timeout, p->stream));
         for (size_t i = 0; i < p->c3.size(); ++i) {
           const Combo& cb = p->c3[i];
           double* acc3i = acc3 + (long long)i * combo_stride;
@@ -458,8 +458,8 @@ ss_status process_device(ss_plan_s* p, const void* ptr, long long n, long long s
             SS_TRY(p, launch_k3_trispec_gram(
                           p->tm_g32, p->tm_g64, p->oi, cnt, p->m, p->M,
                           p->col4 ? p->M - 1 : p->M, p->d_tiles4g, p->n_tiles4g,
-                          acc4 + (long long)i * p->rows4 * p->M, plane, bg, bs, p->nsm,
-                          p->d_counter, p->d_status, p->stream));
+                          acc4 + (long long)i * p->rows4 * p->M, plane, bg, bs, &p->cache,
+                          p->d_ticket, p->d_status, p->stream));
           else if (p->precision == SS_PREC_FP32)
             SS_TRY(p, launch_k3_trispec(p->tm64, cb.c[0] * p->Gb_max * p->m, cnt, p->m, p->FC,
                                         p->M, p->d_tiles4, p->n_tiles4, pref4a, pref4b,
@@ -470,7 +470,7 @@ ss_status process_device(ss_plan_s* p, const void* ptr, long long n, long long s
                                            p->Mp,
                                            p->d_tiles4tc, p->n_tiles4tc, p->precision,
                                            acc4 + (long long)i * p->rows4 * p->M, plane, bg, bs,
-                                           p->nsm, p->d_counter, p->d_status, p->stream));
+                                           &p->cache, p->d_ticket, p->d_status, p->stream));
           if (p->col4)
             SS_TRY(p, launch_k3_column(spec + cb.c[0] * chan_stride, p->Ms, cnt, p->m,
                                        p->M, pref4a, pref4b,
@@ -523,16 +523,15 @@ ss_status process_device(ss_plan_s* p, const void* ptr, long long n, long long s
 // A kernel whose bounded wait gave up leaves a non-zero device status; the
 // sums of that launch are incomplete, so the plan is marked unusable.
 ss_status check_status(ss_plan_s* p) {
-  int st = 0;
-  if (p->shadow) {
-    SS_TRY(p, cudaMemcpy(&st, p->shadow->d_status, sizeof(int), cudaMemcpyDeviceToHost));
-    if (st != kStatusOk) {
-      p->broken = true;
-      return fail(p, SS_ETIMEOUT, "a device-side wait for staged data gave up; results discarded");
-    }
-  }
-  SS_TRY(p, cudaMemcpy(&st, p->d_status, sizeof(int), cudaMemcpyDeviceToHost));
-  if (st != kStatusOk) {
+  // in the plan's stream after its kernels; the copies to pageable memory return when
+  // they are done, so they are also what the caller waits for
+  int st[2] = {kStatusOk, kStatusOk};
+  if (p->shadow)
+    SS_TRY(p, cudaMemcpyAsync(&st[1], p->shadow->d_status, sizeof(int), cudaMemcpyDeviceToHost,
+                              p->stream));
+  SS_TRY(p, cudaMemcpyAsync(&st[0], p->d_status, sizeof(int), cudaMemcpyDeviceToHost, p->stream));
+  SS_TRY(p, cudaStreamSynchronize(p->stream));
+  if (st[0] != kStatusOk || st[1] != kStatusOk) {
     p->broken = true;
     return fail(p, SS_ETIMEOUT, "a device-side wait for staged data gave up; results discarded");
   }
@@ -605,6 +604,7 @@ ss_status process_host(ss_plan_s* p, const void* chunk, long long n) {
 
 ss_status zero_state(ss_plan_s* p) {
   if (p->d_sums) SS_TRY(p, cudaMemsetAsync(p->d_sums, 0, p->sums_bytes, p->stream));
+  p->cache.drawn = 0;  // the ticket counter is among the sums
   if (p->d_prev)
     SS_TRY(p, cudaMemsetAsync(p->d_prev, 0,
                               (p->n_acc2 + p->n_acc3 + p->n_acc4) * sizeof(double), p->stream));
@@ -981,6 +981,7 @@ static ss_status plan_create(ss_plan_t* out, int channels, int T, double dt, int
     return st;
   }
   cudaDeviceGetAttribute(&p->nsm, cudaDevAttrMultiProcessorCount, p->device);
+  p->cache.nsm = p->nsm;
 
   // window (Eq. 17 / App. B) and its power sums, in float64
   std::vector<double> g(T);
@@ -1067,9 +1068,9 @@ static ss_status plan_create(ss_plan_t* out, int channels, int T, double dt, int
   p->n_acc3 = (size_t)kPlanes * p->c3.size() * p->rows3 * p->M;
   p->n_acc4 = (size_t)kPlanes * p->c4.size() * p->rows4 * p->M;
   {
-    // orders 2 to 4 in a row (as in d_prev and d_blocks), then order 1, status, counter
+    // orders 2 to 4 in a row (as in d_prev and d_blocks), then order 1, status, counters
     const size_t n = p->n_acc2 + p->n_acc3 + p->n_acc4;
-    p->sums_bytes = (n + p->n_acc1) * sizeof(double) + 2 * sizeof(int);
+    p->sums_bytes = (n + p->n_acc1) * sizeof(double) + 4 * sizeof(int);
     PLAN_TRY(dev_alloc(p, &p->d_sums, p->sums_bytes));
     if (p->n_acc2) p->d_acc2 = p->d_sums;
     if (p->n_acc3) p->d_acc3 = p->d_sums + p->n_acc2;
@@ -1077,6 +1078,7 @@ static ss_status plan_create(ss_plan_t* out, int channels, int T, double dt, int
     if (p->n_acc1) p->d_acc1 = p->d_sums + n;
     p->d_status = reinterpret_cast<int*>(p->d_sums + n + p->n_acc1);
     p->d_counter = p->d_status + 1;
+    p->d_ticket = reinterpret_cast<unsigned*>(p->d_status + 2);
   }
   if (!t3.empty()) PLAN_TRY(dev_alloc(p, &p->d_tiles3, t3.size() * sizeof(TileInfo)));
   if (!pts3.empty()) PLAN_TRY(dev_alloc(p, &p->d_pts3, pts3.size() * sizeof(int2)));
@@ -1288,7 +1290,6 @@ ss_status ss_finalize(ss_plan_t p, double* S2, double* S3, double* S4, double* S
   DeviceGuard guard(p->device);
   ss_status st = finalize_launch(p, S2, S3, S4, S2_err, S3_err, S4_err);
   if (st != SS_OK) return st;
-  SS_TRY(p, cudaStreamSynchronize(p->stream));
   return check_status(p);
 }
 
@@ -1312,7 +1313,6 @@ ss_status ss_finalize_s1(ss_plan_t p, double* S1, double* S1_err) {
   if (S1) SS_TRY(p, cudaMemcpyAsync(S1, o1, n1 * sizeof(double), cudaMemcpyDefault, p->stream));
   if (S1_err)
     SS_TRY(p, cudaMemcpyAsync(S1_err, e1, n1 * sizeof(double), cudaMemcpyDefault, p->stream));
-  SS_TRY(p, cudaStreamSynchronize(p->stream));
   return check_status(p);
 }
 
@@ -1477,7 +1477,6 @@ ss_status ss_finalize_complex(ss_plan_t p, double* S, double* S_err) {
     ++seen[i];
     out_off += per;
   }
-  SS_TRY(p, cudaStreamSynchronize(p->stream));
   return check_status(p);
 }
 

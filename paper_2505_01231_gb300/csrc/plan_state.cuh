@@ -78,6 +78,8 @@ struct ss_plan_s {
   std::vector<int> cx_order;  // order of each record, in the caller's order
   int cx_shift = 0;
   int* d_counter = nullptr;        // work-queue counter of the pair kernels
+  unsigned* d_ticket = nullptr;    // and of the kernels that take tickets (LaunchCache)
+  ss::LaunchCache cache;
   int FC = 0;                      // frames per staged chunk of the pair kernels
   CUtensorMap tm64{}, tm128{}, tm48{};  // 3-D views [rows = C*Gb_max*m][Mp/16][16] of the spectra
   CUtensorMap tm32w{}, tm64w{};          // the same with boxes of kFrames84w rows (k2_bispec84w)
