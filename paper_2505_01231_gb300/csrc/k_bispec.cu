@@ -328,7 +328,7 @@ k2_bispec(const __grid_constant__ CUtensorMap tm64, const __grid_constant__ CUte
       for (int q = 0; q < 16; ++q) {
         const int k = k0 + kt + (q >> 2), l = l0 + lt + (q & 3);
         if (in_domain3(k, l, M, cross))
-          atomicAdd(dst + (long long)(k + koff) * M + l, (double)t[q]);
+          atomicAdd(dst + (long long)(k + koff) * M + l, widen(t[q]));
         z[q] = 0.f;
       }
       tmem_st16(tsum + 16 * part, z);
@@ -619,7 +619,7 @@ k2_bispec84(const __grid_constant__ CUtensorMap tm64, const __grid_constant__ CU
       for (int q = 0; q < 32; ++q) {
         const int k = k0 + kt + (q >> 2), l = l0 + lt + (q & 3);
         if (in_domain3(k, l, M, cross))
-          atomicAdd(dst + (long long)(k + koff) * M + l, (double)tt[q]);
+          atomicAdd(dst + (long long)(k + koff) * M + l, widen(tt[q]));
         z[q] = 0.f;
       }
       tmem_st32(tsum + 32 * part, z);
@@ -654,15 +654,15 @@ k2_bispec84(const __grid_constant__ CUtensorMap tm64, const __grid_constant__ CU
 //
 // At an item's end the four warps' float32 sums meet in shared memory (the warps'
 // rings, free by then; 32 x 32 floats a warp and part, chunk XOR keeps the exchange
-// free of bank conflicts), are added in float64 and go to the accumulators a row of
-// 32 consecutive doubles per warp instruction.  What this is for is the number of
-// float64 atomics, of which the L2 takes about 200 a clock: an item's 4096 cost as
-// much as 1.4 groups of m = 10 frames of one warp.  With an item per warp instead
-// (each flushing its own sums), T = 1024, m = 10: 6.95 ms for 2^28 samples, 0.93 ms
-// for 2^25; now 6.75 and 0.88 ms.  2^20 samples at T = 256: 0.099 ms with 64 x 64
-// tiles, one group an item, and now 0.033 ms.  Four channels, 2^21 samples, T = 512,
-// m = 20, 20 combinations: 10.5 ms in 20 launches of 64 x 64 tiles (the half with
-// negative bins staged by the threads), now 3.3 ms.
+// free of bank conflicts), are added up (widen_sum4) and go to the accumulators a row of
+// 32 consecutive doubles per warp instruction.  That cuts the ends' cost, float64 most of
+// all: an item per warp with 4096 conversions on the float64 pipe (two a clock and SM) and
+// as many atomics cost as much as 1.4 groups of m = 10 frames of one warp.  T = 1024, m =
+// 10: 6.95 ms for 2^28 samples and 0.93 ms for 2^25 with an item per warp, now 6.60 and
+// 0.88 ms (K2 alone).  2^20 samples at T = 256: 0.099 ms with 64 x 64 tiles, one group an
+// item, and now 0.033 ms.  Four channels, 2^21 samples, T = 512, m = 20, 20 combinations:
+// 10.5 ms in 20 launches of 64 x 64 tiles (the half with negative bins staged by the
+// threads), now 3.2 ms.
 constexpr int kThreads84w = 128;
 constexpr int kFS84w = kFrames84w;  // frames per stage
 constexpr int kSt84w = 3;   // stages per warp
@@ -907,10 +907,11 @@ k2_bispec84w(const __grid_constant__ CUtensorMap tm32, const __grid_constant__ C
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
         const int r = 8 * warp + i;
-        double v = 0.0;
-#pragma unroll
-        for (int w = 0; w < 4; ++w) v += (double)col[w * (kRing84w / 4) + r * 32];
-        if (in_domain3(k0 + r, l, M, cross)) atomicAdd(dst + (long long)r * M, v);
+        const float* c = col + r * 32;
+        if (in_domain3(k0 + r, l, M, cross))
+          atomicAdd(dst + (long long)r * M,
+                    widen_sum4(c[0], c[kRing84w / 4], c[2 * (kRing84w / 4)], c[3 * (kRing84w / 4)],
+                               wq.group_chunk <= 4));
       }
       __syncthreads();
     }

@@ -72,10 +72,10 @@ __device__ __forceinline__ float2 operand(const float2* __restrict__ spec, long 
 
 __device__ __forceinline__ void flush4(double* __restrict__ acc, long long plane, long long o,
                                        float sr, float si, float qr, float qi) {
-  atomicAdd(acc + o, (double)sr);
-  atomicAdd(acc + plane + o, (double)si);
-  atomicAdd(acc + 2 * plane + o, (double)qr);
-  atomicAdd(acc + 3 * plane + o, (double)qi);
+  atomicAdd(acc + o, widen(sr));
+  atomicAdd(acc + plane + o, widen(si));
+  atomicAdd(acc + 2 * plane + o, widen(qr));
+  atomicAdd(acc + 3 * plane + o, widen(qi));
 }
 
 // S2: thread = (bin, combination), blockIdx.y = run of groups

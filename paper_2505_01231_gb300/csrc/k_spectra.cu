@@ -325,8 +325,8 @@ __device__ __forceinline__ void flush_k1_sums(int C, int M, const int* __restric
     const int ia = s2_auto[c];
     if (ia < 0) continue;
     for (int k = threadIdx.x; k < M; k += blockDim.x) {
-      atomicAdd(acc2 + 0 * plane + (long long)ia * M + k, (double)s2sum[c * M + k]);
-      atomicAdd(acc2 + 2 * plane + (long long)ia * M + k, (double)s2sq[c * M + k]);
+      atomicAdd(acc2 + 0 * plane + (long long)ia * M + k, widen(s2sum[c * M + k]));
+      atomicAdd(acc2 + 2 * plane + (long long)ia * M + k, widen(s2sq[c * M + k]));
       s2sum[c * M + k] = 0.f;
       s2sq[c * M + k] = 0.f;
     }
@@ -334,7 +334,7 @@ __device__ __forceinline__ void flush_k1_sums(int C, int M, const int* __restric
   if (threadIdx.x == 0)
     for (int c = 0; c < C; ++c)
       for (int q = 0; q < 4; ++q) {
-        if (acc1) atomicAdd(acc1 + q * C + c, (double)s1s[c][q]);
+        if (acc1) atomicAdd(acc1 + q * C + c, widen(s1s[c][q]));
         s1s[c][q] = 0.f;
       }
 }
@@ -1100,8 +1100,8 @@ k1_fft(SampleSource src, long long sample0, int G, int m, const float* __restric
       double* dst = acc2 + blk * sp.block_stride + (long long)ia * M;
       auto put = [&](int k, float a, float b) {
         if (ia < 0) return;
-        atomicAdd(dst + k, (double)a);
-        atomicAdd(dst + 2 * plane + k, (double)b);
+        atomicAdd(dst + k, widen(a));
+        atomicAdd(dst + 2 * plane + k, widen(b));
       };
 #pragma unroll
       for (int s = 0; s < kSlots; ++s) {
@@ -1112,7 +1112,7 @@ k1_fft(SampleSource src, long long sample0, int G, int m, const float* __restric
       if (tid == 0) {
         put(N / 2, sum[2 * kSlots], sq[2 * kSlots]);
         for (int q = 0; q < 4; ++q) {
-          if (acc1) atomicAdd(acc1 + q * C + c, (double)s1[q]);
+          if (acc1) atomicAdd(acc1 + q * C + c, widen(s1[q]));
           s1[q] = 0.f;
         }
       }
@@ -1209,8 +1209,8 @@ k1_centre(int G, int m, int M, int Mp, int groups_per_cta, SpecRows sp,
   auto flush = [&]() {
     if (k >= M || ia < 0) return;
     double* dst = acc2 + cur * sp.block_stride + (long long)ia * M + k;
-    atomicAdd(dst, (double)sum);
-    atomicAdd(dst + 2 * (long long)n_s2 * M, (double)sq);
+    atomicAdd(dst, widen(sum));
+    atomicAdd(dst + 2 * (long long)n_s2 * M, widen(sq));
     sum = sq = 0.f;
   };
   for (int g = g0; g < g1; ++g) {
@@ -1231,7 +1231,7 @@ k1_centre(int G, int m, int M, int Mp, int groups_per_cta, SpecRows sp,
   }
   flush();
   if (k == 0 && acc1)
-    for (int q = 0; q < 4; ++q) atomicAdd(acc1 + q * C + c, (double)s1[q]);
+    for (int q = 0; q < 4; ++q) atomicAdd(acc1 + q * C + c, widen(s1[q]));
 }
 
 // Cross-channel S2 (Sec. 7, Eq. 47): c2(a_k, b_k*) = 1/(m-1) sum_j da_jk db_jk*
@@ -1264,10 +1264,10 @@ __global__ void k1_cross_s2(const float2* __restrict__ spec, long long chan_stri
     qi = fmaf(ci, ci, qi);
   }
   const long long o = (long long)pr.z * M + k;
-  atomicAdd(acc2 + o, (double)sr);
-  atomicAdd(acc2 + plane + o, (double)si);
-  atomicAdd(acc2 + 2 * plane + o, (double)qr);
-  atomicAdd(acc2 + 3 * plane + o, (double)qi);
+  atomicAdd(acc2 + o, widen(sr));
+  atomicAdd(acc2 + plane + o, widen(si));
+  atomicAdd(acc2 + 2 * plane + o, widen(qr));
+  atomicAdd(acc2 + 3 * plane + o, widen(qi));
 }
 
 }  // namespace

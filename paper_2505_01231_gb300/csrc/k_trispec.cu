@@ -186,8 +186,8 @@ k3_trispec(const __grid_constant__ CUtensorMap tm64, int row0, int G, int m, int
         const int k = k0 + kt + a, l = l0 + lt + b;
         if (k > l || l >= M) continue;
         const long long o = (long long)k * M + l;
-        atomicAdd(acc + o, (double)sum[a * 4 + b]);
-        atomicAdd(acc + 2 * plane + o, (double)sq[a * 4 + b]);
+        atomicAdd(acc + o, widen(sum[a * 4 + b]));
+        atomicAdd(acc + 2 * plane + o, widen(sq[a * 4 + b]));
       }
     }
   }
@@ -265,8 +265,8 @@ k3_column(const float2* __restrict__ spec, int Mp, int G, int m, int M, float pr
     sq = fmaf(c4, c4, sq);
   }
   const long long o = blockIdx.z * block_stride + (long long)l * sl_out + (long long)k * sk_out;
-  atomicAdd(acc + o, (double)sum);
-  atomicAdd(acc + 2 * plane + o, (double)sq);
+  atomicAdd(acc + o, widen(sum));
+  atomicAdd(acc + 2 * plane + o, widen(sq));
 }
 
 cudaError_t launch_k3_column(const float2* spec, int Mp, int G, int m, int M, float pref4a,

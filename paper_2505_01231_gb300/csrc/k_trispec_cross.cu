@@ -69,10 +69,10 @@ k3_trispec_cross(const float2* __restrict__ spec, long long chan_stride, int G, 
         const int l = lc + i;
         if (l < M) {
           const long long o = (long long)blockIdx.z * combo_stride + (long long)r * M + l;
-          atomicAdd(acc + o, (double)sre[i]);
-          atomicAdd(acc + plane + o, (double)sim[i]);
-          atomicAdd(acc + 2 * plane + o, (double)qre[i]);
-          atomicAdd(acc + 3 * plane + o, (double)qim[i]);
+          atomicAdd(acc + o, widen(sre[i]));
+          atomicAdd(acc + plane + o, widen(sim[i]));
+          atomicAdd(acc + 2 * plane + o, widen(qre[i]));
+          atomicAdd(acc + 3 * plane + o, widen(qim[i]));
         }
         sre[i] = sim[i] = qre[i] = qim[i] = 0.f;
       }

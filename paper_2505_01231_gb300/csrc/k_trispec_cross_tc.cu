@@ -720,10 +720,10 @@ k3_trispec_cross_tc(const __grid_constant__ CUtensorMap tm_ab,
           const int lc = l0 + kXLw * h + e;
           if (r <= rows_hi && lc < M) {
             const long long o = cbase + (long long)r * M + lc;
-            atomicAdd(acc + o, (double)sre[e]);
-            atomicAdd(acc + plane + o, (double)sim[e]);
-            atomicAdd(acc + 2 * plane + o, (double)qre[e]);
-            atomicAdd(acc + 3 * plane + o, (double)qim[e]);
+            atomicAdd(acc + o, widen(sre[e]));
+            atomicAdd(acc + plane + o, widen(sim[e]));
+            atomicAdd(acc + 2 * plane + o, widen(qre[e]));
+            atomicAdd(acc + 3 * plane + o, widen(qim[e]));
           }
           sre[e] = sim[e] = qre[e] = qim[e] = 0.f;
         }

@@ -298,10 +298,10 @@ k3_trispec_gram(const __grid_constant__ CUtensorMap tm32, const __grid_constant_
           const int l = 32 * h + lane;
           const float* col = reinterpret_cast<const float*>(ring0) + r * 64 +
                              4 * ((l >> 2) ^ perm) + (l & 3);
-          double v = 0.0;
-#pragma unroll
-          for (int w = 0; w < kGWarps; ++w) v += (double)col[w * (kGRing / 4)];
-          if (k0 + r <= l0 + l && l0 + l < lim) atomicAdd(dst + (long long)r * M + l, v);
+          if (k0 + r <= l0 + l && l0 + l < lim)
+            atomicAdd(dst + (long long)r * M + l,
+                      widen_sum4(col[0], col[kGRing / 4], col[2 * (kGRing / 4)],
+                                 col[3 * (kGRing / 4)], wq.group_chunk <= 4));
         }
       }
       __syncthreads();

@@ -452,8 +452,8 @@ k3_trispec_tc(const __grid_constant__ CUtensorMap tm_img, const float* __restric
           const int l = r.l0 + col0 + i;
           if (i < 16 * nh && k <= l && l < M) {
             const long long o = r.off + (long long)l * M + k;
-            atomicAdd(acc + o, (double)sm[i]);
-            atomicAdd(acc + 2 * plane + o, (double)sq[i]);
+            atomicAdd(acc + o, widen(sm[i]));
+            atomicAdd(acc + 2 * plane + o, widen(sq[i]));
           }
           sm[i] = sq[i] = 0.f;
         }

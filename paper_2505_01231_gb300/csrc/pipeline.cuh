@@ -17,6 +17,34 @@ constexpr unsigned long long kWaitLimitNs = 2000000000ull;
 // Limit of the wait that the timeout test injects (on a barrier nothing completes).
 constexpr unsigned long long kInjectedWaitNs = 1000000ull;
 
+// (double)f by integer operations.  The conversion instruction runs on the float64 pipe,
+// two a clock and SM: an item's end that widened 4096 sums cost 2000 clocks of it, and
+// four times that with the four warps' sums added in float64.
+__device__ __forceinline__ double widen(float f) {
+  const uint32_t b = __float_as_uint(f), mag = b & 0x7fffffffu;
+  if (mag - 0x00800000u < 0x7f000000u)  // a normal number
+    return __hiloint2double((int)((b & 0x80000000u) | ((mag >> 3) + 0x38000000u)), (int)(b << 29));
+  return mag == 0u ? __hiloint2double((int)b, 0) : (double)f;
+}
+
+// The sum of four warps' float32 sums, widened.  exact (each holds one group at most):
+// to float64's accuracy, so that sums over few groups do not depend on how a record was
+// cut into calls; the rounding errors of the float32 additions (two-sum, Knuth) enter
+// with one float64 addition.  Else as inexact as the runs themselves.
+__device__ __forceinline__ double widen_sum4(float a, float b, float c, float d, bool exact) {
+  if (!exact) return widen((a + b) + (c + d));
+  float s = a, e = 0.f;
+  auto add = [&](float x) {
+    const float t = __fadd_rn(s, x), u = __fadd_rn(t, -s);
+    e = __fadd_rn(e, __fadd_rn(__fadd_rn(s, -__fadd_rn(t, -u)), __fadd_rn(x, -u)));
+    s = t;
+  };
+  add(b);
+  add(c);
+  add(d);
+  return e == 0.f ? widen(s) : widen(s) + widen(e);
+}
+
 __device__ __forceinline__ uint32_t smem_addr(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
