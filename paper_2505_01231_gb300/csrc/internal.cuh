@@ -249,9 +249,31 @@ size_t k3tc_smem_bytes(int precision);
 // K3 for several channels (FP32 CUDA cores): C4(a_k, b_k*, c_l, d_l*) of every
 // combination (combos: device array of n_combos (a, b, c, d)) on the grid
 // k in [-(M-1), M-1] x l in [0, M-1], accumulated at acc[plane][combo][k+M-1][l].
+// A combination with a == b or c == d is symmetric: exchanging x and y (a == b) or z
+// and w together with the conjugation of all four (c == d) gives
+//   S4(-k, l) = S4(k, l) (a == b),  S4(-k, l) = S4(k, l)* (c == d),
+// so only its rows k >= 0 are computed and mirrored (34 of 55 combinations of four
+// channels).  rowtiles: device array of n_rowtiles (combination, first row r = k + M - 1);
+// half: device array of n_half (combination, 1 to conjugate) of the mirrored ones.
+constexpr int kCrossRows32 = 16;  // rows of a tile of the FP32 kernel
+struct CrossTiles {
+  const int2* rowtiles = nullptr;
+  const int2* half = nullptr;
+  int n_rowtiles = 0, n_half = 0;
+};
 cudaError_t launch_k3_trispec_cross(const float2* spec, long long chan_stride, int G, int m, int M,
-                                    int Mp, const int4* combos, int n_combos, double* acc,
-                                    long long plane, int nsm, bool natural, cudaStream_t stream);
+                                    int Mp, const int4* combos, int n_combos, const CrossTiles& ct,
+                                    double* acc, long long plane, int nsm, bool natural,
+                                    cudaStream_t stream);
+// the row k = M - 1 of the mirrored combinations, in FP32
+cudaError_t launch_k3_cross_last_row(const float2* spec, long long chan_stride, int G, int m, int M,
+                                     int Mp, const int4* combos, const CrossTiles& ct, float pref,
+                                     float fmm, float fm1, double* acc, long long plane,
+                                     cudaStream_t stream);
+// rows k < 0 of the mirrored combinations from the rows k > 0 (by assignment, after
+// every batch), and with row0 also the row k = -(M - 1) of the others from k = M - 1
+cudaError_t launch_k3_cross_mirror(const CrossTiles& ct, int n_combos, int M, double* acc,
+                                   long long plane, bool row0, cudaStream_t stream);
 int k3tc_stage_chunks(int precision);
 
 // The same on the tcgen05 tensor cores: tiles of 128 rows k x 24 columns l,
@@ -262,14 +284,16 @@ int k3tc_stage_chunks(int precision);
 // The spectra are read through 2-D views [rows][Mp] (8-byte elements, no swizzle):
 // tm_ab with boxes of kF rows x min(box bins, Mp) bins, tm_cd with boxes of kF
 // rows x col box bins (kF = 4 frames, 8 for FP16); a channel's rows start at
-// channel x chan_rows.  FP16 also reads the row scales [channel x grp_rows +
+// channel x chan_rows; spec, chan_stride and Ms address the same coefficients.  The
+// mirrored combinations' row k = M - 1, alone in its tile where M - 1 is a multiple of
+// 128, is left to a CUDA-core kernel.  FP16 also reads the row scales [channel x grp_rows +
 // group][Mp] (float) through tm_sab (boxes of min(kCrossScaleBins, Mp) bins) and
 // tm_scd (kCrossScaleCols bins).  The row k = -(M-1) is copied from k = M-1 (equal
 // for real signals).  counter and status as for the pair kernels.
 // Box widths (bins) of tm_ab and tm_cd, TF32 and FP16 forms: wider than the bins
 // used, so that the rows of a thread's two frame chunks fall on other banks.
 constexpr int kCrossBoxBins = 140, kCrossBoxBinsH = 142, kCrossColBox = 28, kCrossColBoxH = 30;
-constexpr int kCrossTileCols = 24, kCrossScaleBins = 144, kCrossScaleCols = 28;
+constexpr int kCrossTileRows = 128, kCrossTileCols = 24, kCrossScaleBins = 144, kCrossScaleCols = 28;
 struct CrossViews {
   const CUtensorMap* tm_ab = nullptr;
   const CUtensorMap* tm_cd = nullptr;
@@ -279,9 +303,10 @@ struct CrossViews {
   bool f16 = false;
 };
 cudaError_t launch_k3_trispec_cross_tc(const CrossViews& v, int G, int m, int M, int Mp,
-                                       const int4* combos, int n_combos, double* acc,
-                                       long long plane, int nsm, bool natural, int* counter,
-                                       int* status, cudaStream_t stream);
+                                       const int4* combos, int n_combos, const CrossTiles& ct,
+                                       const float2* spec, long long chan_stride, int Ms,
+                                       double* acc, long long plane, int nsm, bool natural,
+                                       int* counter, int* status, cudaStream_t stream);
 
 // Most groups whose per-group estimates a kernel adds up in float32 before the
 // run goes to the float64 accumulators (bounds the float32 rounding of the sums

@@ -24,7 +24,7 @@
 namespace ss {
 namespace {
 
-constexpr int kRT = 16, kLT = 64, kFrames = 16, kThreads = 256, kFlushGroups = 64;
+constexpr int kRT = kCrossRows32, kLT = 64, kFrames = 16, kThreads = 256, kFlushGroups = 64;
 
 __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
   return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
@@ -37,18 +37,19 @@ __device__ __forceinline__ float2 conjf2(float2 a) { return make_float2(a.x, -a.
 
 __global__ void __launch_bounds__(kThreads, 2)
 k3_trispec_cross(const float2* __restrict__ spec, long long chan_stride, int G, int m, int M,
-                 int Mp, const int4* __restrict__ combos, int tiles_l, int groups_per_cta,
+                 int Mp, const int4* __restrict__ combos,
+                 const int2* __restrict__ rowtiles, int tiles_l, int groups_per_cta,
                  float pref, float fmm, float fm1, double* __restrict__ acc, long long plane,
                  long long combo_stride) {
   __shared__ __align__(16) float2 sx[kFrames][kRT], sy[kFrames][kRT], sxy[kFrames][kRT];
   __shared__ __align__(16) float2 sz[kFrames][kLT], sw[kFrames][kLT], szw[kFrames][kLT];
   const int tid = threadIdx.x;
-  const int tile = blockIdx.x;
-  const int r0 = (tile / tiles_l) * kRT, l0 = (tile % tiles_l) * kLT;
+  const int2 rt = rowtiles[blockIdx.x / tiles_l];  // (combination, first row)
+  const int r0 = rt.y, l0 = (blockIdx.x % tiles_l) * kLT;
   const int g0 = blockIdx.y * groups_per_cta;
   const int g1 = min(G, g0 + groups_per_cta);
   if (g0 >= g1) return;
-  const int4 cb = combos[blockIdx.z];
+  const int4 cb = combos[rt.x];
   const float2* A = spec + cb.x * chan_stride;
   const float2* B = spec + cb.y * chan_stride;
   const float2* C = spec + cb.z * chan_stride;
@@ -68,7 +69,7 @@ k3_trispec_cross(const float2* __restrict__ spec, long long chan_stride, int G, 
       for (int i = 0; i < 4; ++i) {
         const int l = lc + i;
         if (l < M) {
-          const long long o = (long long)blockIdx.z * combo_stride + (long long)r * M + l;
+          const long long o = (long long)rt.x * combo_stride + (long long)r * M + l;
           atomicAdd(acc + o, widen(sre[i]));
           atomicAdd(acc + plane + o, widen(sim[i]));
           atomicAdd(acc + 2 * plane + o, widen(qre[i]));
@@ -171,23 +172,132 @@ k3_trispec_cross(const float2* __restrict__ spec, long long chan_stride, int G, 
   if (since_flush) flush();
 }
 
+// The row k = M - 1 of the mirrored combinations (the tensor-core tiles of 128 rows leave
+// it out when it would be alone in a tile): thread = column, one group at a time.
+constexpr int kRowThreads = 128;
+
+__global__ void __launch_bounds__(kRowThreads)
+k3_cross_last_row(const float2* __restrict__ spec, long long chan_stride, int G, int m, int M, int Mp,
+                  const int4* __restrict__ combos, const int2* __restrict__ half, float pref,
+                  float fmm, float fm1, double* __restrict__ acc, long long plane,
+                  long long combo_stride) {
+  const int l = blockIdx.x * kRowThreads + threadIdx.x, q = half[blockIdx.z].x;
+  if (l >= M) return;
+  const int4 cb = combos[q];
+  float sr = 0.f, si = 0.f, qr = 0.f, qi = 0.f;
+  for (int g = blockIdx.y; g < G; g += gridDim.y) {
+    const long long base = (long long)g * m * Mp;
+    const float2* A = spec + cb.x * chan_stride + base + (M - 1);
+    const float2* B = spec + cb.y * chan_stride + base + (M - 1);
+    const float2* C = spec + cb.z * chan_stride + base + l;
+    const float2* D = spec + cb.w * chan_stride + base + l;
+    const float2 o = make_float2(0.f, 0.f);
+    float2 xyzw = o, xz = o, yw = o, xw = o, yz = o, sxy = o, szw = o;
+#pragma unroll 4
+    for (int j = 0; j < m; ++j) {
+      const float2 x = __ldg(A + (long long)j * Mp), y = conjf2(__ldg(B + (long long)j * Mp));
+      const float2 z = __ldg(C + (long long)j * Mp), w = conjf2(__ldg(D + (long long)j * Mp));
+      const float2 xy = cmul(x, y), zw = cmul(z, w);
+      cmac(xyzw, xy, zw);
+      cmac(xz, x, z);
+      cmac(yw, y, w);
+      cmac(xw, x, w);
+      cmac(yz, y, z);
+      sxy = make_float2(sxy.x + xy.x, sxy.y + xy.y);
+      szw = make_float2(szw.x + zw.x, szw.y + zw.y);
+    }
+    float2 t = cmul(sxy, szw);
+    cmac(t, xz, yw);
+    cmac(t, xw, yz);
+    const float cr = pref * fmaf(fmm, xyzw.x, -fm1 * t.x);
+    const float ci = pref * fmaf(fmm, xyzw.y, -fm1 * t.y);
+    sr += cr;
+    si += ci;
+    qr = fmaf(cr, cr, qr);
+    qi = fmaf(ci, ci, qi);
+  }
+  const long long off = (long long)q * combo_stride + (long long)(2 * M - 2) * M + l;
+  atomicAdd(acc + off, widen(sr));
+  atomicAdd(acc + plane + off, widen(si));
+  atomicAdd(acc + 2 * plane + off, widen(qr));
+  atomicAdd(acc + 3 * plane + off, widen(qi));
+}
+
+// blockIdx.z: combination (of the mirrored ones) x plane; rows r < M - 1 from 2M - 2 - r
+__global__ void k3_cross_mirror(double* __restrict__ acc, const int2* __restrict__ half, int M,
+                                long long combo_stride, long long plane) {
+  const int2 h = half[blockIdx.z >> 2];
+  const int pl = blockIdx.z & 3;
+  double* a = acc + pl * plane + h.x * combo_stride;
+  const bool negate = h.y != 0 && pl == 1;  // the sum of Im of the conjugate
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < (M - 1) * M; i += gridDim.x * blockDim.x) {
+    const int r = i / M, l = i - r * M;
+    const double v = a[(long long)(2 * M - 2 - r) * M + l];
+    a[i] = negate ? __hiloint2double(__double2hiint(v) ^ 0x80000000, __double2loint(v)) : v;
+  }
+}
+
+// row r = 0 (k = -(M - 1)) of every plane and combination <- row r = 2M - 2
+__global__ void k3_cross_row0(double* __restrict__ acc, int n, int M, long long combo_stride,
+                              long long plane) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const int l = i % M, pc = i / M;
+  const int c = pc >> 2, pl = pc & 3;
+  double* a = acc + pl * plane + (long long)c * combo_stride;
+  a[l] = a[(long long)(2 * M - 2) * M + l];
+}
+
 }  // namespace
 
+cudaError_t launch_k3_cross_last_row(const float2* spec, long long chan_stride, int G, int m, int M,
+                                     int Mp, const int4* combos, const CrossTiles& ct, float pref,
+                                     float fmm, float fm1, double* acc, long long plane,
+                                     cudaStream_t stream) {
+  if (ct.n_half <= 0) return cudaSuccess;
+  const int gx = (M + kRowThreads - 1) / kRowThreads;
+  // at most kMaxFp32Groups groups in a thread's float32 sums
+  const int gy = std::min(G, std::min(65535, std::max(std::max(1, 4096 / (gx * ct.n_half)),
+                                                      (G + kMaxFp32Groups - 1) / kMaxFp32Groups)));
+  k3_cross_last_row<<<dim3((unsigned)gx, (unsigned)gy, (unsigned)ct.n_half), kRowThreads, 0, stream>>>(
+      spec, chan_stride, G, m, M, Mp, combos, ct.half, pref, fmm, fm1, acc, plane,
+      (long long)(2 * M - 1) * M);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_k3_cross_mirror(const CrossTiles& ct, int n_combos, int M, double* acc,
+                                   long long plane, bool row0, cudaStream_t stream) {
+  const long long combo_stride = (long long)(2 * M - 1) * M;
+  if (row0) {
+    const int n = 4 * n_combos * M;
+    k3_cross_row0<<<(n + 255) / 256, 256, 0, stream>>>(acc, n, M, combo_stride, plane);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
+  if (ct.n_half > 0) {
+    const int gx = std::min(256, ((M - 1) * M + 255) / 256);
+    k3_cross_mirror<<<dim3((unsigned)gx, 1, (unsigned)(4 * ct.n_half)), 256, 0, stream>>>(
+        acc, ct.half, M, combo_stride, plane);
+  }
+  return cudaGetLastError();
+}
+
 cudaError_t launch_k3_trispec_cross(const float2* spec, long long chan_stride, int G, int m, int M,
-                                    int Mp, const int4* combos, int n_combos, double* acc,
-                                    long long plane, int nsm, bool natural, cudaStream_t stream) {
+                                    int Mp, const int4* combos, int n_combos, const CrossTiles& ct,
+                                    double* acc, long long plane, int nsm, bool natural,
+                                    cudaStream_t stream) {
   if (G <= 0 || n_combos <= 0) return cudaSuccess;
   const int rows = 2 * M - 1;
-  const int tiles_r = (rows + kRT - 1) / kRT, tiles_l = (M + kLT - 1) / kLT;
-  const long long tiles = (long long)tiles_r * tiles_l;
+  const int tiles_l = (M + kLT - 1) / kLT;
+  const long long tiles = (long long)ct.n_rowtiles * tiles_l;  // of all combinations
   // enough CTAs for about four waves of two CTAs per SM
-  long long chunks = (8ll * nsm + tiles * n_combos - 1) / (tiles * n_combos);
+  long long chunks = (8ll * nsm + tiles - 1) / tiles;
   if (chunks < 1) chunks = 1;
   if (chunks > G) chunks = G;
   if (chunks > 65535) chunks = 65535;
   const int gpc = (int)((G + chunks - 1) / chunks);
   chunks = (G + gpc - 1) / gpc;
-  if (tiles > 0x7fffffffll || n_combos > 65535) return cudaErrorInvalidValue;
+  if (tiles > 0x7fffffffll || 4 * ct.n_half > 65535) return cudaErrorInvalidValue;
   const double md = m;
   // c4 = pref [fmm sum xyzw - fm1 (sum xy sum zw + ...)]: the k-statistic (Eq. 85),
   // or the natural estimator 1/m sum xyzw - 1/m^2 (...)
@@ -195,11 +305,13 @@ cudaError_t launch_k3_trispec_cross(const float2* spec, long long chan_stride, i
       (float)(natural ? 1.0 / (md * md) : 1.0 / ((md - 1.0) * (md - 2.0) * (md - 3.0)));
   const float fmm = (float)(natural ? md : md * (md + 1.0));
   const float fm1 = (float)(natural ? 1.0 : md - 1.0);
-  dim3 grid((unsigned)tiles, (unsigned)chunks, (unsigned)n_combos);
-  k3_trispec_cross<<<grid, kThreads, 0, stream>>>(spec, chan_stride, G, m, M, Mp, combos, tiles_l,
-                                                  gpc, pref, fmm, fm1, acc, plane,
+  dim3 grid((unsigned)tiles, (unsigned)chunks);
+  k3_trispec_cross<<<grid, kThreads, 0, stream>>>(spec, chan_stride, G, m, M, Mp, combos, ct.rowtiles,
+                                                  tiles_l,                                                  gpc, pref, fmm, fm1, acc, plane,
                                                   (long long)rows * M);
-  return cudaGetLastError();
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  return launch_k3_cross_mirror(ct, n_combos, M, acc, plane, false, stream);
 }
 
 }  // namespace ss

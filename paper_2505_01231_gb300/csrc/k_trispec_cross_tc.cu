@@ -62,7 +62,7 @@
 namespace ss {
 namespace {
 
-constexpr int kXT = 128;     // rows of a tile
+constexpr int kXT = kCrossTileRows;  // rows of a tile (128)
 constexpr int kXL = kCrossTileCols;  // columns of a tile (24)
 constexpr int kXLw = kXL / 2;        // columns of an epilogue warp
 constexpr int kXEpiWarps = 8, kXBuildWarps = 8;
@@ -239,7 +239,8 @@ __device__ __forceinline__ void mbar_arrive_x(uint64_t* bar) {
 
 struct CrossQueue {
   int* counter;
-  int n_items, n_tiles, n_combos, n_cb, group_chunk;
+  int n_items, n_tiles, n_cb, group_chunk;  // n_tiles: of all combinations
+  const int2* rowtiles;                      // (combination, first row)
 };
 
 template <bool kF16>
@@ -569,13 +570,12 @@ k3_trispec_cross_tc(const __grid_constant__ CUtensorMap tm_ab,
     if (lane == 0) {
       uint32_t rq = 0;
       bool ok = true;
-      const int per_chunk = wq.n_tiles * wq.n_combos;
       for (;;) {
         const int item = *(volatile int*)&s_fail ? wq.n_items : atomicAdd(wq.counter, 1);
         if (item >= wq.n_items) break;
-        const int chunk = item / per_chunk, rest = item - chunk * per_chunk;
-        const int combo = rest / wq.n_tiles, tile = rest - combo * wq.n_tiles;
-        const int r0 = 1 + (tile / wq.n_cb) * kXT, l0 = (tile % wq.n_cb) * kXL;
+        const int chunk = item / wq.n_tiles, rest = item - chunk * wq.n_tiles;
+        const int2 rt = wq.rowtiles[rest / wq.n_cb];
+        const int combo = rt.x, r0 = rt.y, l0 = (rest % wq.n_cb) * kXL;
         const int g0 = chunk * wq.group_chunk, g1 = min(G, g0 + wq.group_chunk);
         const int4 cb = combos[combo];
         // bins |k| of the tile's rows: one range of at most 128 bins, staged from a
@@ -739,36 +739,27 @@ k3_trispec_cross_tc(const __grid_constant__ CUtensorMap tm_ab,
   }
 }
 
-// row r = 0 (k = -(M - 1)) of every plane and combination <- row r = 2M - 2
-__global__ void k3_cross_row0(double* __restrict__ acc, int n, int M, long long combo_stride,
-                              long long plane) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const int l = i % M, pc = i / M;
-  const int c = pc >> 2, pl = pc & 3;
-  double* a = acc + pl * plane + (long long)c * combo_stride;
-  a[l] = a[(long long)(2 * M - 2) * M + l];
-}
-
 }  // namespace
 
 cudaError_t launch_k3_trispec_cross_tc(const CrossViews& v, int G, int m, int M, int Mp,
-                                       const int4* combos, int n_combos, double* acc,
-                                       long long plane, int nsm, bool natural, int* counter,
-                                       int* status, cudaStream_t stream) {
+                                       const int4* combos, int n_combos, const CrossTiles& ct,
+                                       const float2* spec, long long chan_stride, int Ms,
+                                       double* acc, long long plane, int nsm, bool natural,
+                                       int* counter, int* status, cudaStream_t stream) {
   if (G <= 0 || n_combos <= 0) return cudaSuccess;
   if (m < 1 || M < 2 || nsm <= 0 || (Mp & 15) || Mp < M) return cudaErrorInvalidValue;
   if (v.f16 && (!v.tm_sab || !v.tm_scd)) return cudaErrorInvalidValue;
-  const int n_rb = (2 * M - 2 + kXT - 1) / kXT, n_cb = (M + kXL - 1) / kXL;
-  const long long n_tiles = (long long)n_rb * n_cb;
+  const int n_cb = (M + kXL - 1) / kXL;
+  const long long n_tiles = (long long)ct.n_rowtiles * n_cb;  // of all combinations
+  if (n_tiles <= 0 || n_tiles > 1 << 30 || 4 * ct.n_half > 65535) return cudaErrorInvalidValue;
   CrossQueue wq;
   wq.counter = counter;
   wq.n_tiles = (int)n_tiles;
-  wq.n_combos = n_combos;
   wq.n_cb = n_cb;
-  wq.group_chunk = work_group_chunk(G, (int)std::min<long long>(n_tiles * n_combos, 1 << 30), nsm);
+  wq.rowtiles = ct.rowtiles;
+  wq.group_chunk = work_group_chunk(G, (int)n_tiles, nsm);
   const long long n_chunks = (G + wq.group_chunk - 1) / wq.group_chunk;
-  const long long n_items = n_chunks * n_tiles * n_combos;
+  const long long n_items = n_chunks * n_tiles;
   if (n_items > 0x7fffffffll) return cudaErrorInvalidValue;
   wq.n_items = (int)n_items;
   auto kern = v.f16 ? k3_trispec_cross_tc<true> : k3_trispec_cross_tc<false>;
@@ -793,9 +784,12 @@ cudaError_t launch_k3_trispec_cross_tc(const CrossViews& v, int G, int m, int M,
                                          plane, combo_stride, status);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  const int n = 4 * n_combos * M;
-  k3_cross_row0<<<(n + 255) / 256, 256, 0, stream>>>(acc, n, M, combo_stride, plane);
-  return cudaGetLastError();
+  if ((M - 1) % kXT == 0) {
+    e = launch_k3_cross_last_row(spec, chan_stride, G, m, M, Ms, combos, ct, pref, fmm, fm1, acc,
+                                 plane, stream);
+    if (e != cudaSuccess) return e;
+  }
+  return launch_k3_cross_mirror(ct, n_combos, M, acc, plane, true, stream);
 }
 
 }  // namespace ss

@@ -137,6 +137,28 @@ std::vector<TileInfo> build_tc_tiles(int M, bool* last_col) {
   return t;
 }
 
+// Several channels: first the combinations whose rows k < 0 are mirrored (CrossTiles:
+// those with a == b or c == d), as (combination, conjugate), then the row tiles of all
+// combinations, as (combination, first row r = k + M - 1).  FP32: tiles of 16 rows over
+// all rows, or k = 0 .. M - 1 of the mirrored ones.  Tensor cores: 128 rows from k =
+// -(M - 2) on (row 0 is a copy), or from k = 0 on, without k = M - 1 where it would be
+// alone in a tile; with M - 1 < 128 one tile takes all rows and nothing is mirrored.
+// Returns the number of mirrored combinations.
+int build_cross_tiles(const std::vector<int4>& c4, int M, bool fp32, std::vector<int2>& out) {
+  const bool mirror = fp32 || M - 1 >= kCrossTileRows;
+  auto half = [&](const int4& c) { return mirror && (c.x == c.y || c.z == c.w); };
+  for (size_t i = 0; i < c4.size(); ++i)
+    if (half(c4[i])) out.push_back(make_int2((int)i, c4[i].x == c4[i].y ? 0 : 1));
+  const int n = (int)out.size();
+  const int step = fp32 ? kCrossRows32 : kCrossTileRows;
+  for (size_t i = 0; i < c4.size(); ++i) {
+    const bool h = half(c4[i]);
+    const int end = !fp32 && h && (M - 1) % kCrossTileRows == 0 ? 2 * M - 2 : 2 * M - 1;
+    for (int r = h ? M - 1 : fp32 ? 0 : 1; r < end; r += step) out.push_back(make_int2((int)i, r));
+  }
+  return n;
+}
+
 // Tiles of k3_trispec_gram: 32 k-bins by 64 l-bins that touch the upper triangle
 // k <= l.  A last column block that holds only l = M - 1 (T >= 128) is left to
 // k3_column (*last_col = true).
@@ -437,8 +459,8 @@ ss_status process_device(ss_plan_s* p, const void* ptr, long long n, long long s
         const long long plane = (long long)p->c4.size() * p->rows4 * p->M;
         if (p->C > 1 && p->precision == SS_PREC_FP32)
           SS_TRY(p, launch_k3_trispec_cross(spec, chan_stride, cnt, p->m, p->M, p->Ms,
-                                            p->d_c4cross, (int)p->c4.size(), p->d_acc4, plane,
-                                            p->nsm, nat, p->stream));
+                                            p->d_c4cross, (int)p->c4.size(), p->cross, p->d_acc4,
+                                            plane, p->nsm, nat, p->stream));
         else if (p->C > 1) {
           CrossViews v;
           v.tm_ab = &p->tmx_ab;
@@ -449,8 +471,9 @@ ss_status process_device(ss_plan_s* p, const void* ptr, long long n, long long s
           v.grp_rows = p->Gb_max;
           v.f16 = p->oi.rmax != nullptr;
           SS_TRY(p, launch_k3_trispec_cross_tc(v, cnt, p->m, p->M, p->Mp, p->d_c4cross,
-                                               (int)p->c4.size(), p->d_acc4, plane, p->nsm, nat,
-                                               p->d_counter, p->d_status, p->stream));
+                                               (int)p->c4.size(), p->cross, spec, chan_stride, p->Ms,
+                                               p->d_acc4, plane, p->nsm, nat, p->d_counter,
+                                               p->d_status, p->stream));
         }
         for (size_t i = 0; i < p->c4.size() && p->C == 1; ++i) {
           const Combo& cb = p->c4[i];
@@ -868,6 +891,7 @@ void destroy(ss_plan_s* p) {
   cudaFree(p->d_tiles3w);
   cudaFree(p->d_pts3w);
   cudaFree(p->d_c3);
+  cudaFree(p->d_c4tiles);
   cudaFree(p->d_tiles4g);
   cudaFree(p->d_tiles4);
   cudaFree(p->d_tiles4tc);
@@ -1104,6 +1128,15 @@ static ss_status plan_create(ss_plan_t* out, int channels, int T, double dt, int
     PLAN_TRY(dev_alloc(p, &p->d_c4cross, c4x.size() * sizeof(int4)));
     PLAN_TRY(cudaMemcpy(p->d_c4cross, c4x.data(), c4x.size() * sizeof(int4),
                         cudaMemcpyHostToDevice));
+    std::vector<int2> tiles;
+    const int n_half = build_cross_tiles(c4x, p->M, precision == SS_PREC_FP32, tiles);
+    PLAN_TRY(dev_alloc(p, &p->d_c4tiles, tiles.size() * sizeof(int2)));
+    PLAN_TRY(cudaMemcpy(p->d_c4tiles, tiles.data(), tiles.size() * sizeof(int2),
+                        cudaMemcpyHostToDevice));
+    p->cross.half = p->d_c4tiles;
+    p->cross.n_half = n_half;
+    p->cross.rowtiles = p->d_c4tiles + n_half;
+    p->cross.n_rowtiles = (int)tiles.size() - n_half;
   }
   PLAN_TRY(cudaMemcpy(p->d_win, gw.data(), T * sizeof(float), cudaMemcpyHostToDevice));
   PLAN_TRY(cudaMemcpy(p->d_tw, tw.data(), T * sizeof(float2), cudaMemcpyHostToDevice));

@@ -89,6 +89,8 @@ struct ss_plan_s {
   CUtensorMap tm_img[4]{};               // 4-D views of each channel's Gram operand image
   ss::TileInfo* d_tiles4tc = nullptr;  // tiles of the tensor-core S4 kernel (one channel)
   int4* d_c4cross = nullptr;       // (a, b, c, d) of each S4 combination (several channels)
+  int2* d_c4tiles = nullptr;       // its row tiles and mirrored combinations (CrossTiles)
+  ss::CrossTiles cross;
   int n_tiles4tc = 0;
   // FP32 S4 of one channel with m <= kGram32MaxM: the tiles of k3_trispec_gram
   bool gram32 = false;
