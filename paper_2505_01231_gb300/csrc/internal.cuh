@@ -255,7 +255,7 @@ size_t k3tc_smem_bytes(int precision);
 // so only its rows k >= 0 are computed and mirrored (34 of 55 combinations of four
 // channels).  rowtiles: device array of n_rowtiles (combination, first row r = k + M - 1);
 // half: device array of n_half (combination, 1 to conjugate) of the mirrored ones.
-constexpr int kCrossRows32 = 16;  // rows of a tile of the FP32 kernel
+constexpr int kCrossRows32 = 32;  // rows and columns of a tile of the FP32 kernel
 struct CrossTiles {
   const int2* rowtiles = nullptr;
   const int2* half = nullptr;
@@ -323,6 +323,19 @@ inline int work_group_chunk(int G, int n_tiles, int n_cta) {
   if (gc > kMaxFp32Groups) gc = kMaxFp32Groups;
   if (gc > G) gc = G;
   return (int)gc;
+}
+
+// Runs of groups of k3_trispec_cross and K5, of at most kMaxFp32Groups groups: CTAs for
+// one full wave of kRunCtas per SM where that leaves at most a seventh of the places
+// empty, else for four waves.
+constexpr int kRunCtas = 3;
+inline int group_runs(int G, long long ctas_per_run, int nsm) {
+  const long long places = (long long)kRunCtas * nsm;
+  long long runs = places / ctas_per_run;
+  if (runs * ctas_per_run * 7 < places * 6) runs = (4 * places + ctas_per_run - 1) / ctas_per_run;
+  runs = std::max(runs, (long long)(G + kMaxFp32Groups - 1) / kMaxFp32Groups);
+  runs = std::min<long long>(std::min<long long>(runs, G), 65535);
+  return (int)std::max(1ll, runs);
 }
 
 // Spectra of complex-valued signals (App. D) and shifted S4 planes (App. E) on

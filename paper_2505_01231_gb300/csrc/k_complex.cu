@@ -43,7 +43,6 @@ namespace {
 constexpr int kThreads = 128, kChunk = 8;  // frames staged at a time
 constexpr int kT4 = 32;                    // S4 tile: 32 x 32
 constexpr int kR3 = 32, kL3 = 64;          // S3 tile
-constexpr int kResident = 3;               // CTAs per SM
 constexpr int kBins2 = 32, kLanes2 = 8;    // S2: bins of a CTA, its groups at a time
 
 __device__ __forceinline__ float2 cmulc(float2 a, float2 b) {
@@ -158,7 +157,7 @@ __device__ __forceinline__ void flush_point(double* __restrict__ acc, long long 
 // S3: thread = 4 x 4 points.  A frame's operands: a[32] | b[64] | c[96], c at
 // -(k + l) for row + column = 0 .. 94; the 16-byte pieces of c are exchanged in pairs
 // in every other 128 bytes, for the lanes of a row that lie 128 bytes apart.
-__global__ void __launch_bounds__(kThreads, kResident)
+__global__ void __launch_bounds__(kThreads, kRunCtas)
 k5_cplx_s3(const float2* __restrict__ spec, long long chan_stride, int G, int m, int M, int Mp,
            const int4* __restrict__ ops, int tiles_l, int groups_per_cta, float pref3,
            double* __restrict__ acc, long long plane) {
@@ -260,7 +259,7 @@ k5_cplx_s3(const float2* __restrict__ spec, long long chan_stride, int G, int m,
 // y = B(-k - s) of row e / 2 < 32, z = C(l - s) and w = D(-l + s) of column e / 2 - 32, in
 // even and odd threads; the even one also writes the product, and at a group's last frame
 // the group's sum of it (the two sums that belong to a row or a column, not to a point).
-__global__ void __launch_bounds__(kThreads, kResident)
+__global__ void __launch_bounds__(kThreads, kRunCtas)
 k5_cplx_s4(const float2* __restrict__ spec, long long chan_stride, int G, int m, int M, int Mp,
            const int4* __restrict__ ops, int tiles_l, int groups_per_cta, int shift, float pref,
            float fmm, float fm1, double* __restrict__ acc, long long plane) {
@@ -357,17 +356,6 @@ k5_cplx_s4(const float2* __restrict__ spec, long long chan_stride, int G, int m,
   for (int p = 0; p < 8; ++p)
     flush_point(acc, plane, n, r0 + 2 * ti + p / 4, c0 + 4 * tj + p % 4, 2 * M, sr[p], si[p], qr[p],
                 qi[p]);
-}
-
-// Runs of groups: of at most kMaxFp32Groups groups; CTAs for one full wave where that
-// leaves at most a seventh of the SMs' places empty, else for four waves.
-int group_runs(int G, long long ctas_per_run, int nsm) {
-  const long long places = (long long)kResident * nsm;
-  long long runs = places / ctas_per_run;
-  if (runs * ctas_per_run * 7 < places * 6) runs = (4 * places + ctas_per_run - 1) / ctas_per_run;
-  runs = std::max(runs, (long long)(G + kMaxFp32Groups - 1) / kMaxFp32Groups);
-  runs = std::min<long long>(std::min<long long>(runs, G), 65535);
-  return (int)std::max(1ll, runs);
 }
 
 }  // namespace

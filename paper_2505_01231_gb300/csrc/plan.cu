@@ -139,10 +139,10 @@ std::vector<TileInfo> build_tc_tiles(int M, bool* last_col) {
 
 // Several channels: first the combinations whose rows k < 0 are mirrored (CrossTiles:
 // those with a == b or c == d), as (combination, conjugate), then the row tiles of all
-// combinations, as (combination, first row r = k + M - 1).  FP32: tiles of 16 rows over
-// all rows, or k = 0 .. M - 1 of the mirrored ones.  Tensor cores: 128 rows from k =
-// -(M - 2) on (row 0 is a copy), or from k = 0 on, without k = M - 1 where it would be
-// alone in a tile; with M - 1 < 128 one tile takes all rows and nothing is mirrored.
+// combinations, as (combination, first row r = k + M - 1).  Tiles of 32 rows
+// (FP32) or 128 (tensor cores) from k = -(M - 2) on (row 0 is a copy), or from k = 0 on
+// of the mirrored ones, without k = M - 1 where it would be alone in a tile; on the
+// tensor cores with M - 1 < 128 one tile takes all rows and nothing is mirrored.
 // Returns the number of mirrored combinations.
 int build_cross_tiles(const std::vector<int4>& c4, int M, bool fp32, std::vector<int2>& out) {
   const bool mirror = fp32 || M - 1 >= kCrossTileRows;
@@ -153,8 +153,8 @@ int build_cross_tiles(const std::vector<int4>& c4, int M, bool fp32, std::vector
   const int step = fp32 ? kCrossRows32 : kCrossTileRows;
   for (size_t i = 0; i < c4.size(); ++i) {
     const bool h = half(c4[i]);
-    const int end = !fp32 && h && (M - 1) % kCrossTileRows == 0 ? 2 * M - 2 : 2 * M - 1;
-    for (int r = h ? M - 1 : fp32 ? 0 : 1; r < end; r += step) out.push_back(make_int2((int)i, r));
+    const int end = h && (M - 1) % step == 0 ? 2 * M - 2 : 2 * M - 1;
+    for (int r = h ? M - 1 : 1; r < end; r += step) out.push_back(make_int2((int)i, r));
   }
   return n;
 }
