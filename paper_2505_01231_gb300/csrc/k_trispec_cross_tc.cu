@@ -19,7 +19,7 @@
 // scaled per group and bin by powers of two that keep them below 2^14: x sx,
 // y sy, (x sx)(y sy) 2^-14 and z tz, w tw, (z tz)(w tw) 2^-14, with the scales
 // written by K1; the epilogue undoes them one power of two at a time.  Sxy and
-// Szw depend on one bin each and are summed, unscaled, by the threads that build
+// Szw depend on one bin each and are summed, scaled alike, by the threads that build
 // the operands.
 //
 // Building the operands is the limit: an M = 128, N <= 128 product reads its
@@ -171,6 +171,18 @@ __device__ __forceinline__ void put_split16(unsigned char* blk, uint32_t lo_off,
   }
   *reinterpret_cast<uint4*>(blk + off) = make_uint4(h[0], h[1], h[2], h[3]);
   *reinterpret_cast<uint4*>(blk + lo_off + off) = make_uint4(l[0], l[1], l[2], l[3]);
+}
+
+// kF16 ? 4 : 2 complex values (one 16-byte chunk) into the hi and lo blocks
+template <bool kF16>
+__device__ __forceinline__ void put_operand(unsigned char* blk, uint32_t lo_off, uint32_t off,
+                                            const float2 (&c)[kF16 ? 4 : 2]) {
+  if constexpr (kF16) {
+    const float v[8] = {c[0].x, c[0].y, c[1].x, c[1].y, c[2].x, c[2].y, c[3].x, c[3].y};
+    put_split16(blk, lo_off, off, v);
+  } else {
+    put_split(blk, lo_off, off, c[0].x, c[0].y, c[1].x, c[1].y);
+  }
 }
 
 // 1 / s for a normal power of two s (exact): the exponent field mirrored
@@ -334,30 +346,55 @@ k3_trispec_cross_tc(const __grid_constant__ CUtensorMap tm_ab,
       if (!ok) break;
       const RawRec rec = rrec[rs];
       if (rec.flags & kRecStop) break;
-      const int r = rec.r0 + R, k = r - (M - 1);
-      const bool rv = r <= rows_hi;
-      const int kb = k < 0 ? -k : k;
-      const int j0 = rec.st * F::kF;  // first frame of the stage
+      // Rows past the grid build from what their places hold (staged bins, or zeros): a
+      // row of A reaches only its own row of the products, which is not stored.
+      const int k = rec.r0 + R - (M - 1);
+      const bool neg = k < 0;
+      const int kb = (neg ? -k : k) - rec.bstart;
+      const int left = m - rec.st * F::kF;  // frames of the group from this stage on
       const unsigned char* rbase = raws + (size_t)rs * F::kRawBytes;
-      const float2* raw = reinterpret_cast<const float2*>(rbase);
-      float2 va[kH], vb[kH], vc[kH], vd[kH];
+      const float2* ra = reinterpret_cast<const float2*>(rbase) + F::kRawA / 8 + kH * fp * rawk + kb;
+      const float2* rb = ra + (F::kRawB - F::kRawA) / 8;
+      const float2* rc =
+          reinterpret_cast<const float2*>(rbase) + F::kRawC / 8 + kH * tfq * F::kColBox + tli;
+      const float2* rd = rc + (F::kRawD - F::kRawC) / 8;
+      float2 x[kH], y[kH], z[kH], w[kH];
       const bool lv = top >= 0 && rec.l0 + tli < M;
+      if (left >= F::kF) {
 #pragma unroll
-      for (int jj = 0; jj < kH; ++jj) {
-        const int fj = kH * fp + jj;  // frame within the stage
-        const bool v = rv && j0 + fj < m;
-        va[jj] = v ? raw[F::kRawA / 8 + fj * rawk + kb - rec.bstart] : zero;
-        vb[jj] = v ? raw[F::kRawB / 8 + fj * rawk + kb - rec.bstart] : zero;
-        const int fk = kH * tfq + jj;
-        const bool w = lv && j0 + fk < m;
-        vc[jj] = w && top != 1 ? raw[F::kRawC / 8 + fk * F::kColBox + tli] : zero;
-        vd[jj] = w && top != 0 ? raw[F::kRawD / 8 + fk * F::kColBox + tli] : zero;
+        for (int jj = 0; jj < kH; ++jj) {
+          x[jj] = ra[jj * rawk];
+          y[jj] = rb[jj * rawk];
+        }
+        if (top >= 0) {
+#pragma unroll
+          for (int jj = 0; jj < kH; ++jj) {
+            z[jj] = lv ? rc[jj * F::kColBox] : zero;
+            w[jj] = lv ? rd[jj * F::kColBox] : zero;
+          }
+        }
+      } else {
+#pragma unroll
+        for (int jj = 0; jj < kH; ++jj) {
+          const bool in = kH * fp + jj < left;
+          x[jj] = in ? ra[jj * rawk] : zero;
+          y[jj] = in ? rb[jj * rawk] : zero;
+        }
+        if (top >= 0) {
+#pragma unroll
+          for (int jj = 0; jj < kH; ++jj) {
+            const bool in = lv && kH * tfq + jj < left;
+            z[jj] = in ? rc[jj * F::kColBox] : zero;
+            w[jj] = in ? rd[jj * F::kColBox] : zero;
+          }
+        }
       }
       if constexpr (kF16) {
         if (rec.flags & kRecFirst) {  // the group's row scales, staged with its first stage
           const float* ssc = reinterpret_cast<const float*>(rbase);
-          sx = rv ? ssc[F::kRawSA / 4 + kb - rec.bstart] : 1.f;
-          sy = rv ? ssc[F::kRawSB / 4 + kb - rec.bstart] : 1.f;
+          const bool rv = rec.r0 + R <= rows_hi;
+          sx = rv ? ssc[F::kRawSA / 4 + kb] : 1.f;
+          sy = rv ? ssc[F::kRawSB / 4 + kb] : 1.f;
           tz = lv ? ssc[F::kRawSC / 4 + tli] : 1.f;
           tw = lv ? ssc[F::kRawSD / 4 + tli] : 1.f;
         }
@@ -370,82 +407,49 @@ k3_trispec_cross_tc(const __grid_constant__ CUtensorMap tm_ab,
       if (!ok) break;
       if (rec.flags & kRecFirst) sxy = szw = zero;
       unsigned char* stg = stages + (size_t)s * kXStageBytes;
-      // rows: k < 0: x = a_{|k|}*, y = b_{|k|};  k >= 0: x = a_k, y = b_k*
-      float2 x[kH], y[kH], xy[kH];
+      // rows: k < 0: x = a_{|k|}*, y = b_{|k|};  k >= 0: x = a_k, y = b_k*; with FP16
+      // scaled by powers of two, so that the group's sum of xy is the unscaled one's,
+      // rounded alike
+      const float cx = neg ? -sx : sx, cy = neg ? sy : -sy;
+      float2 xy[kH];
 #pragma unroll
       for (int jj = 0; jj < kH; ++jj) {
-        x[jj] = k < 0 ? make_float2(va[jj].x, -va[jj].y) : va[jj];
-        y[jj] = k < 0 ? vb[jj] : make_float2(vb[jj].x, -vb[jj].y);
+        x[jj] = make_float2(x[jj].x * sx, x[jj].y * cx);
+        y[jj] = make_float2(y[jj].x * sy, y[jj].y * cy);
         xy[jj] = cmulf(x[jj], y[jj]);
         sxy.x += xy[jj].x;
         sxy.y += xy[jj].y;
+        if constexpr (kF16) xy[jj] = make_float2(xy[jj].x * kPairScale, xy[jj].y * kPairScale);
       }
       const uint32_t o = core_off(R, fp);
-      if constexpr (!kF16) {
-        put_split(stg + kOffAX, kAMat, o, x[0].x, x[0].y, x[1].x, x[1].y);
-        put_split(stg + kOffAY, kAMat, o, y[0].x, y[0].y, y[1].x, y[1].y);
-        put_split(stg + kOffAP, kAMat, o, xy[0].x, xy[0].y, xy[1].x, xy[1].y);
-      } else {
-        // scaled rows: x sx, y sy and (x sx)(y sy) 2^-14, each below 2^14
-        float ex[8], ey[8], ep[8];
-#pragma unroll
-        for (int jj = 0; jj < kH; ++jj) {
-          const float2 xs = make_float2(x[jj].x * sx, x[jj].y * sx);
-          const float2 ys = make_float2(y[jj].x * sy, y[jj].y * sy);
-          const float2 ps = cmulf(xs, ys);
-          ex[2 * jj] = xs.x;
-          ex[2 * jj + 1] = xs.y;
-          ey[2 * jj] = ys.x;
-          ey[2 * jj + 1] = ys.y;
-          ep[2 * jj] = ps.x * kPairScale;
-          ep[2 * jj + 1] = ps.y * kPairScale;
-        }
-        put_split16(stg + kOffAX, kAMat, o, ex);
-        put_split16(stg + kOffAY, kAMat, o, ey);
-        put_split16(stg + kOffAP, kAMat, o, ep);
-      }
+      put_operand<kF16>(stg + kOffAX, kAMat, o, x);
+      put_operand<kF16>(stg + kOffAY, kAMat, o, y);
+      put_operand<kF16>(stg + kOffAP, kAMat, o, xy);
       if (top >= 0) {
         // operand top of bin l: z = c_l, w = d_l*, zw; its Re column (ur, -ui) and
         // its Im column (ui, ur)
-        float2 v[kH];
+        float2 re[kH], im[kH];
 #pragma unroll
         for (int jj = 0; jj < kH; ++jj) {
-          float2 z = vc[jj], w = make_float2(vd[jj].x, -vd[jj].y);
+          const float2 zs = make_float2(z[jj].x * tz, z[jj].y * tz);
+          const float2 ws = make_float2(w[jj].x * tw, w[jj].y * -tw);
+          float2 v = top == 0 ? zs : ws;
           if (top == 2) {
-            const float2 zw = cmulf(z, w);
-            szw.x += zw.x;
-            szw.y += zw.y;
+            v = cmulf(zs, ws);
+            szw.x += v.x;
+            szw.y += v.y;
+            if constexpr (kF16) v = make_float2(v.x * kPairScale, v.y * kPairScale);
           }
-          if constexpr (kF16) {
-            z = make_float2(z.x * tz, z.y * tz);
-            w = make_float2(w.x * tw, w.y * tw);
-            const float2 zws = cmulf(z, w);
-            v[jj] = top == 0 ? z
-                             : (top == 1 ? w : make_float2(zws.x * kPairScale, zws.y * kPairScale));
-          } else {
-            v[jj] = top == 0 ? z : (top == 1 ? w : cmulf(z, w));
-          }
+          re[jj] = make_float2(v.x, -v.y);
+          im[jj] = make_float2(v.y, v.x);
         }
         const uint32_t cre = top < 2 ? kOffBXY + core_off(kXL * (2 * top) + tli, tfq)
                                      : kOffBP + core_off(tli, tfq);
         const uint32_t cim = top < 2 ? kOffBXY + core_off(kXL * (2 * top + 1) + tli, tfq)
                                      : kOffBP + core_off(kXL + tli, tfq);
         const uint32_t lo = top < 2 ? kBXYMat : kBPMat;
-        if constexpr (!kF16) {
-          put_split(stg, lo, cre, v[0].x, -v[0].y, v[1].x, -v[1].y);
-          put_split(stg, lo, cim, v[0].y, v[0].x, v[1].y, v[1].x);
-        } else {
-          float er[8], ei[8];
-#pragma unroll
-          for (int jj = 0; jj < kH; ++jj) {
-            er[2 * jj] = v[jj].x;
-            er[2 * jj + 1] = -v[jj].y;
-            ei[2 * jj] = v[jj].y;
-            ei[2 * jj + 1] = v[jj].x;
-          }
-          put_split16(stg, lo, cre, er);
-          put_split16(stg, lo, cim, ei);
-        }
+        put_operand<kF16>(stg, lo, cre, re);
+        put_operand<kF16>(stg, lo, cim, im);
       }
       if (bt == 0) srec[s] = StageRec{rec.flags & (kRecFirst | kRecLast)};
       // the generic-proxy writes become visible to the tensor cores' reads
@@ -676,27 +680,18 @@ k3_trispec_cross_tc(const __grid_constant__ CUtensorMap tm_ab,
                                            slot[p].szw[0][li0 + i].y + slot[p].szw[1][li0 + i].y);
             const float2 xz = make_float2(d[0][i], d[1][i]), xw = make_float2(d[2][i], d[3][i]);
             const float2 yz = make_float2(d[4][i], d[5][i]), yw = make_float2(d[6][i], d[7][i]);
-            float cr, ci;
+            float2 t = cmulf(sxy, szw);
+            cmacf(t, xz, yw);
+            cmacf(t, xw, yz);
+            float ur = fmaf(fmm_p, d[8][i], -fm1 * t.x), ui = fmaf(fmm_p, d[9][i], -fm1 * t.y);
             if constexpr (kF16) {
-              // the scaled products: [fmm P - fm1 (Sxz Syw + Sxw Syz)] sx sy tz tw, undone
-              // one power of two at a time (their product alone may leave the float
-              // range); Sxy Szw is unscaled
-              float2 t = cmulf(xz, yw);
-              cmacf(t, xw, yz);
+              // [fmm P - fm1 (...)] sx sy tz tw, undone one power of two at a time (their
+              // product alone may leave the float range)
               const float2 rzw = slot[p].rzw[li0 + i];
-              float ur = fmaf(fmm_p, d[8][i], -fm1 * t.x), ui = fmaf(fmm_p, d[9][i], -fm1 * t.y);
               ur = ur * rxy.x * rxy.y * rzw.x * rzw.y;
               ui = ui * rxy.x * rxy.y * rzw.x * rzw.y;
-              const float2 u = cmulf(sxy, szw);
-              cr = pref * fmaf(-fm1, u.x, ur);
-              ci = pref * fmaf(-fm1, u.y, ui);
-            } else {
-              float2 t = cmulf(sxy, szw);
-              cmacf(t, xz, yw);
-              cmacf(t, xw, yz);
-              cr = pref * fmaf(fmm_p, d[8][i], -fm1 * t.x);
-              ci = pref * fmaf(fmm_p, d[9][i], -fm1 * t.y);
             }
+            const float cr = pref * ur, ci = pref * ui;
             const int e = 2 * hh + i;
             sre[e] += cr;
             sim[e] += ci;
