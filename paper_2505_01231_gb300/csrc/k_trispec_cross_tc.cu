@@ -54,8 +54,6 @@
 // a small kernel copies that row's sums after every batch.  Every wait is
 // bounded; on a failure the CTA stops, waits for the copies and products it
 // issued and frees its TMEM.
-#include <cuda_fp16.h>
-
 #include "internal.cuh"
 #include "pipeline.cuh"
 
@@ -129,9 +127,8 @@ struct RawRec {  // a staged stage: its tile, combination, first staged bin, fra
 
 struct CrossSlot {  // one group: its one-bin sums, scales and record, for the epilogue
   float2 sxy[kXT];
-  float2 szw[2][kXL];   // over the first and the second half of each stage's frames
-  float2 rxy[kXT];      // FP16: 1 / (row scales of x and y)
-  float2 rzw[kXL];      // FP16: 1 / (column scales of z and w)
+  float4 szw[kXL];      // Szw, FP16: 1 / (the column scales of z and w, multiplied)
+  float rxy[kXT];       // FP16: the same of the row scales of x and y
   int r0, l0, combo, flags;
 };
 
@@ -162,13 +159,7 @@ __device__ __forceinline__ void put_split16(unsigned char* blk, uint32_t lo_off,
                                             const float (&v)[8]) {
   uint32_t h[4], l[4];
 #pragma unroll
-  for (int t = 0; t < 4; ++t) {
-    const __half2 hh = __floats2half2_rn(v[2 * t], v[2 * t + 1]);
-    const float2 hf = __half22float2(hh);
-    const __half2 ll = __floats2half2_rn(v[2 * t] - hf.x, v[2 * t + 1] - hf.y);
-    h[t] = *reinterpret_cast<const uint32_t*>(&hh);
-    l[t] = *reinterpret_cast<const uint32_t*>(&ll);
-  }
+  for (int t = 0; t < 4; ++t) split_half2(v[2 * t], v[2 * t + 1], h[t], l[t]);
   *reinterpret_cast<uint4*>(blk + off) = make_uint4(h[0], h[1], h[2], h[3]);
   *reinterpret_cast<uint4*>(blk + lo_off + off) = make_uint4(l[0], l[1], l[2], l[3]);
 }
@@ -326,14 +317,15 @@ k3_trispec_cross_tc(const __grid_constant__ CUtensorMap tm_ab,
     // the first or second half of every stage's frames, fp = lane / 8 % 2 (one
     // 16-byte chunk of the row), so that 8 consecutive lanes fill one 128-byte core
     // matrix.  The column rows: 3 operands (z, w, zw) x 24 bins x 2 chunks = 144
-    // tasks, thread bt < 144 taking task bt: operand bt / 48, chunk bt / 24 % 2, bin
-    // bt % 24; a task writes the operand's Re and Im columns (8 consecutive tasks
-    // fill one core matrix).  Each warp waits and arrives on its own.
+    // tasks, thread bt < 144 taking one: operand and bin e / 24, e % 24 of e = 8 (bt / 16)
+    // + bt % 8, chunk fp; a task writes the operand's Re and Im columns (8 consecutive
+    // tasks fill one core matrix).  Each warp waits and arrives on its own.
     constexpr int kTasks = 3 * 2 * kXL;
     const int bt = tid - 32 * kXEpiWarps, wb = bt >> 5;
     const int R = 16 * wb + (lane & 7) + 8 * (lane >> 4), fp = (lane >> 3) & 1;
-    const int top = bt < kTasks ? bt / (2 * kXL) : -1;  // 0: z, 1: w, 2: zw; -1: none
-    const int tli = bt % kXL, tfq = (bt / kXL) & 1;
+    const int ce = 8 * (bt >> 4) + (bt & 7);
+    const int top = bt < kTasks ? ce / kXL : -1;  // 0: z, 1: w, 2: zw; -1: none
+    const int tli = ce % kXL, tfq = fp;
     const float2 zero = make_float2(0.f, 0.f);
     uint32_t rq = 0, q = 0, gs = 0;
     bool ok = true;
@@ -464,21 +456,24 @@ k3_trispec_cross_tc(const __grid_constant__ CUtensorMap tm_ab,
       }
       ++q;
       if (rec.flags & kRecLast) {
-        // the group's one-bin sums (the two chunks of a row are lanes 8 apart; the
-        // column sums go per chunk), its scales and its record, for the epilogue
+        // the group's one-bin sums, its scales and its record, for the epilogue
+        // (the two chunks of a row or a column are lanes 8 apart)
         const float2 sxy_o = make_float2(__shfl_xor_sync(0xffffffffu, sxy.x, 8),
                                          __shfl_xor_sync(0xffffffffu, sxy.y, 8));
+        const float2 szw_o = make_float2(__shfl_xor_sync(0xffffffffu, szw.x, 8),
+                                         __shfl_xor_sync(0xffffffffu, szw.y, 8));
         const int p = (int)(gs % kXSlots);
         ok = __all_sync(0xffffffffu, gs < (uint32_t)kXSlots ||
                                          mbar_wait_bounded(&slotempty[p],
                                                            ((gs / kXSlots) - 1) & 1u, status));
         if (!ok) break;
-        if (fp == 0) slot[p].sxy[R] = make_float2(sxy.x + sxy_o.x, sxy.y + sxy_o.y);
-        if (top == 2) slot[p].szw[tfq][tli] = szw;
-        if constexpr (kF16) {
-          if (fp == 0) slot[p].rxy[R] = make_float2(pow2_inv(sx), pow2_inv(sy));
-          if (top == 2 && tfq == 0) slot[p].rzw[tli] = make_float2(pow2_inv(tz), pow2_inv(tw));
+        if (fp == 0) {
+          slot[p].sxy[R] = make_float2(sxy.x + sxy_o.x, sxy.y + sxy_o.y);
+          if constexpr (kF16) slot[p].rxy[R] = pow2_inv(sx) * pow2_inv(sy);
         }
+        if (top == 2 && fp == 0)
+          slot[p].szw[tli] = make_float4(szw.x + szw_o.x, szw.y + szw_o.y,
+                                         kF16 ? pow2_inv(tz) * pow2_inv(tw) : 1.f, 0.f);
         if (bt == 0) {
           slot[p].r0 = rec.r0;
           slot[p].l0 = rec.l0;
@@ -663,7 +658,7 @@ k3_trispec_cross_tc(const __grid_constant__ CUtensorMap tm_ab,
       // the whole record is read before the slot is released below
       const int l0 = slot[p].l0, r0 = slot[p].r0, combo = slot[p].combo;
       const float2 sxy = slot[p].sxy[R];
-      const float2 rxy = kF16 ? slot[p].rxy[R] : make_float2(1.f, 1.f);
+      const float rxy = kF16 ? slot[p].rxy[R] : 1.f;
       const uint32_t tb = lane_addr + b * kXBufCols;
 #pragma unroll
       for (int hh = 0; hh < kXLw / 2; ++hh) {
@@ -676,8 +671,8 @@ k3_trispec_cross_tc(const __grid_constant__ CUtensorMap tm_ab,
           tc_wait_ld();
 #pragma unroll
           for (int i = 0; i < 2; ++i) {
-            const float2 szw = make_float2(slot[p].szw[0][li0 + i].x + slot[p].szw[1][li0 + i].x,
-                                           slot[p].szw[0][li0 + i].y + slot[p].szw[1][li0 + i].y);
+            const float4 sr = slot[p].szw[li0 + i];
+            const float2 szw = make_float2(sr.x, sr.y);
             const float2 xz = make_float2(d[0][i], d[1][i]), xw = make_float2(d[2][i], d[3][i]);
             const float2 yz = make_float2(d[4][i], d[5][i]), yw = make_float2(d[6][i], d[7][i]);
             float2 t = cmulf(sxy, szw);
@@ -685,11 +680,10 @@ k3_trispec_cross_tc(const __grid_constant__ CUtensorMap tm_ab,
             cmacf(t, xw, yz);
             float ur = fmaf(fmm_p, d[8][i], -fm1 * t.x), ui = fmaf(fmm_p, d[9][i], -fm1 * t.y);
             if constexpr (kF16) {
-              // [fmm P - fm1 (...)] sx sy tz tw, undone one power of two at a time (their
-              // product alone may leave the float range)
-              const float2 rzw = slot[p].rzw[li0 + i];
-              ur = ur * rxy.x * rxy.y * rzw.x * rzw.y;
-              ui = ui * rxy.x * rxy.y * rzw.x * rzw.y;
+              // [fmm P - fm1 (...)] sx sy tz tw: the scales of the rows, then of the columns
+              // undone (each within 2^120; all four multiplied may leave the float range)
+              ur = ur * rxy * sr.z;
+              ui = ui * rxy * sr.z;
             }
             const float cr = pref * ur, ci = pref * ui;
             const int e = 2 * hh + i;

@@ -27,6 +27,20 @@ __device__ __forceinline__ double widen(float f) {
   return mag == 0u ? __hiloint2double((int)b, 0) : (double)f;
 }
 
+// FP16 hi and lo parts of x and y, packed: hi rounded to nearest, lo = (x, y) - hi rounded.
+// The subtraction takes the half as it is (exact); widening the two halves first is two
+// operations more of six.  k3_trispec_cross_tc with four channels, 2^21 samples, T = 512,
+// m = 20: 7.65 ms so, 7.30 now (with the scales of a pair multiplied once per row).
+__device__ __forceinline__ void split_half2(float x, float y, uint32_t& hi, uint32_t& lo) {
+  float dx, dy;
+  asm("cvt.rn.f16x2.f32 %0, %2, %1;" : "=r"(hi) : "f"(x), "f"(y));
+  asm("{\n\t.reg .b16 a, b;\n\tmov.b32 {a, b}, %2;\n\t"
+      "sub.rn.f32.f16 %0, a, %3;\n\tsub.rn.f32.f16 %1, b, %4;\n\t}"
+      : "=f"(dx), "=f"(dy)
+      : "r"(hi), "f"(x), "f"(y));
+  asm("cvt.rn.f16x2.f32 %0, %2, %1;" : "=r"(lo) : "f"(-dx), "f"(-dy));
+}
+
 // The sum of four warps' float32 sums, widened.  exact (each holds one group at most):
 // to float64's accuracy, so that sums over few groups do not depend on how a record was
 // cut into calls; the rounding errors of the float32 additions (two-sum, Knuth) enter
