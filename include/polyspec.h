@@ -483,7 +483,7 @@ const char* ss_version(void);
  * intermediate (window and twiddle tables, built on the device; centred
  * spectra; float64 sums) kept in one static device array of
  * SS_NOALLOC_SCRATCH_BYTES bytes that every GPU which loads the library holds
- * until the process exits.  The call enqueues kernels and memsets only.
+ * until the process exits.  The call enqueues kernels only.
  *   d_signal   device pointer to n_samples float32 samples.
  *   T, dt, m, window, win_param   as for ss_plan (m >= 2).
  *   d_S2       device output, [M] complex128 as interleaved (re, im) doubles.

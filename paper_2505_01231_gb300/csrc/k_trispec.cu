@@ -15,7 +15,8 @@
 // and its sum of squares over groups are accumulated (Eq. 35-36).
 //
 // This is the plain FP32 CUDA-core form of the fourth-order moment sums: five
-// length-m dot products per grid point and group.  Work split as in K2:
+// length-m dot products per grid point and group, for m > kGram32MaxM (below,
+// k3_trispec_gram takes fewer operations and half the time).  Work split as in K2:
 // persistent CTAs take (group chunk, 64 x 64 tile of the upper triangle k <= l)
 // items from a group-major queue; chunks of FC frames of the coefficients at
 // k0.. and l0.. arrive by 128-byte-swizzled 3-D TMA box loads into kStages

@@ -829,14 +829,41 @@ ss_status alloc_spec(ss_plan_s* p) {
   const long long max_rows = (1ll << 31) - 1;
   const long long group_rows = std::max((long long)p->C * p->m, p->gram32 ? (long long)grows : 0ll);
   if (gb * group_rows > max_rows) gb = (int)(max_rows / group_rows);
+  void* img = nullptr;
+  float *rsc = nullptr, *rmax = nullptr;
+  auto scratch = [&](int n) {
+    cudaError_t e = dev_alloc(p, &p->d_spec, spec_group * n);
+    if (e == cudaSuccess && image) e = dev_alloc(p, &img, img_group * n);
+    if (e == cudaSuccess && scaled) e = dev_alloc(p, &rsc, rsc_group * n);
+    if (e == cudaSuccess && cross16) e = dev_alloc(p, &rmax, rmax_group * n);
+    return e;
+  };
+  cudaError_t e = scratch(gb);
+  // a batch asked for whose unmirrored spectra, without the F32 image, would fit: as many
+  // groups as fit the memory of those
+  const size_t least = per_group - (p->gram32 ? img_group : 0) -
+                       (size_t)p->C * p->m * (p->Ms - p->Mp) * sizeof(float2);
+  const int fewer = (int)std::max<size_t>(1, least * gb / per_group);
+  if (e == cudaErrorMemoryAllocation && fewer < gb) {
+    cudaGetLastError();
+    void* got[4] = {p->d_spec, img, rsc, rmax};
+    const size_t bytes[4] = {spec_group, img_group, rsc_group, rmax_group};
+    for (int i = 0; i < 4; ++i) release(got[i], bytes[i] * gb);
+    p->d_spec = nullptr;
+    img = nullptr;
+    rsc = rmax = nullptr;
+    gb = fewer;
+    e = scratch(gb);
+  }
   p->Gb_max = gb;
-  SS_TRY(p, dev_alloc(p, &p->d_spec, spec_group * gb));
+  p->oi = OperandImage();
+  p->oi.img = img;
+  p->oi.rsc = rsc;
+  p->oi.rmax = rmax;
+  SS_TRY(p, e);
   // the bins below -(M - 1) of mirrored rows are read (as zeros) but never written
   if (p->mirror) SS_TRY(p, cudaMemsetAsync(p->d_spec, 0, spec_group * gb, p->stream));
-  p->oi = OperandImage();
   if (image) {
-    SS_TRY(p, dev_alloc(p, &p->oi.img, img_group * gb));
-    if (scaled) SS_TRY(p, dev_alloc(p, &p->oi.rsc, rsc_group * gb));
     p->oi.rows = p->gram32 ? grows : 0;
     p->oi.fmt = p->gram32                        ? kImageGramF32
                 : p->precision == SS_PREC_TF32X3 ? kImageGramTF32
@@ -852,10 +879,7 @@ ss_status alloc_spec(ss_plan_s* p) {
     // no tile reads the rows of bins from M - 1 on when k3_column takes that column
     p->oi.img_bins = p->col4 ? p->M - 1 : p->Mp;
   }
-  if (cross16) {
-    SS_TRY(p, dev_alloc(p, &p->oi.rmax, rmax_group * gb));
-    p->oi.chan_rmax = (long long)gb * p->Mp;
-  }
+  if (cross16) p->oi.chan_rmax = (long long)gb * p->Mp;
   return encode_maps(p);
 }
 
@@ -1379,14 +1403,19 @@ ss_status ss_set_sequential(ss_plan_t p, int block_groups, double* out, long lon
   p->seq_cap = block_groups > 0 ? max_blocks : 0;
   p->seq_blocks = 0;
   const size_t n = p->n_acc2 + p->n_acc3 + p->n_acc4;
+  if (block_groups > 0 && !p->d_prev && n) SS_TRY(p, dev_alloc(p, &p->d_prev, n * sizeof(double)));
   if (block_groups > 0 && !p->d_blocks && n && p->C == 1 && p->n_s2cross == 0) {
-    // sums of a set of blocks that one batch computes: at most 256, 128 MB
+    // sums of a set of blocks that one batch computes: at most 256, 128 MB (without
+    // them a batch ends at every block's end)
     const size_t fit = (128ull << 20) / (n * sizeof(double));
     p->seq_set = (int)std::min<size_t>(256, fit);
     p->seq_stride = n;
-    if (p->seq_set >= 2) SS_TRY(p, dev_alloc(p, &p->d_blocks, p->seq_set * n * sizeof(double)));
+    if (p->seq_set >= 2 &&
+        dev_alloc(p, &p->d_blocks, p->seq_set * n * sizeof(double)) != cudaSuccess) {
+      cudaGetLastError();
+      p->d_blocks = nullptr;
+    }
   }
-  if (block_groups > 0 && !p->d_prev && n) SS_TRY(p, dev_alloc(p, &p->d_prev, n * sizeof(double)));
   if (p->d_prev) SS_TRY(p, cudaMemsetAsync(p->d_prev, 0, n * sizeof(double), p->stream));
   return SS_OK;
 }

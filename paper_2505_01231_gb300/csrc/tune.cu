@@ -4,9 +4,10 @@
 // A plan's results do not depend on these choices; only its speed does.  Two
 // stages have alternative forms:
 //   K1 (frame/window/FFT/centre): groups resident in shared memory within 74 KB
-//       (three CTAs per SM) or 96 KB (two), or one frame at a time;
-//   K2 (bispectrum): 4 x 4 micro-tiles in CTAs of 256 threads (4 stages), or
-//       8 x 4 micro-tiles in CTAs of 128 threads with 2 or 3 stages.
+//       (three CTAs per SM) or 96 KB (two), a warp per frame, or one frame at a time;
+//   K2 (bispectrum): 4 x 4 micro-tiles in CTAs of 256 threads (4 stages), 8 x 4
+//       micro-tiles in CTAs of 128 threads with 2 or 3 stages, or 8 x 4 micro-tiles in
+//       warps with rings of their own (84w, what a new plan has).
 // ss_autotune times every form on the plan's own shapes (frame length, group
 // size, channels, precision) on this GPU, on a synthetic record of Gaussian
 // noise generated on the device, and keeps the fastest of each stage.  The
