@@ -22,10 +22,16 @@
 // Szw depend on one bin each and are summed, scaled alike, by the threads that build
 // the operands.
 //
-// Building the operands is the limit: an M = 128, N <= 128 product reads its
-// operands from shared memory at about 120 bytes per clock, so the tile is as
-// wide as two TMEM buffers allow, and the builders' staging reads and operand
-// stores are kept to one pass each, free of bank conflicts.
+// Instruction issue is the limit (61 % of the slots, most of them the builders', whose
+// warps otherwise wait on one another's stages; tensor pipe 17 % busy), and shared memory
+// next: an M = 128, N <= 128 product reads its operands at about 120 bytes per clock, so
+// the tile is as wide as two TMEM buffers allow, and the builders' staging reads and
+// operand stores are kept to one pass each, free of bank conflicts.  Four channels, 2^21
+// samples, T = 512, m = 20, 55 combinations in FP16X3: 11.5 ms with all rows of every
+// combination, 8.30 with the rows k >= 0 of the symmetric ones, 7.65 with the sums of xy
+// and zw taken of the scaled operands and no check of full stages, 7.29 with the splits in
+// four operations a pair.  Five more builder warps for the columns made it 8.6 (80
+// registers a thread), 8.85 with the registers split between the roles.
 //
 // Grid: one persistent CTA per SM (all 512 TMEM columns).  Items (group chunk,
 // combination, tile) come from a group-major queue.  Warp roles, coupled only by
